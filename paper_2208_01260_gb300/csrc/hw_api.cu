@@ -220,7 +220,7 @@ int hw_create(const hw_grid* grid, const hw_params* params, void* cuda_stream, h
     const double dy = (grid->y1 - grid->y0) / ny;
     d.nx = nx; d.ny = ny; d.bc_x = grid->bc_x; d.bc_y = grid->bc_y;
     set_spacing2d(d, dx, dy);
-    d.g = params->g; d.eps_w = params->eps_w; d.eps_lim = params->eps_lim;
+    hw::set_physics2d(d, params->g, params->eps_w, params->eps_lim);
     for (int q = 0; q < 3; ++q) A(&d.stat[q], s->n);
     for (int q = 0; q < 2; ++q) A(&d.bxy[q], s->n);
     for (int q = 0; q < 12; ++q) { A(&d.X[q], (size_t)(nx + 1) * ny); A(&d.Y[q], (size_t)nx * (ny + 1)); }
@@ -234,7 +234,7 @@ int hw_create(const hw_grid* grid, const hw_params* params, void* cuda_stream, h
       for (int q = 0; q < 9; ++q) { F(&s->FA[q], s->n); F(&s->FB[q], s->n); F(&s->fbase[q], s->n); }
       f.nx = d.nx; f.ny = d.ny; f.bc_x = d.bc_x; f.bc_y = d.bc_y;
       f.dx = (float)d.dx; f.dy = (float)d.dy; f.inv_dx = (float)d.inv_dx; f.inv_dy = (float)d.inv_dy;
-      f.g = (float)d.g; f.eps_w = (float)d.eps_w; f.eps_lim = (float)d.eps_lim;
+      hw::set_physics2d(f, d.g, d.eps_w, d.eps_lim);
       f.c_bx = (float)d.c_bx; f.c_by = (float)d.c_by; f.c_gx = (float)d.c_gx; f.c_gy = (float)d.c_gy;
       f.c_mx = (float)d.c_mx; f.c_my = (float)d.c_my;
       F(&s->fsc, 4);

@@ -6,8 +6,7 @@
 // graph. The sweeps use the single-grid tiles over flattened extended lines (hw_stencil2d.cuh), so no
 // grid size leaves a ragged tile; the y-tile width is per instance, chosen by the autotuner. The
 // arithmetic is the single-grid kernels', so each instance's result equals a single-grid solver's to
-// rounding (the compiler may contract multiply-adds differently in the two kernels), with the same
-// share of products on the integer pipes (each bit-identical to DMUL, hw_fp64_int.h). The kernels read
+// rounding (the compiler may contract multiply-adds differently in the two kernels). The kernels read
 // the pooled planes through the parameters' base pointers plus the instance's offsets, so that no
 // per-instance pointer takes a register. No block ever waits on another block. hw_batch_set_persistent
 // switches a batch to one cooperative launch per step instead (hw_bstep.cu).
@@ -20,7 +19,7 @@
 
 namespace hw {
 
-constexpr int BN_T = 256;  // nodes per node-kernel item
+constexpr int BN_T = 128;  // nodes per node-kernel item
 
 // ---- alpha per instance in two passes, as the single-grid reduction (a float estimate of every node,
 // the double value only near the float maximum): items (inst, first node, count) ----
@@ -105,8 +104,8 @@ __global__ void k_btime(BatchDev B, int n) {
 
 // ---- x-sweep: items (inst, first extended node of the tile) over the flattened extended rows ----
 template <bool LINEAR, bool CHAR>
-__global__ void __launch_bounds__(TILE_T, 2) k_bsweep_x(BatchDev B, const int4* __restrict__ items, int nitems) {
-  __shared__ double sm[NREC * TILE_T];
+__global__ void __launch_bounds__(TILE_T, 5) k_bsweep_x(BatchDev B, const int4* __restrict__ items, int nitems) {
+  __shared__ double sm[NRECX * TILE_T];
   {
     const int4 it = items[blockIdx.x];
     const BInst& I = B.inst[it.x];
@@ -118,8 +117,8 @@ __global__ void __launch_bounds__(TILE_T, 2) k_bsweep_x(BatchDev B, const int4* 
 
 // ---- y-sweep: items (inst, first extended row of the tile) over the flattened column groups ----
 template <bool LINEAR, bool CHAR>
-__global__ void __launch_bounds__(TILE_T, 2) k_bsweep_y(BatchDev B, const int4* __restrict__ items, int nitems) {
-  __shared__ double sm[NREC * TILE_T];
+__global__ void __launch_bounds__(TILE_T, 4) k_bsweep_y(BatchDev B, const int4* __restrict__ items, int nitems) {
+  __shared__ double sm[NRECX * TILE_T];
   {
     const int4 it = items[blockIdx.x];
     const BInst& I = B.inst[it.x];
@@ -131,11 +130,10 @@ __global__ void __launch_bounds__(TILE_T, 2) k_bsweep_y(BatchDev B, const int4* 
 }
 
 // ---- node update: items (inst, first node) of BN_T consecutive nodes of one grid ----
-// Two blocks per SM: the instance's grid constants come from global memory and take registers that the
-// single-grid kernel keeps in its parameters (measured: 3 blocks per SM spill 0.75 KB per thread and run
-// no faster).
+// The instance's grid constants come from global memory and take registers that the single-grid kernel keeps
+// in its parameters: 128 registers per thread (16 warps per SM).
 template <bool LINEAR, bool CHAR>
-__global__ void __launch_bounds__(BN_T, 2) k_bnode(BatchDev B, const int4* __restrict__ items, int nitems) {
+__global__ void __launch_bounds__(BN_T, 4) k_bnode(BatchDev B, const int4* __restrict__ items, int nitems) {
   {
     const int4 it = items[blockIdx.x];
     const BInst& I = B.inst[it.x];
@@ -214,7 +212,7 @@ hw::Dev2D dev_of(hw_batch* b, int i, double** S) {
   hw::Dev2D d{};
   d.nx = I.nx; d.ny = I.ny; d.bc_x = I.bc_x; d.bc_y = I.bc_y;
   d.dx = I.dx; d.dy = I.dy; d.inv_dx = I.inv_dx; d.inv_dy = I.inv_dy;
-  d.g = b->params.g; d.eps_w = b->params.eps_w; d.eps_lim = b->params.eps_lim;
+  hw::set_physics2d(d, b->params.g, b->params.eps_w, b->params.eps_lim);
   d.c_bx = I.c_bx; d.c_by = I.c_by; d.c_gx = I.c_gx; d.c_gy = I.c_gy; d.c_mx = I.c_mx; d.c_my = I.c_my;
   for (int q = 0; q < 9; ++q) d.S[q] = S[q] + I.off_n;
   for (int q = 0; q < 3; ++q) d.stat[q] = b->B.stat[q] + I.off_n;
@@ -408,7 +406,8 @@ int hw_batch_create(int n, const hw_grid* grids, const hw_params* params, void* 
   b->B.t = misc + 7 * n;
   b->B.nsteps = (unsigned long long*)(misc + 8 * n);
   b->B.status = (int*)(misc + 9 * n);
-  b->B.g = params->g; b->B.eps_w = params->eps_w; b->B.eps_lim = params->eps_lim; b->B.cfl = params->cfl;
+  hw::set_physics2d(b->B, params->g, params->eps_w, params->eps_lim);
+  b->B.cfl = params->cfl;
   b->B.limiter = params->limiter;
   b->B.inst = b->d_inst;
   cudaError_t e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);

@@ -14,7 +14,7 @@ struct BInst {
 };
 
 struct BatchDev {
-  double g, eps_w, eps_lim, cfl;
+  double g, eps_w, eps_lim, half_g, fx_eps13, fx_eps2, fx_eps13l, fx_eps2l, cfl;
   int limiter, k;
   const BInst* inst;
   double* S[9];
@@ -42,6 +42,8 @@ __device__ __forceinline__ void make_dev(const BatchDev& B, const BInst& I, Dev2
   d.nx = I.nx; d.ny = I.ny; d.bc_x = I.bc_x; d.bc_y = I.bc_y;
   d.dx = I.dx; d.dy = I.dy; d.inv_dx = I.inv_dx; d.inv_dy = I.inv_dy;
   d.g = B.g; d.eps_w = B.eps_w; d.eps_lim = B.eps_lim;
+  d.half_g = B.half_g; d.fx_eps13 = B.fx_eps13; d.fx_eps2 = B.fx_eps2;
+  d.fx_eps13l = B.fx_eps13l; d.fx_eps2l = B.fx_eps2l;
   d.c_bx = I.c_bx; d.c_by = I.c_by; d.c_gx = I.c_gx; d.c_gy = I.c_gy; d.c_mx = I.c_mx; d.c_my = I.c_my;
 #pragma unroll
   for (int q = 0; q < 9; ++q) d.S[q] = B.S[q];

@@ -84,7 +84,7 @@ __device__ __forceinline__ void make_dev_in(const BatchDev& B, const BInst& I, b
 // Shared memory of a block: two sweep tiles (consecutive tiles alternate, so one barrier per tile
 // suffices) and the block-uniform values the phases pass around.
 struct BStepSmem {
-  double tile[2][NREC * TILE_T];
+  double tile[2][NRECX * TILE_T];
   int item[2];     // the next sweep tile, written by thread 0 during the current one
   int node_item;   // the block's current node item
   int flag;        // grid barrier: 1 = continue
@@ -246,7 +246,7 @@ __device__ __forceinline__ bool bstep_stage(const BatchDev& B, const StepItems& 
 // (One copy of the stage code selects the input pointers: two inlined copies, one per direction, spill
 // several times more.) Dynamic shared memory: one BStepSmem.
 template <bool LINEAR, bool CHAR>
-__global__ void __launch_bounds__(TILE_T, 2) k_bstep(const BatchDev B, const StepItems P, int cur) {
+__global__ void __launch_bounds__(TILE_T, 4) k_bstep(const BatchDev B, const StepItems P, int cur) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BStepSmem& sh = *reinterpret_cast<BStepSmem*>(smem_raw);
   if ((int)blockIdx.x == P.drop_block) return;  // test of the bounded wait: this block never arrives

@@ -19,6 +19,9 @@ struct Dev2DT {
   R dx, dy, inv_dx, inv_dy, g, eps_w, eps_lim;
   // assembly constants: 1/(2dx), 1/(2dy), 1/(24dx), 1/(24dy), 1/(12dx), 1/(12dy)
   R c_bx, c_by, c_gx, c_gy, c_mx, c_my;
+  R half_g;            // g / 2
+  R fx_eps13, fx_eps2;    // the weights' epsilon of the fixed-point sweeps: (160/781) g eps_w, (80/781) eps_w
+  R fx_eps13l, fx_eps2l;  // and of the limiter: (12/13) g eps_lim, (3/13) eps_lim
   R* S[9];      // current state (eta, m, w, dx V, dy Q)
   R* stat[3];   // b, dx b_x, dy b_y
   R* bxy[2];    // b_x, b_y (physical, for conversions and static terms)
@@ -30,6 +33,20 @@ struct Dev2DT {
   R* sq[2];     // ... of the Q equations
 };
 using Dev2D = Dev2DT<double>;
+
+// g and the weights' epsilons with the constants derived from them.
+template <class D>
+inline void set_physics2d(D& d, double g, double eps_w, double eps_lim) {
+  using R = decltype(d.g);
+  d.g = (R)g;
+  d.eps_w = (R)eps_w;
+  d.eps_lim = (R)eps_lim;
+  d.half_g = (R)(0.5 * g);
+  d.fx_eps13 = (R)((160.0 / 781.0) * eps_w * g);
+  d.fx_eps2 = (R)((80.0 / 781.0) * eps_w);
+  d.fx_eps13l = (R)((12.0 / 13.0) * eps_lim * g);
+  d.fx_eps2l = (R)((3.0 / 13.0) * eps_lim);
+}
 
 template <class R>
 struct StageArgsT {

@@ -19,29 +19,34 @@ namespace hw {
 // ---------------------------------------------------------------------------------------------
 constexpr int YS_C = 2;  // columns per y-tile group of the double y-sweep (measured: 2 beats 1 and 4)
 
-// The double kernels form their products (and the node kernel also its reciprocals) on the integer
-// pipes (hw_fp64_int.h: each product bit-identical to DMUL): the FP64 pipe is their bound, the integer
-// pipes idle. The node records stay on the FP64 pipe (moving them measured slower).
+// The double kernels run the nonlinear reconstruction and the limiter in fixed point (hw_fixed.h): on the FP64
+// pipe alone these kernels took 2.80 (x), 2.85 (y) and 2.03 ms (node) per stage at 2048^2, its operations at the
+// pipe's rate; now 0.77, 0.83 and 1.04 ms. What bounds them is the sum of what is left on the FP64 pipe (71
+// operations per x-interface, 60% busy) and integer issue (4060 instructions per warp, 54% of the slots).
 template <class R>
-constexpr bool kIntMul = std::is_same<R, double>::value;
-// Blocks per SM the sweeps and the node kernel are compiled for: the double kernels carry the
-// integer-pipe products in registers (168 per thread in the sweeps); the float kernels are bound by
-// memory and issue and want occupancy.
+constexpr bool kFixed = std::is_same<R, double>::value;
 template <class R>
-constexpr int kXsBlocks = std::is_same<R, double>::value ? 2 : 5;
+constexpr int kTileRec = std::is_same<R, double>::value ? NRECX : NREC;
+// Threads per x-tile and blocks per SM the kernels are compiled for. The register file holds 3, 4, 5 or 6 warps per
+// SM partition at 168, 128, 96 or 80 registers: measured at 2048^2, x-sweep 0.79 / 0.77 ms at 4 / 5 (tiles of 192
+// threads 0.79, of 96 0.84), y-sweep 0.83 / 0.85, node kernel 1.16 / 1.15 / 1.04 ms at 4 / 5 / 6.
+template <class R>
+constexpr int kXT = std::is_same<R, double>::value ? TILE_T : 192;
+constexpr int kXsBlocks = 5, kYsBlocks = 4;
+constexpr int kNodeT = 256;
 template <class R>
 constexpr int kNodeBlocks = std::is_same<R, double>::value ? 3 : 5;
 
 template <bool LINEAR, bool CHAR, class R>
-__global__ void __launch_bounds__(TILE_T, kXsBlocks<R>) k_sweep_x(Dev2DT<R> d, const R* __restrict__ alpha) {
-  __shared__ R sm[NREC * TILE_T];
-  sweep_x_tile<LINEAR, CHAR, kIntMul<R>>(d, alpha[0], blockIdx.x * (TILE_T - 3), sm);
+__global__ void __launch_bounds__(kXT<R>, kXsBlocks) k_sweep_x(Dev2DT<R> d, const R* __restrict__ alpha) {
+  __shared__ R sm[kTileRec<R> * kXT<R>];
+  sweep_x_tile<LINEAR, CHAR, kFixed<R>, false, kXT<R>>(d, alpha[0], blockIdx.x * (kXT<R> - 3), sm);
 }
 
-template <bool LINEAR, bool CHAR, class R>
-__global__ void __launch_bounds__(TILE_T, kXsBlocks<R>) k_sweep_y(Dev2DT<R> d, const R* __restrict__ alpha) {
-  __shared__ R sm[NREC * TILE_T];
-  sweep_y_tile<LINEAR, CHAR, kIntMul<R>>(d, alpha[1], blockIdx.x * (TILE_T / YS_C - 3), YS_C, sm);
+template <bool LINEAR, bool CHAR>
+__global__ void __launch_bounds__(TILE_T, kYsBlocks) k_sweep_y(Dev2D d, const double* __restrict__ alpha) {
+  __shared__ double sm[NRECX * TILE_T];
+  sweep_y_tile<LINEAR, CHAR, true>(d, alpha[1], blockIdx.x * (TILE_T / YS_C - 3), YS_C, sm);
 }
 
 // Single-precision y-sweep: bound by memory rather than arithmetic, it keeps the column march, whose
@@ -77,7 +82,7 @@ __global__ void __launch_bounds__(YS_W, 32) k_sweep_y_col(Dev2DT<float> d, const
 #pragma unroll
       for (int q = 0; q < 6; ++q) qb[q] = __ldg(d.qby[q] + o);
       float out[12];
-      interface_values<1, LINEAR, CHAR, false>(s0, s1, s2, s3, YS_W, qb, d.g, d.eps_w, out);
+      interface_values<1, LINEAR, CHAR>(s0, s1, s2, s3, YS_W, qb, d.g, d.eps_w, out);
 #pragma unroll
       for (int q = 0; q < 12; ++q) d.Y[q][o] = out[q];
     }
@@ -85,11 +90,11 @@ __global__ void __launch_bounds__(YS_W, 32) k_sweep_y_col(Dev2DT<float> d, const
 }
 
 template <int MODE, bool LINEAR, bool CHAR, class R>
-__global__ void __launch_bounds__(256, kNodeBlocks<R>) k_node2d(Dev2DT<R> d, StageArgsT<R> sa) {
+__global__ void __launch_bounds__(kNodeT, kNodeBlocks<R>) k_node2d(Dev2DT<R> d, StageArgsT<R> sa) {
   const int i = blockIdx.x * 32 + threadIdx.x;
-  const int j = blockIdx.y * 8 + threadIdx.y;
+  const int j = blockIdx.y * (kNodeT / 32) + threadIdx.y;
   if (i >= d.nx || j >= d.ny) return;
-  node_update<MODE, LINEAR, CHAR, kIntMul<R>>(d, sa, i, j);
+  node_update<MODE, LINEAR, CHAR, kFixed<R>>(d, sa, i, j);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -421,7 +426,8 @@ __global__ void k_static2d(Dev2D d) {
 template <bool L, bool C, class R>
 static void launch_sx(const Dev2DT<R>& d, const R* alpha, cudaStream_t st) {
   const unsigned long long total = (unsigned long long)d.ny * (d.nx + 4);
-  k_sweep_x<L, C, R><<<(unsigned)((total + TILE_T - 4) / (TILE_T - 3)), TILE_T, 0, st>>>(d, alpha);
+  constexpr int T = kXT<R>;
+  k_sweep_x<L, C, R><<<(unsigned)((total + T - 4) / (T - 3)), T, 0, st>>>(d, alpha);
 }
 
 // Segment length of the float column march: one balanced wave of resident blocks when the grid allows
@@ -453,14 +459,15 @@ static void launch_sy(const Dev2DT<R>& d, const R* alpha, cudaStream_t st) {
   } else {
     constexpr int IFS = TILE_T / YS_C - 3;
     const unsigned long long total = (unsigned long long)((d.nx + YS_C - 1) / YS_C) * (d.ny + 4);
-    k_sweep_y<L, C, R><<<(unsigned)((total + IFS - 1) / IFS), TILE_T, 0, st>>>(d, alpha);
+    k_sweep_y<L, C><<<(unsigned)((total + IFS - 1) / IFS), TILE_T, 0, st>>>(d, alpha);
   }
 }
 
 template <int MODE, bool L, bool C, class R>
 static void launch_node(const Dev2DT<R>& d, const StageArgsT<R>& sa, cudaStream_t st) {
-  dim3 g((d.nx + 31) / 32, (d.ny + 7) / 8);
-  k_node2d<MODE, L, C, R><<<g, dim3(32, 8), 0, st>>>(d, sa);
+  constexpr int rows = kNodeT / 32;
+  dim3 g((d.nx + 31) / 32, (d.ny + rows - 1) / rows);
+  k_node2d<MODE, L, C, R><<<g, dim3(32, rows), 0, st>>>(d, sa);
 }
 
 int set_kernel_attributes2d() { return 0; }

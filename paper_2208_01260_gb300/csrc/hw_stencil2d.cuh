@@ -4,6 +4,7 @@
 // and the node update (eq. swe-form-2d-dis, limiter, eq. RK). See hw_device.cuh for the conventions.
 #pragma once
 #include "hw_device.cuh"
+#include "hw_fixed.h"
 #include "hw_internal.h"
 
 namespace hw {
@@ -27,6 +28,14 @@ __device__ __forceinline__ T ldp(const T* p) {
   else return __ldg(p);
 }
 
+// x with its sign flipped where mask is 0x80000000 (0: x itself), on the integer pipes.
+__device__ __forceinline__ double flip_sign(double x, uint32_t mask) {
+  uint32_t lo, hi;
+  f64_words(x, lo, hi);
+  return f64_from_words(lo, hi ^ mask);
+}
+__device__ __forceinline__ float flip_sign(float x, uint32_t mask) { return __uint_as_float(__float_as_uint(x) ^ mask); }
+
 // base: offset of the grid's first node in the node planes (0 unless the planes pool several grids).
 template <bool COH = false, class R>
 __device__ __forceinline__ void load_node(const Dev2DT<R>& d, int i, int j, Node12T<R>& n, size_t base = 0) {
@@ -34,81 +43,110 @@ __device__ __forceinline__ void load_node(const Dev2DT<R>& d, int i, int j, Node
   const int ii = map_index(i, d.nx, d.bc_x, fx);
   const int jj = map_index(j, d.ny, d.bc_y, fy);
   const size_t o = base + (size_t)jj * d.nx + ii;
+  const uint32_t mx = fx ? 0x80000000u : 0u, my = fy ? 0x80000000u : 0u;
 #pragma unroll
-  for (int q = 0; q < 9; ++q) {
-    R x = ldp<COH>(d.S[q] + o);
-    if (fx) x *= R(par_x2d(q));
-    if (fy) x *= R(par_y2d(q));
-    n.v[q] = x;
-  }
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    R x = __ldg(d.stat[q] + o);
-    if (fx) x *= R(par_x2d(9 + q));
-    if (fy) x *= R(par_y2d(9 + q));
-    n.v[9 + q] = x;
-  }
+  for (int q = 0; q < 12; ++q)
+    n.v[q] = flip_sign(q < 9 ? ldp<COH>(d.S[q] + o) : __ldg(d.stat[q - 9] + o),
+                       (par_x2d(q) < 0 ? mx : 0u) ^ (par_y2d(q) < 0 ? my : 0u));
 }
 
 // Per-node record a sweep keeps for its stencil (18 doubles).
 enum { R_FP = 0, R_FM = 3, R_GP = 6, R_GM = 9, R_MIX = 12, R_H = 15, R_M = 16, R_W = 17, NREC = 18 };
 
-// Pointwise fluxes of eq. (swe-form-2d-e) and their chain-rule derivatives of eq. (swe-form-2d-h),
-// split with the global alpha (Sec. R(2.1) Step 1, without the factor 1/2). DIR = 0: x-sweep record
-// (F1, d_x F1 for the split, d_y F1 for the mixed term); DIR = 1: y-sweep record (F2, d_y F2, d_x F2).
-template <int DIR, class R, class M>
-__device__ __forceinline__ void node_record_m(const Node12T<R>& n, R g, R alpha, R rec[NREC], M& mul) {
+// Pointwise fluxes of eq. (swe-form-2d-e) and their chain-rule derivatives of eq. (swe-form-2d-h). DIR = 0:
+// x-sweep (F1, d_x F1 along the sweep, d_y F1 for the mixed term); DIR = 1: y-sweep (F2, d_y F2, d_x F2).
+template <int DIR, class R>
+__device__ __forceinline__ void node_fluxes(const Node12T<R>& n, R g, R F[3], R Gs[3], R Gm[3], R& h) {
   const R eta = n.v[0], m = n.v[1], w = n.v[2], b = n.v[9];
-  const R h = eta - b;
+  h = eta - b;
   const R rh = fast_rcp(h);
-  const R u = mul(m, rh), v = mul(w, rh);
-  const R gh = mul(g, h), ge = mul(g, eta);
-  const R pres = mul(ge, fma(R(0.5), eta, -b));  // g/2 (eta^2 - 2 eta b)
-  const R uv = mul(u, v);
+  const R u = m * rh, v = w * rh;
+  const R gh = g * h, ge = g * eta;
+  const R pres = ge * fma(R(0.5), eta, -b);  // g/2 (eta^2 - 2 eta b)
+  const R uv = u * v;
   // derivative data along the sweep (split) and across it (mixed)
   const int qs = DIR == 0 ? 3 : 6, qm = DIR == 0 ? 6 : 3;
   const R Hs = n.v[qs], Ms = n.v[qs + 1], Ws = n.v[qs + 2], Bs = n.v[DIR == 0 ? 10 : 11];
   const R Hm = n.v[qm], Mm = n.v[qm + 1], Wm = n.v[qm + 2], Bm = n.v[DIR == 0 ? 11 : 10];
-  R F[3], Gs[3], Gm[3];
-  const R mv = mul(m, v);
+  const R mv = m * v;
   if (DIR == 0) {
-    const R uu = mul(u, u), a1 = gh - uu, a2 = uu - ge, u2 = u + u;
+    const R uu = u * u, a1 = gh - uu, a2 = uu - ge, u2 = u + u;
     F[0] = m; F[1] = fma(m, u, pres); F[2] = mv;
     Gs[0] = Ms;
-    Gs[1] = fma(u2, Ms, fma(a1, Hs, mul(a2, Bs)));
-    Gs[2] = fma(uv, Bs - Hs, fma(v, Ms, mul(u, Ws)));
+    Gs[1] = fma(u2, Ms, fma(a1, Hs, a2 * Bs));
+    Gs[2] = fma(uv, Bs - Hs, fma(v, Ms, u * Ws));
     Gm[0] = Mm;
-    Gm[1] = fma(u2, Mm, fma(a1, Hm, mul(a2, Bm)));
-    Gm[2] = fma(uv, Bm - Hm, fma(v, Mm, mul(u, Wm)));
+    Gm[1] = fma(u2, Mm, fma(a1, Hm, a2 * Bm));
+    Gm[2] = fma(uv, Bm - Hm, fma(v, Mm, u * Wm));
   } else {
-    const R vv = mul(v, v), a1 = gh - vv, a2 = vv - ge, v2 = v + v;
+    const R vv = v * v, a1 = gh - vv, a2 = vv - ge, v2 = v + v;
     F[0] = w; F[1] = mv; F[2] = fma(w, v, pres);
     Gs[0] = Ws;
-    Gs[1] = fma(uv, Bs - Hs, fma(v, Ms, mul(u, Ws)));
-    Gs[2] = fma(v2, Ws, fma(a1, Hs, mul(a2, Bs)));
+    Gs[1] = fma(uv, Bs - Hs, fma(v, Ms, u * Ws));
+    Gs[2] = fma(v2, Ws, fma(a1, Hs, a2 * Bs));
     Gm[0] = Wm;
-    Gm[1] = fma(uv, Bm - Hm, fma(v, Mm, mul(u, Wm)));
-    Gm[2] = fma(v2, Wm, fma(a1, Hm, mul(a2, Bm)));
+    Gm[1] = fma(uv, Bm - Hm, fma(v, Mm, u * Wm));
+    Gm[2] = fma(v2, Wm, fma(a1, Hm, a2 * Bm));
   }
-  const R U[3] = {eta, m, w}, D[3] = {Hs, Ms, Ws};
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    rec[R_FP + c] = fma(alpha, U[c], F[c]);
-    rec[R_FM + c] = fma(-alpha, U[c], F[c]);
-    rec[R_GP + c] = fma(alpha, D[c], Gs[c]);
-    rec[R_GM + c] = fma(-alpha, D[c], Gs[c]);
-    rec[R_MIX + c] = Gm[c];
-  }
-  rec[R_H] = h;
-  rec[R_M] = m;
-  rec[R_W] = w;
 }
 
-// The record on the FP64 pipe (moving its products to the integer pipes measured slower).
+// The node's record: fluxes split with the global alpha (Sec. R(2.1) Step 1, without the factor 1/2).
 template <int DIR, class R>
 __device__ __forceinline__ void node_record(const Node12T<R>& n, R g, R alpha, R rec[NREC]) {
-  MulFP64 mf;
-  node_record_m<DIR>(n, g, alpha, rec, mf);
+  R F[3], Gs[3], Gm[3];
+  node_fluxes<DIR>(n, g, F, Gs, Gm, rec[R_H]);
+  const int qs = DIR == 0 ? 3 : 6;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    rec[R_FP + c] = fma(alpha, n.v[c], F[c]);
+    rec[R_FM + c] = fma(-alpha, n.v[c], F[c]);
+    rec[R_GP + c] = fma(alpha, n.v[qs + c], Gs[c]);
+    rec[R_GM + c] = fma(-alpha, n.v[qs + c], Gs[c]);
+    rec[R_MIX + c] = Gm[c];
+  }
+  rec[R_M] = n.v[1];
+  rec[R_W] = n.v[2];
+}
+
+// The record with its split fluxes and derivative fluxes (entries R_FP .. R_GM + 2) in fixed point for the
+// nonlinear reconstruction (hw_fixed.h): per component, the four entries as 64-bit integers (below 2^60) of one
+// unit, set by the exponents of F, G and alpha times U, D; the split itself is formed in fixed point (six products
+// for the twelve fmas of node_record). R_GM holds -G-, the derivative the mirrored side takes. R_X holds the three
+// units' biased exponents and, above them, whether an operand does not fit (infinite, NaN or subnormal data, or
+// near the ends of the range).
+enum { R_X = NREC, NRECX = NREC + 1 };
+constexpr int kFxExpMin = 256, kFxExpMax = 1900;  // exponents whose products and squares stay far from the ends
+
+template <int DIR>
+__device__ __forceinline__ void node_record_fixed(const Node12& n, double g, double alpha, double rec[NRECX]) {
+  double F[3], Gs[3], Gm[3];
+  node_fluxes<DIR>(n, g, F, Gs, Gm, rec[R_H]);
+  const int qs = DIR == 0 ? 3 : 6;
+  int ua;
+  const FxS al = fx_split(fx_mantissa(alpha, ua));
+  const int ea = ua + 1084;  // alpha's biased exponent
+  bool bad = (unsigned)(ea - 600) > 600u;
+  int em[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double U = n.v[c], D = n.v[qs + c];
+    const uint32_t wf = max(fx_absw(F[c]), fx_absw(Gs[c])), wu = max(fx_absw(U), fx_absw(D));
+    em[c] = max((int)(wf >> 20) + 1, (int)(wu >> 20) + ea - 1020);
+    const bool any = (fx_any(F[c]) | fx_any(Gs[c]) | fx_any(U) | fx_any(D)) != 0u;
+    bad |= (max(wf, wu) >= (uint32_t)kFxExpMax << 20) | (em[c] > kFxExpMax) | ((em[c] < kFxExpMin) & any);
+    em[c] = max(em[c], kFxExpMin);
+    const int eu = em[c] - ea + 1020;  // alpha times a multiple of 2^(eu - 1082) is one of 2^(em - 1082)
+    const int64_t f = fx_from_double(F[c], em[c]), q = fx_from_double(Gs[c], em[c]);
+    const int64_t pu = fx_mulhi(fx_split(fx_from_double(U, eu)), al, 0), pd = fx_mulhi(fx_split(fx_from_double(D, eu)), al, 0);
+    rec[R_FP + c] = __longlong_as_double(f + pu);
+    rec[R_FM + c] = __longlong_as_double(f - pu);
+    rec[R_GP + c] = __longlong_as_double(q + pd);
+    rec[R_GM + c] = __longlong_as_double(pd - q);
+    rec[R_MIX + c] = Gm[c];
+  }
+  rec[R_M] = n.v[1];
+  rec[R_W] = n.v[2];
+  rec[R_X] = f64_from_words((uint32_t)(em[0] | (em[1] << 16)), (uint32_t)em[2] | (bad ? 0x10000u : 0u));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -117,29 +155,28 @@ __device__ __forceinline__ void node_record(const Node12T<R>& n, R g, R alpha, R
 // where dS is the spacing along the sweep and dT the spacing across it.
 // qb[6] = source candidates q_1..q_3 of (b, dS b_s) for the '+' side then the mirrored '-' side.
 // ---------------------------------------------------------------------------------------------
-// `mul` forms the products and reciprocals (MulFP64 or MulIntT, see hw_device.cuh).
-template <int DIR, bool LINEAR, bool CHAR, class R, class M>
-__device__ __forceinline__ void interface_values_m(const R* r0, const R* r1, const R* r2,
+template <int DIR, bool LINEAR, bool CHAR, class R>
+__device__ __forceinline__ void interface_values(const R* r0, const R* r1, const R* r2,
                                                    const R* r3, int stride, const R qb[6], R g,
-                                                   R eps_w, R out[12], M& mul) {
+                                                   R eps_w, R out[12]) {
 #define RV(r, f) (r)[(f) * stride]
   // interface state: h = (h_i + h_{i+1})/2, u = (m_i + m_{i+1})/(h_i + h_{i+1}), v likewise
   const R hs = RV(r1, R_H) + RV(r2, R_H);
-  const R rhs = mul.rcp(hs);
-  const R ub = mul(RV(r1, R_M) + RV(r2, R_M), rhs);
-  const R vb = mul(RV(r1, R_W) + RV(r2, R_W), rhs);
-  const R gh = mul(mul.k(R(0.5), g), hs);
+  const R rhs = fast_rcp(hs);
+  const R ub = (RV(r1, R_M) + RV(r2, R_M)) * rhs;
+  const R vb = (RV(r1, R_W) + RV(r2, R_W)) * rhs;
+  const R gh = (R(0.5) * g) * hs;
   const R rs = fast_rsqrt(gh);
-  const R ic2 = mul.k(R(0.5), rs);  // 1/(2c)
+  const R ic2 = R(0.5) * rs;  // 1/(2c)
   // normal / tangential velocity of this sweep
   const R un = DIR == 0 ? ub : vb, ut = DIR == 0 ? vb : ub;
-  // un +- c with c = gh / sqrt(gh): fmas (a product on the integer pipes would leave the adds)
+  // un +- c with c = gh / sqrt(gh)
   const R upc = fma(gh, rs, un), umc = fma(-gh, rs, un);
   // component indices: normal momentum and tangential momentum
   const int cn = DIR == 0 ? 1 : 2, ct = DIR == 0 ? 2 : 1;
   // scaled epsilon: fields 1, 3 carry s = 4c, field 2 carries s = 2 (both 2 without projection)
-  const R eps2 = mul.k(R(4.0), eps_w);
-  const R eps13 = CHAR ? mul(mul(mul.k(R(8.0), g), eps_w), hs) : eps2;
+  const R eps2 = R(4.0) * eps_w;
+  const R eps13 = CHAR ? (((R(8.0) * g) * eps_w) * hs) : eps2;
 
   R G[3], GB1 = R(0.0), GB3 = R(0.0);  // per-field sums over both sides; source fields 1 and 3
   const R* rp[4] = {r0, r1, r2, r3};
@@ -174,28 +211,28 @@ __device__ __forceinline__ void interface_values_m(const R* r0, const R* r1, con
     for (int k = 0; k < 3; ++k) {
       WeightsT<R> W;
       const R e = (k == 1) ? eps2 : eps13;
-      const R v = hweno_side_m<LINEAR>(f[k][0], f[k][1], f[k][2], p[k][0], p[k][1], p[k][2], e, W, mul);
+      const R v = hweno_side<LINEAR>(f[k][0], f[k][1], f[k][2], p[k][0], p[k][1], p[k][2], e, W);
       G[k] = side == 0 ? v : G[k] + v;
       if (CHAR) {
         // source data per field: (-b, 0, +b) (row entries of the normal-momentum column)
-        if (k == 0) GB1 -= weighted_m(W, qbs[0], qbs[1], qbs[2], mul);
-        if (k == 2) GB3 += weighted_m(W, qbs[0], qbs[1], qbs[2], mul);
+        if (k == 0) GB1 -= weighted(W, qbs[0], qbs[1], qbs[2]);
+        if (k == 2) GB3 += weighted(W, qbs[0], qbs[1], qbs[2]);
       } else {
-        if (k == 1) GB1 += weighted_m(W, qbs[0], qbs[1], qbs[2], mul);  // the normal-momentum component itself
+        if (k == 1) GB1 += weighted(W, qbs[0], qbs[1], qbs[2]);  // the normal-momentum component itself
       }
     }
   }
   // back to physical components: 2 Fhat = R diag(1/s) G * 2
   R F2[3], B2[3];
   if (CHAR) {
-    const R A = mul(G[0] + G[2], ic2);
+    const R A = (G[0] + G[2]) * ic2;
     F2[0] = A;
-    F2[cn] = fma(un, A, mul.k(R(0.5), G[2] - G[0]));
+    F2[cn] = fma(un, A, R(0.5) * (G[2] - G[0]));
     F2[ct] = fma(ut, A, G[1]);
-    const R Bs = mul(GB1 + GB3, ic2);
+    const R Bs = (GB1 + GB3) * ic2;
     B2[0] = Bs;
-    B2[cn] = fma(un, Bs, mul.k(R(0.5), GB3 - GB1));
-    B2[ct] = mul(ut, Bs);
+    B2[cn] = fma(un, Bs, R(0.5) * (GB3 - GB1));
+    B2[ct] = ut * Bs;
   } else {
     F2[0] = G[0]; F2[cn] = G[1]; F2[ct] = G[2];
     B2[0] = R(0.0); B2[cn] = GB1; B2[ct] = R(0.0);
@@ -217,26 +254,193 @@ __device__ __forceinline__ void interface_values_m(const R* r0, const R* r1, con
 #undef RV
 }
 
-// One interface. IMUL: the products run on the integer pipes (hw_fp64_int.h: each product is
-// bit-identical to DMUL, but rounded on its own where the FP64 form may fuse it with an add into an fma,
-// so the results differ from the FP64-pipe form by rounding; the reciprocals stay on the FP64 pipe:
-// moving them raised spills); if any of them leaves the integer fast path (subnormal, infinite or NaN
-// data), the interface is recomputed on the FP64 pipe from the same records.
-template <int DIR, bool LINEAR, bool CHAR, bool IMUL = false, class R>
-__device__ __forceinline__ void interface_values(const R* r0, const R* r1, const R* r2,
-                                                 const R* r3, int stride, const R qb[6], R g,
-                                                 R eps_w, R out[12]) {
-  if constexpr (IMUL && !LINEAR && std::is_same<R, double>::value) {
-    MulIntT<false> mi;
-    interface_values_m<DIR, LINEAR, CHAR>(r0, r1, r2, r3, stride, qb, g, eps_w, out, mi);
-    if (mi.bad) {
-      MulFP64 mf;
-      interface_values_m<DIR, LINEAR, CHAR>(r0, r1, r2, r3, stride, qb, g, eps_w, out, mf);
-    }
-  } else {
-    MulFP64 mf;
-    interface_values_m<DIR, LINEAR, CHAR>(r0, r1, r2, r3, stride, qb, g, eps_w, out, mf);
+// The same interface with the reconstruction and the derivative flux in fixed point (hw_fixed.h), from four
+// records of node_record_fixed. Returns false, with out unspecified, when an operand does not fit.
+template <int DIR, bool CHAR>
+__device__ __forceinline__ bool interface_values_fixed(const double* r0, const double* r1, const double* r2,
+                                                       const double* r3, int stride, const double qb[6],
+                                                       const Dev2D& d, double out[12]) {
+#define RV(r, f) (r)[(f) * stride]
+  const int cn = DIR == 0 ? 1 : 2, ct = DIR == 0 ? 2 : 1;
+  const double* rp[4] = {r0, r1, r2, r3};
+  bool bad = false;
+  // per component: the largest exponent over the four nodes; node s is shifted down by the difference
+  int e0[4], en[4], et[4];
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    uint32_t lo, hi;
+    f64_words(RV(rp[s], R_X), lo, hi);
+    e0[s] = (int)(lo & 0xffffu);
+    const int e1 = (int)(lo >> 16), e2 = (int)(hi & 0xffffu);
+    en[s] = DIR == 0 ? e1 : e2;
+    et[s] = DIR == 0 ? e2 : e1;
+    bad |= (hi >> 16) != 0u;
   }
+  if (bad) return false;
+  const int m0 = max(max(e0[0], e0[1]), max(e0[2], e0[3])), mn = max(max(en[0], en[1]), max(en[2], en[3])),
+            mt = max(max(et[0], et[1]), max(et[2], et[3]));
+  // interface state (as interface_values)
+  const double hs = RV(r1, R_H) + RV(r2, R_H);
+  const double rhs = fast_rcp(hs);
+  const double ub = (RV(r1, R_M) + RV(r2, R_M)) * rhs;
+  const double vb = (RV(r1, R_W) + RV(r2, R_W)) * rhs;
+  const double gh = d.half_g * hs;
+  const double rs = fast_rsqrt(gh);
+  const double un = DIR == 0 ? ub : vb, ut = DIR == 0 ? vb : ub;
+  const double upc = fma(gh, rs, un), umc = fma(-gh, rs, un);
+  const FxEps eps2 = fx_eps(d.fx_eps2, bad);
+  const FxEps eps13 = CHAR ? fx_eps(d.fx_eps13 * hs, bad) : eps2;
+  // units of the fields' data (below 2^57): field k is its component (normal, tangential, normal) plus c_k F_0,
+  // c = (-(un + c), -ut, -(un - c)); a coefficient's shift brings its products to the field's unit
+  int U02 = 0, U1 = 0;
+  FxS ck[3] = {};
+  if (CHAR) {
+    int up, um, uv;
+    const int64_t xp = fx_mantissa(-upc, up), xm = fx_mantissa(-umc, um), xv = fx_mantissa(-ut, uv);
+    const int u0 = m0 - 1082 + 64;
+    U02 = max(max(max(up, um) + u0 + 2, mn - 1078), -900);
+    U1 = max(max(uv + u0 + 2, mt - 1078), -900);
+    bad |= max(U02, U1) > 900;
+    ck[0] = fx_split(xp >> min(U02 - up - u0, 63));
+    ck[1] = fx_split(xv >> min(U1 - uv - u0, 63));
+    ck[2] = fx_split(xm >> min(U02 - um - u0, 63));
+  }
+  // shifts of the four nodes, one byte each
+  auto shifts = [](int b, const int e[4]) {
+    return (uint32_t)min(b - e[0], 63) | ((uint32_t)min(b - e[1], 63) << 8) | ((uint32_t)min(b - e[2], 63) << 16) |
+           ((uint32_t)min(b - e[3], 63) << 24);
+  };
+  const uint32_t s0 = shifts(CHAR ? m0 : m0 + 4, e0), sn = shifts(CHAR ? U02 + 1082 : mn + 4, en),
+                 st = shifts(CHAR ? U1 + 1082 : mt + 4, et);
+  int64_t G[3] = {0, 0, 0}, BA = 0, BD = 0, Q[3] = {0, 0, 0};
+  uint32_t bw = 0;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) bw = max(bw, fx_absw(qb[q]));
+  const int eb = max((int)(bw >> 20), kFxExpMin);  // source candidates: below 2^60, of one unit
+  bad |= eb > kFxExpMax;
+  // derivative of the quintic (eq. Rec-phi), exact: 3 (f_0 - 8 f_1 + 7 f_2) + p_0 - 2 p_1 - 5 p_2 for data below 2^56
+  auto quintic = [](const int64_t f[3], const int64_t p[3]) {
+    return 3 * ((f[0] - f[1]) - 7 * (f[1] - f[2])) + (p[0] - 2 * p[1] - 5 * p[2]);
+  };
+#pragma unroll 1
+  for (int side = 1; side >= 0; --side) {
+    // '+': nodes 0, 1, 2 of (F+, G+); '-': nodes 3, 2, 1 of (F-, -G-)
+    const double* const q = side == 0 ? r0 : r3 + R_FM * stride;
+    const int step = side == 0 ? (int)(r1 - r0) : -(int)(r1 - r0);
+    const uint32_t rev = side == 0 ? 0x3210u : 0x0123u;
+    const uint32_t z0 = __byte_perm(s0, 0, rev), zn = __byte_perm(sn, 0, rev), zt = __byte_perm(st, 0, rev);
+    auto load = [&](int t, int f, uint32_t z) {
+      return (int64_t)__double_as_longlong(q[t * step + f * stride]) >> ((z >> (8 * t)) & 0xffu);
+    };
+    FxS x[3], y[3];
+    if (CHAR) {
+      int64_t f[3], p[3];
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        f[t] = load(t, 0, z0);
+        p[t] = load(t, R_GP, z0);
+        x[t] = fx_split(f[t]);
+        y[t] = fx_split(p[t]);
+        f[t] >>= 4;
+        p[t] >>= 4;
+      }
+      Q[0] = quintic(f, p) - Q[0];  // the mirrored side's derivative counts negative
+    }
+    int64_t v1 = 0, v2 = 0;  // field 1's weights
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int c = CHAR ? (k == 1 ? ct : cn) : (k == 0 ? 0 : k == 1 ? cn : ct);
+      const uint32_t z = CHAR ? (k == 1 ? zt : zn) : (k == 0 ? z0 : k == 1 ? zn : zt);
+      int64_t f[3], p[3];
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        f[t] = load(t, c, z);
+        p[t] = load(t, R_GP + c, z);
+      }
+      if (CHAR) {
+        if (k == 0) Q[1] = quintic(f, p) - Q[1];
+        const FxS a = k == 0 ? ck[0] : k == 1 ? ck[1] : ck[2];
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+          f[t] = fx_mulhi(x[t], a, f[t]);
+          p[t] = fx_mulhi(y[t], a, p[t]);
+        }
+      } else {
+        Q[k] = quintic(f, p) - Q[k];
+      }
+      const FxEps ek = k == 1 ? eps2 : eps13;
+      const int u = CHAR ? (k == 1 ? U1 : U02) : (k == 0 ? m0 : k == 1 ? mn : mt) - 1078;
+      int64_t w1, w2;
+      const int64_t v = fx_hweno_side(f[0], f[1], f[2], p[0], p[1], p[2], ek, u, w1, w2);
+      if (k == 0) G[0] += v;
+      if (k == 1) G[1] += v;
+      if (k == 2) G[2] += v;
+      // the source with the weights of fields 1 and 3 (of the normal component without projection)
+      if (k == (CHAR ? 0 : 1)) { v1 = w1; v2 = w2; }
+      if (k == 2) {
+        const int64_t c3 = fx_from_double(qb[3 * side + 2], eb);
+        const FxS d1 = fx_split(fx_from_double(qb[3 * side], eb) - c3), d2 = fx_split(fx_from_double(qb[3 * side + 1], eb) - c3);
+        if (CHAR) {
+          BA += fx_dot2<2>(d1, fx_split(w1 - v1), d2, fx_split(w2 - v2));
+          BD += c3 + fx_dot2<2>(d1, fx_split(w1 + v1), d2, fx_split(w2 + v2));
+        } else {
+          BD += c3 + fx_dot2<3>(d1, fx_split(v1), d2, fx_split(v2));
+        }
+      }
+    }
+  }
+  // back to physical components: G carries a factor 6, BA and BD (the sums over fields 1 and 3 of -+ and of
+  // the source values) a factor 1/2
+  const int ub_ = eb - 1082;
+  if (CHAR) {
+    const double ic2 = 0.5 * rs;
+    const double A = fx_to_double(G[2] - G[0], U02) * ((1.0 / 6.0) * ic2);
+    out[0] = A;
+    out[cn] = fma(un, A, (1.0 / 12.0) * fx_to_double(G[2] + G[0], U02));
+    out[ct] = fma(ut, A, (1.0 / 6.0) * fx_to_double(G[1], U1));
+    const double Bs = fx_to_double(BA, ub_) * rs;
+    out[3] = Bs;
+    out[3 + cn] = fma(un, Bs, fx_to_double(BD, ub_));
+    out[3 + ct] = ut * Bs;
+  } else {
+    out[0] = (1.0 / 6.0) * fx_to_double(G[0], m0 - 1078);
+    out[cn] = (1.0 / 6.0) * fx_to_double(G[1], mn - 1078);
+    out[ct] = (1.0 / 6.0) * fx_to_double(G[2], mt - 1078);
+    out[3] = 0.0;
+    out[3 + cn] = fx_to_double(BD, ub_);
+    out[3 + ct] = 0.0;
+  }
+  // derivative-equation flux and mixed term
+  if (CHAR) {
+    // the tangential component in its own unit (the field's may be coarser)
+    auto load = [&](int s, int q) { return (int64_t)__double_as_longlong(RV(rp[s], q + ct)) >> min(mt + 4 - et[s], 63); };
+    const int64_t f0[3] = {load(0, R_FP), load(1, R_FP), load(2, R_FP)}, p0[3] = {load(0, R_GP), load(1, R_GP), load(2, R_GP)};
+    const int64_t f1[3] = {load(3, R_FM), load(2, R_FM), load(1, R_FM)}, p1[3] = {load(3, R_GM), load(2, R_GM), load(1, R_GM)};
+    Q[2] = quintic(f0, p0) - quintic(f1, p1);
+  }
+  out[6] = fx_to_double(Q[0], m0 - 1078);
+  out[6 + cn] = fx_to_double(Q[1], CHAR ? U02 : mn - 1078);
+  out[6 + ct] = fx_to_double(Q[2], mt - 1078);
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    out[9 + c] = fma(7.0, RV(r1, R_MIX + c) + RV(r2, R_MIX + c), -(RV(r0, R_MIX + c) + RV(r3, R_MIX + c)));
+#undef RV
+  return !bad;
+}
+
+// An interface whose data does not fit the fixed-point form, from its nodes again on the FP64 pipe: nodes
+// (i - 2 .. i + 1, j) for DIR = 0, (i, j - 2 .. j + 1) for DIR = 1.
+template <int DIR, bool CHAR, bool COH>
+__device__ __noinline__ void interface_fallback(const Dev2D& d, double alpha, int i, int j, size_t on, const double qb[6],
+                                                double out[12]) {
+  double rec[4 * NREC];
+#pragma unroll 1
+  for (int s = 0; s < 4; ++s) {
+    Node12 n;
+    load_node<COH>(d, DIR == 0 ? i - 2 + s : i, DIR == 0 ? j : j - 2 + s, n, on);
+    node_record<DIR>(n, d.g, alpha, rec + s * NREC);
+  }
+  interface_values<DIR, false, CHAR>(rec, rec + NREC, rec + 2 * NREC, rec + 3 * NREC, 1, qb, d.g, d.eps_w, out);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -335,13 +539,14 @@ __device__ __forceinline__ void alpha_exact_range(const Dev2D& d, const unsigned
 // A tile of TILE_T threads forms the node records of TILE_T consecutive extended nodes (x; yc columns of
 // TILE_T / yc extended rows in y), then, after one barrier, the interfaces whose four records lie in the
 // tile: tiles run across line ends, so no grid size leaves a ragged tile. All TILE_T threads must call;
-// sm holds NREC * TILE_T values. on / oi: offsets of the grid in pooled node / interface planes (the
+// sm holds NRECX * TILE_T values (NREC
+// in single precision). on / oi: offsets of the grid in pooled node / interface planes (the
 // batched form keeps the planes' base pointers in the kernel parameters and adds these, so that no
 // per-grid pointer occupies a register). COH: state loads as in ldp.
 // ---------------------------------------------------------------------------------------------
-constexpr int TILE_T = 192;
+constexpr int TILE_T = 128;
 
-template <bool LINEAR, bool CHAR, bool IMUL, bool COH = false, class R>
+template <bool LINEAR, bool CHAR, bool FIXED, bool COH = false, int T = TILE_T, class R>
 __device__ __forceinline__ void sweep_x_tile(const Dev2DT<R>& d, R ax, unsigned E0, R* sm, size_t on = 0,
                                              size_t oi = 0) {
   const unsigned W = d.nx + 4, total = (unsigned)d.ny * W;
@@ -352,15 +557,22 @@ __device__ __forceinline__ void sweep_x_tile(const Dev2DT<R>& d, R ax, unsigned 
       const unsigned j = E / W, e = E - j * W;
       Node12T<R> n;
       load_node<COH>(d, (int)e - 2, (int)j, n, on);
-      R rec[NREC];
-      node_record<0>(n, R(d.g), ax, rec);
+      if constexpr (FIXED && !LINEAR) {
+        R rec[NRECX];
+        node_record_fixed<0>(n, d.g, ax, rec);
 #pragma unroll
-      for (int f = 0; f < NREC; ++f) sm[f * TILE_T + t] = rec[f];
+        for (int f = 0; f < NRECX; ++f) sm[f * T + t] = rec[f];
+      } else {
+        R rec[NREC];
+        node_record<0>(n, R(d.g), ax, rec);
+#pragma unroll
+        for (int f = 0; f < NREC; ++f) sm[f * T + t] = rec[f];
+      }
     }
   }
   __syncthreads();
   const unsigned E = E0 + t;
-  if (t >= TILE_T - 3 || E >= total) return;
+  if (t >= T - 3 || E >= total) return;
   const unsigned j = E / W, k = E - j * W;
   if (k > (unsigned)d.nx) return;
   const size_t o = oi + (size_t)j * (d.nx + 1) + k;
@@ -368,12 +580,17 @@ __device__ __forceinline__ void sweep_x_tile(const Dev2DT<R>& d, R ax, unsigned 
 #pragma unroll
   for (int q = 0; q < 6; ++q) qb[q] = __ldg(d.qbx[q] + o);
   R out[12];
-  interface_values<0, LINEAR, CHAR, IMUL>(sm + t, sm + t + 1, sm + t + 2, sm + t + 3, TILE_T, qb, R(d.g), R(d.eps_w), out);
+  if constexpr (FIXED && !LINEAR) {
+    if (!interface_values_fixed<0, CHAR>(sm + t, sm + t + 1, sm + t + 2, sm + t + 3, T, qb, d, out))
+      interface_fallback<0, CHAR, COH>(d, ax, (int)k, (int)j, on, qb, out);
+  } else {
+      interface_values<0, LINEAR, CHAR>(sm + t, sm + t + 1, sm + t + 2, sm + t + 3, T, qb, R(d.g), R(d.eps_w), out);
+  }
 #pragma unroll
   for (int q = 0; q < 12; ++q) d.X[q][o] = out[q];
 }
 
-template <bool LINEAR, bool CHAR, bool IMUL, bool COH = false, class R>
+template <bool LINEAR, bool CHAR, bool FIXED, bool COH = false, class R>
 __device__ __forceinline__ void sweep_y_tile(const Dev2DT<R>& d, R ay, unsigned E0, int yc, R* sm, size_t on = 0,
                                              size_t oi = 0) {
   const int rows = TILE_T / yc, ifs = rows - 3;
@@ -387,10 +604,17 @@ __device__ __forceinline__ void sweep_y_tile(const Dev2DT<R>& d, R ay, unsigned 
       if (i < d.nx) {
         Node12T<R> n;
         load_node<COH>(d, i, (int)e - 2, n, on);
-        R rec[NREC];
-        node_record<1>(n, R(d.g), ay, rec);
+        if constexpr (FIXED && !LINEAR) {
+          R rec[NRECX];
+          node_record_fixed<1>(n, d.g, ay, rec);
 #pragma unroll
-        for (int f = 0; f < NREC; ++f) sm[f * TILE_T + t] = rec[f];
+          for (int f = 0; f < NRECX; ++f) sm[f * TILE_T + t] = rec[f];
+        } else {
+          R rec[NREC];
+          node_record<1>(n, R(d.g), ay, rec);
+#pragma unroll
+          for (int f = 0; f < NREC; ++f) sm[f * TILE_T + t] = rec[f];
+        }
       }
     }
   }
@@ -406,7 +630,12 @@ __device__ __forceinline__ void sweep_y_tile(const Dev2DT<R>& d, R ay, unsigned 
   for (int q = 0; q < 6; ++q) qb[q] = __ldg(d.qby[q] + o);
   R out[12];
   const R* s0 = sm + t;
-  interface_values<1, LINEAR, CHAR, IMUL>(s0, s0 + yc, s0 + 2 * yc, s0 + 3 * yc, TILE_T, qb, R(d.g), R(d.eps_w), out);
+  if constexpr (FIXED && !LINEAR) {
+    if (!interface_values_fixed<1, CHAR>(s0, s0 + yc, s0 + 2 * yc, s0 + 3 * yc, TILE_T, qb, d, out))
+      interface_fallback<1, CHAR, COH>(d, ay, i, (int)k, on, qb, out);
+  } else {
+      interface_values<1, LINEAR, CHAR>(s0, s0 + yc, s0 + 2 * yc, s0 + 3 * yc, TILE_T, qb, R(d.g), R(d.eps_w), out);
+  }
 #pragma unroll
   for (int q = 0; q < 12; ++q) d.Y[q][o] = out[q];
 }
@@ -416,10 +645,10 @@ __device__ __forceinline__ void sweep_y_tile(const Dev2DT<R>& d, R ay, unsigned 
 // ---------------------------------------------------------------------------------------------
 // Limiter along one direction at one node (Sec. R(2.2)), scaled data. L-rows without 1/(2c):
 // x: (u+c, -1, 0), (-v, 0, 1), (-(u-c), 1, 0); y: (v+c, 0, -1), (-u, 1, 0), (-(v-c), 0, 1).
-template <int DIR, bool LINEAR, bool CHAR, class R, class M>
+template <int DIR, bool LINEAR, bool CHAR, class R>
 __device__ __forceinline__ void limit_dir(const R Um[3], const R U0[3], const R Up[3],
                                           const R Dm[3], const R Dp[3], R u, R v, R c,
-                                          R ic2, R gh, R eps, R out[3], M& mul) {
+                                          R ic2, R gh, R eps, R out[3]) {
   const int cn = DIR == 0 ? 1 : 2, ct = DIR == 0 ? 2 : 1;
   const R un = DIR == 0 ? u : v, ut = DIR == 0 ? v : u;
   const R upc = un + c, umc = un - c;
@@ -434,28 +663,149 @@ __device__ __forceinline__ void limit_dir(const R Um[3], const R U0[3], const R 
   };
   R m0[3], m1[3], m2[3], nl[3], nr[3];
   proj(Um, m0); proj(U0, m1); proj(Up, m2); proj(Dm, nl); proj(Dp, nr);
-  const R e13 = CHAR ? mul(mul.k(R(4.0), eps), gh) : eps;
+  const R e13 = CHAR ? ((R(4.0) * eps) * gh) : eps;
   R nu[3];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) nu[k] = limiter_field_m<LINEAR>(m0[k], m1[k], m2[k], nl[k], nr[k], k == 1 ? eps : e13, mul);
+  for (int k = 0; k < 3; ++k) nu[k] = limiter_field<LINEAR>(m0[k], m1[k], m2[k], nl[k], nr[k], k == 1 ? eps : e13);
   if (CHAR) {
-    const R A = mul(nu[0] + nu[2], ic2);
+    const R A = (nu[0] + nu[2]) * ic2;
     out[0] = A;
-    out[cn] = fma(un, A, mul.k(R(0.5), nu[2] - nu[0]));
+    out[cn] = fma(un, A, R(0.5) * (nu[2] - nu[0]));
     out[ct] = fma(ut, A, nu[1]);
   } else {
     out[0] = nu[0]; out[cn] = nu[1]; out[ct] = nu[2];
   }
 }
 
-// RHS assembly, limiter and RK combination (or the bare RHS) at node (i, j) of one grid, products
-// formed by `mul`. With MulInt nothing is written when a product left the integer fast path
-// (mul.bad); the caller then recomputes the node with MulFP64 from the same (unchanged) inputs.
-// on, oxo, oyo: offsets of the grid in pooled node, x-interface and y-interface planes (0 for one grid).
-// COH: loads of the state, interface and base planes as in ldp.
-template <int MODE, bool LINEAR, bool CHAR, bool COH, class R, class M>
-__device__ __forceinline__ void node_update_m(const Dev2DT<R>& d, const StageArgsT<R>& sa, int i, int j, M& mul,
-                                              size_t on = 0, size_t oxo = 0, size_t oyo = 0) {
+// The limiter of both directions at node (i, j) on the FP64 pipe: scaled V and Q of the node into mod.
+template <bool LINEAR, bool CHAR, bool COH, class R>
+__device__ __forceinline__ void limit_node(const Dev2DT<R>& d, int i, int j, size_t on, const R cur[9], R mod[6]) {
+  const R h = cur[0] - __ldg(d.stat[0] + on + (size_t)j * d.nx + i);
+  const R gh = R(d.g) * h;
+  const R rh = fast_rcp(h);
+  const R u = cur[1] * rh, v = cur[2] * rh;
+  const R rs = fast_rsqrt(gh);
+  const R c = gh * rs, ic2 = R(0.5) * rs;
+  Node12T<R> nm, np;
+  load_node<COH>(d, i - 1, j, nm, on);
+  load_node<COH>(d, i + 1, j, np, on);
+  limit_dir<0, LINEAR, CHAR>(nm.v, cur, np.v, nm.v + 3, np.v + 3, u, v, c, ic2, gh, R(d.eps_lim), mod);
+  load_node<COH>(d, i, j - 1, nm, on);
+  load_node<COH>(d, i, j + 1, np, on);
+  limit_dir<1, LINEAR, CHAR>(nm.v, cur, np.v, nm.v + 6, np.v + 6, u, v, c, ic2, gh, R(d.eps_lim), mod + 3);
+}
+
+// The same as a call, for the nodes whose data does not fit the fixed-point form.
+template <bool CHAR, bool COH>
+__device__ __noinline__ void limit_node_fallback(const Dev2D& d, int i, int j, size_t on, const double* cur, double* mod) {
+  limit_node<false, CHAR, COH>(d, i, j, on, cur, mod);
+}
+
+// The same in fixed point (hw_fixed.h): the node and its four neighbours as integers of one unit per component,
+// the differences and derivatives projected and limited field by field. False (mod unspecified) when an operand
+// does not fit.
+template <bool CHAR, bool COH>
+__device__ __forceinline__ bool limit_node_fixed(const Dev2D& d, int i, int j, size_t on, const double cur[9],
+                                                 double mod[6]) {
+  // U of the node, then of the neighbours W, E, S, N; their derivatives along x (W, E) or y (S, N)
+  double U[5][3], D[4][3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) U[0][c] = cur[c];
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    bool fx, fy;
+    const int ii = map_index(s == 0 ? i - 1 : s == 1 ? i + 1 : i, d.nx, d.bc_x, fx);
+    const int jj = map_index(s == 2 ? j - 1 : s == 3 ? j + 1 : j, d.ny, d.bc_y, fy);
+    const size_t o = on + (size_t)jj * d.nx + ii;
+    const uint32_t m = (s < 2 ? fx : fy) ? 0x80000000u : 0u;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int q = (s < 2 ? 3 : 6) + c;
+      U[s + 1][c] = flip_sign(ldp<COH>(d.S[c] + o), (s < 2 ? par_x2d(c) : par_y2d(c)) < 0 ? m : 0u);
+      D[s][c] = flip_sign(ldp<COH>(d.S[q] + o), (s < 2 ? par_x2d(q) : par_y2d(q)) < 0 ? m : 0u);
+    }
+  }
+  bool bad = false;
+  int em[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    uint32_t w = 0, any = 0;
+#pragma unroll
+    for (int s = 0; s < 5; ++s) { w = max(w, fx_absw(U[s][c])); any |= fx_any(U[s][c]); }
+#pragma unroll
+    for (int s = 0; s < 4; ++s) { w = max(w, fx_absw(D[s][c])); any |= fx_any(D[s][c]); }
+    em[c] = (int)(w >> 20);
+    bad |= (em[c] > kFxExpMax) | ((em[c] < kFxExpMin) & (any != 0u));
+    em[c] = max(em[c], kFxExpMin);
+  }
+  const double h = cur[0] - __ldg(d.stat[0] + on + (size_t)j * d.nx + i);
+  const double gh = d.g * h;
+  const double rh = fast_rcp(h);
+  const double u = cur[1] * rh, v = cur[2] * rh;
+  const double rs = fast_rsqrt(gh);
+  const FxEps eps2 = fx_eps(d.fx_eps2l, bad);
+  const FxEps eps13 = CHAR ? fx_eps(d.fx_eps13l * h, bad) : eps2;
+  if (bad) return false;
+  int64_t c0[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) c0[c] = fx_from_double(U[0][c], em[c]);
+#pragma unroll
+  for (int dir = 0; dir < 2; ++dir) {
+    const int cn = dir == 0 ? 1 : 2, ct = dir == 0 ? 2 : 1;
+    // differences to the two neighbours and their derivatives, below 2^61
+    int64_t a[4][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      a[0][c] = c0[c] - fx_from_double(U[1 + 2 * dir][c], em[c]);
+      a[1][c] = fx_from_double(U[2 + 2 * dir][c], em[c]) - c0[c];
+      a[2][c] = fx_from_double(D[2 * dir][c], em[c]);
+      a[3][c] = fx_from_double(D[2 * dir + 1][c], em[c]);
+    }
+    double* const out = mod + 3 * dir;
+    if (CHAR) {
+      const double un = dir == 0 ? u : v, ut = dir == 0 ? v : u;
+      // rows (-(un + c), 1, 0), (-ut, 0, 1), (-(un - c), 1, 0) on (mass, normal, tangential)
+      const double upc = fma(gh, rs, un), umc = fma(-gh, rs, un);
+      int up, um, uv;
+      const int64_t xp = fx_mantissa(-upc, up), xm = fx_mantissa(-umc, um), xv = fx_mantissa(-ut, uv);
+      const int u0 = em[0] - 1082 + 64;
+      const int U02 = max(max(max(up, um) + u0 + 2, em[cn] - 1078), -900), U1 = max(max(uv + u0 + 2, em[ct] - 1078), -900);
+      if (max(U02, U1) > 900) return false;
+      const FxS kp = fx_split(xp >> min(U02 - up - u0, 63)), km = fx_split(xm >> min(U02 - um - u0, 63)),
+                kv = fx_split(xv >> min(U1 - uv - u0, 63));
+      const int sn = min(U02 + 1082 - em[cn], 63), st = min(U1 + 1082 - em[ct], 63);
+      int64_t nu[3];
+      FxS x[4];
+#pragma unroll
+      for (int s = 0; s < 4; ++s) x[s] = fx_split(a[s][0]);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const FxS kk = k == 0 ? kp : k == 1 ? kv : km;
+        int64_t f[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) f[s] = fx_mulhi(x[s], kk, k == 1 ? a[s][ct] >> st : a[s][cn] >> sn);
+        nu[k] = fx_limiter_field(f[0], f[1], f[2], f[3], k == 1 ? eps2 : eps13, k == 1 ? U1 : U02);
+      }
+      const double A = fx_to_double(nu[2] - nu[0], U02 - 1) * (0.5 * rs);
+      out[0] = A;
+      out[cn] = fma(un, A, fx_to_double(nu[2] + nu[0], U02 - 2));
+      out[ct] = fma(ut, A, fx_to_double(nu[1], U1 - 1));
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        out[c] = fx_to_double(fx_limiter_field(a[0][c] >> 3, a[1][c] >> 3, a[2][c] >> 3, a[3][c] >> 3, eps2, em[c] - 1079),
+                              em[c] - 1080);
+    }
+  }
+  return true;
+}
+
+// RHS assembly, limiter and RK combination (or the bare RHS) at node (i, j) of one grid. FIXED: the limiter in
+// fixed point where the node's data fits it. on, oxo, oyo: offsets of the grid in pooled node, x-interface and
+// y-interface planes (0 for one grid). COH: loads of the state, interface and base planes as in ldp.
+template <int MODE, bool LINEAR, bool CHAR, bool FIXED = false, bool COH = false, class R>
+__device__ __forceinline__ void node_update(const Dev2DT<R>& d, const StageArgsT<R>& sa, int i, int j, size_t on = 0,
+                                            size_t oxo = 0, size_t oyo = 0) {
   const size_t o = on + (size_t)j * d.nx + i;
   const size_t ox = oxo + (size_t)j * (d.nx + 1) + i;  // left x-interface; right is ox + 1
   const size_t oy = oyo + (size_t)j * d.nx + i;        // lower y-interface; upper is oy + nx
@@ -468,13 +818,27 @@ __device__ __forceinline__ void node_update_m(const Dev2DT<R>& d, const StageArg
     for (int q = 0; q < 9; ++q) sa.out[q][o] = cur[q];
     return;
   }
+  // ---- limiter (Sec. R(2.2), dimension by dimension) ----
+  R mod[6];
+  if (MODE == MODE_STAGE) {
+    if (sa.limiter) {
+      if constexpr (FIXED && !LINEAR && std::is_same<R, double>::value) {
+        if (!limit_node_fixed<CHAR, COH>(d, i, j, on, cur, mod)) limit_node_fallback<CHAR, COH>(d, i, j, on, cur, mod);
+      } else {
+        limit_node<LINEAR, CHAR, COH>(d, i, j, on, cur, mod);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 6; ++q) mod[q] = cur[3 + q];
+    }
+  }
+  // ---- RHS (eq. swe-form-2d-dis) in scaled units: R_U, dx R_V, dy R_Q ----
   const R eta = cur[0], H1 = cur[3], H2 = cur[6];
   const R g = R(d.g);
   // grid constants in the working precision
   const R c_bx = R(d.c_bx), c_by = R(d.c_by), c_gx = R(d.c_gx), c_gy = R(d.c_gy), c_mx = R(d.c_mx),
           c_my = R(d.c_my);
-  const R ge = mul(g, eta);
-  // ---- RHS (eq. swe-form-2d-dis) in scaled units: R_U, dx R_V, dy R_Q ----
+  const R ge = g * eta;
   R Rv[9];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -486,53 +850,29 @@ __device__ __forceinline__ void node_update_m(const Dev2DT<R>& d, const StageArg
     const R dGy = ldp<COH>(d.Y[6 + c] + oy + d.nx) - ldp<COH>(d.Y[6 + c] + oy);
     const R dMx = ldp<COH>(d.X[9 + c] + ox + 1) - ldp<COH>(d.X[9 + c] + ox);
     const R dMy = ldp<COH>(d.Y[9 + c] + oy + d.nx) - ldp<COH>(d.Y[9 + c] + oy);
-    const R db = fma(c_bx, dbx, mul(c_by, dby));  // [b~]_x/dx + [b-]_y/dy
-    Rv[c] = fma(-ge, db, fma(-c_bx, dFx, -mul(c_by, dFy)));
-    R rv = fma(-c_gx, dGx, -mul(c_my, dMy));
-    R rq = fma(-c_mx, dMx, -mul(c_gy, dGy));
+    const R db = fma(c_bx, dbx, c_by * dby);  // [b~]_x/dx + [b-]_y/dy
+    Rv[c] = fma(-ge, db, fma(-c_bx, dFx, -(c_by * dFy)));
+    R rv = fma(-c_gx, dGx, -(c_my * dMy));
+    R rq = fma(-c_mx, dMx, -(c_gy * dGy));
     if (c > 0) {
       rv = fma(-ge, __ldg(d.sv[c - 1] + o), rv);
       rq = fma(-ge, __ldg(d.sq[c - 1] + o), rq);
     }
-    Rv[3 + c] = fma(-mul(g, H1), db, rv);
-    Rv[6 + c] = fma(-mul(g, H2), db, rq);
+    Rv[3 + c] = fma(-(g * H1), db, rv);
+    Rv[6 + c] = fma(-(g * H2), db, rq);
   }
   if (MODE == MODE_RHS) {
-    if (mul.bad) return;
     // physical units: R_V = (dx R_V)/dx, R_Q = (dy R_Q)/dy
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
       const R s = q < 3 ? R(1.0) : R(q < 6 ? d.inv_dx : d.inv_dy);
-      sa.rhs_out[q][o] = mul(Rv[q], s);
+      sa.rhs_out[q][o] = Rv[q] * s;
     }
     return;
-  }
-  // ---- limiter (Sec. R(2.2), dimension by dimension) ----
-  R mod[6];
-  if (sa.limiter) {
-    const R b0 = __ldg(d.stat[0] + o);
-    const R h = eta - b0;
-    const R gh = mul(g, h);
-    const R rh = mul.rcp(h);
-    const R u = mul(cur[1], rh), v = mul(cur[2], rh);
-    const R rs = fast_rsqrt(gh);
-    const R c = mul(gh, rs), ic2 = mul.k(R(0.5), rs);
-    Node12T<R> nm, np;
-    // x neighbours
-    load_node<COH>(d, i - 1, j, nm, on);
-    load_node<COH>(d, i + 1, j, np, on);
-    limit_dir<0, LINEAR, CHAR>(nm.v, cur, np.v, nm.v + 3, np.v + 3, u, v, c, ic2, gh, R(d.eps_lim), mod, mul);
-    load_node<COH>(d, i, j - 1, nm, on);
-    load_node<COH>(d, i, j + 1, np, on);
-    limit_dir<1, LINEAR, CHAR>(nm.v, cur, np.v, nm.v + 6, np.v + 6, u, v, c, ic2, gh, R(d.eps_lim), mod + 3, mul);
-  } else {
-#pragma unroll
-    for (int q = 0; q < 6; ++q) mod[q] = cur[3 + q];
   }
   // ---- SSP-RK3 combination (eq. RK) ----
   const R dt = R(*sa.dt);
   if (sa.k == 1) {
-    if (mul.bad) return;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
       const R cq = q < 3 ? cur[q] : mod[q - 3];
@@ -542,35 +882,11 @@ __device__ __forceinline__ void node_update_m(const Dev2DT<R>& d, const StageArg
   } else {
     const R a = sa.k == 2 ? R(0.75) : R(1.0) / R(3.0);
     const R b = sa.k == 2 ? R(0.25) : R(2.0) / R(3.0);
-    R res[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
       const R cq = q < 3 ? cur[q] : mod[q - 3];
-      res[q] = fma(a, ldp<COH>(sa.base[q] + o), mul(b, fma(dt, Rv[q], cq)));
+      sa.out[q][o] = fma(a, ldp<COH>(sa.base[q] + o), b * fma(dt, Rv[q], cq));
     }
-    if (mul.bad) return;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) sa.out[q][o] = res[q];
-  }
-}
-
-// The node update. IMUL: products on the integer pipes (each bit-identical to DMUL; results differ from
-// the fma-contracted FP64-pipe form by rounding); if any leaves the integer fast path, the node is
-// recomputed on the FP64 pipe, so an interface or node on that fallback rounds differently from its
-// neighbours, within the same tolerances (int_mul_fallback parity case).
-template <int MODE, bool LINEAR, bool CHAR, bool IMUL = false, bool COH = false, class R>
-__device__ __forceinline__ void node_update(const Dev2DT<R>& d, const StageArgsT<R>& sa, int i, int j, size_t on = 0,
-                                            size_t oxo = 0, size_t oyo = 0) {
-  if constexpr (IMUL && !LINEAR && std::is_same<R, double>::value) {
-    MulInt mi;
-    node_update_m<MODE, LINEAR, CHAR, COH>(d, sa, i, j, mi, on, oxo, oyo);
-    if (mi.bad) {
-      MulFP64 mf;
-      node_update_m<MODE, LINEAR, CHAR, COH>(d, sa, i, j, mf, on, oxo, oyo);
-    }
-  } else {
-    MulFP64 mf;
-    node_update_m<MODE, LINEAR, CHAR, COH>(d, sa, i, j, mf, on, oxo, oyo);
   }
 }
 
