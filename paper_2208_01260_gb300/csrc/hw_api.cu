@@ -13,7 +13,8 @@
 
 namespace hw {
 // 1D alpha's reduction with its finish in one launch (hw_kernels1d.cu): slot[0..1] are zero between
-// launches (cleared by each launch's last block); same alpha and step as the separate launches.
+// launches (cleared by each launch's last block, with slot[2], the flags of a stage's output); same alpha and
+// step as the separate launches.
 void launch_alpha_finish1d(const Dev1D& d, unsigned long long* slot, int* status, double* alpha, double* dt_out,
                            double cfl, const double* t_now, double t_end, cudaStream_t st);
 }  // namespace hw
@@ -220,7 +221,7 @@ int hw_create(const hw_grid* grid, const hw_params* params, void* cuda_stream, h
     const double dy = (grid->y1 - grid->y0) / ny;
     d.nx = nx; d.ny = ny; d.bc_x = grid->bc_x; d.bc_y = grid->bc_y;
     set_spacing2d(d, dx, dy);
-    hw::set_physics2d(d, params->g, params->eps_w, params->eps_lim);
+    hw::set_physics(d, params->g, params->eps_w, params->eps_lim);
     for (int q = 0; q < 3; ++q) A(&d.stat[q], s->n);
     for (int q = 0; q < 2; ++q) A(&d.bxy[q], s->n);
     for (int q = 0; q < 12; ++q) { A(&d.X[q], (size_t)(nx + 1) * ny); A(&d.Y[q], (size_t)nx * (ny + 1)); }
@@ -234,7 +235,7 @@ int hw_create(const hw_grid* grid, const hw_params* params, void* cuda_stream, h
       for (int q = 0; q < 9; ++q) { F(&s->FA[q], s->n); F(&s->FB[q], s->n); F(&s->fbase[q], s->n); }
       f.nx = d.nx; f.ny = d.ny; f.bc_x = d.bc_x; f.bc_y = d.bc_y;
       f.dx = (float)d.dx; f.dy = (float)d.dy; f.inv_dx = (float)d.inv_dx; f.inv_dy = (float)d.inv_dy;
-      hw::set_physics2d(f, d.g, d.eps_w, d.eps_lim);
+      hw::set_physics(f, d.g, d.eps_w, d.eps_lim);
       f.c_bx = (float)d.c_bx; f.c_by = (float)d.c_by; f.c_gx = (float)d.c_gx; f.c_gy = (float)d.c_gy;
       f.c_mx = (float)d.c_mx; f.c_my = (float)d.c_my;
       F(&s->fsc, 4);
@@ -247,7 +248,7 @@ int hw_create(const hw_grid* grid, const hw_params* params, void* cuda_stream, h
   } else {
     hw::Dev1D& d = s->d1;
     d.nx = nx; d.bc = grid->bc_x; d.dx = dx; d.inv_dx = 1.0 / dx;
-    d.g = params->g; d.eps_w = params->eps_w; d.eps_lim = params->eps_lim;
+    hw::set_physics(d, params->g, params->eps_w, params->eps_lim);
     d.c_b = 0.5 / dx; d.c_g = 1.0 / (24.0 * dx);
     for (int q = 0; q < 2; ++q) A(&d.stat[q], s->n);
     A(&d.bx, s->n);
@@ -260,7 +261,7 @@ int hw_create(const hw_grid* grid, const hw_params* params, void* cuda_stream, h
   cudaError_t e = cudaStreamCreateWithFlags(&s->cap_stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) { s->cap_stream = nullptr; hw_destroy(s); return fail(HW_ERR_CUDA, cudaGetErrorString(e)); }
   e = cudaMemsetAsync(misc, 0, 16 * sizeof(double), s->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(s->amax + 2, 0, 2 * sizeof(unsigned long long), s->stream);  // 1D alpha slots
+  if (e == cudaSuccess) e = cudaMemsetAsync(s->amax + 2, 0, 4 * sizeof(unsigned long long), s->stream);  // 1D alpha slots
   if (e != cudaSuccess) { hw_destroy(s); return fail(HW_ERR_CUDA, cudaGetErrorString(e)); }
   bind_state(s, s->SA);
   *out = s;
@@ -374,9 +375,13 @@ static void enqueue_alpha(hw_solver* s, bool with_dt, double t_end) {
   }, s->is2d() ? (s->fp32 ? 2 : 3) : 1);  // reduction (two passes in 2D double) and finish; one launch in 1D
 }
 
+// Whether the solver's stages are single launches that also form the next stage's alpha (hw_step1d.cu).
+static bool fused1d(const hw_solver* s) { return !s->is2d() && s->params.linear_weights == 0; }
+
 // One stage: sweeps on the current state (alpha already in s->alpha), node kernel into the other
-// buffer, then swap.
-static void enqueue_stage(hw_solver* s, int k) {
+// buffer, then swap. next (1D): the launch also forms the next stage's alpha and, after stage 3, the time and
+// the next step (clipped to t_end).
+static void enqueue_stage(hw_solver* s, int k, bool next = false, double t_end = -1.0) {
   static const char* kNames[4] = {"", "stage 1", "stage 2", "stage 3"};
   Range nvtx_range(kNames[k]);
   double** in = s->state();
@@ -400,11 +405,16 @@ static void enqueue_stage(hw_solver* s, int k) {
     for (int q = 0; q < 9; ++q) { sa.out[q] = out[q]; sa.base[q] = s->base[q]; }
     timed(s, HW_PROF_NODE, [&] { hw::launch_node2d(s->d2, sa, hw::MODE_STAGE, lin, chr, s->stream); });
   } else {
-    timed(s, HW_PROF_SWEEP_X, [&] { hw::launch_sweep1d(s->d1, s->alpha, lin, chr, s->stream); });
     hw::StageArgs1D sa{};
     sa.k = k; sa.limiter = s->params.limiter; sa.dt = s->dt;
     for (int q = 0; q < 4; ++q) { sa.out[q] = out[q]; sa.base[q] = s->base[q]; }
-    timed(s, HW_PROF_NODE, [&] { hw::launch_node1d(s->d1, sa, hw::MODE_STAGE, lin, chr, s->stream); });
+    if (fused1d(s)) {
+      const hw::Time1D tm{s->amax + 2, s->status, s->alpha, s->dt, s->nsteps, s->params.cfl};
+      timed(s, HW_PROF_NODE, [&] { hw::launch_stage1d(s->d1, sa, tm, next, t_end, chr, s->stream); });
+    } else {
+      timed(s, HW_PROF_SWEEP_X, [&] { hw::launch_sweep1d(s->d1, s->alpha, chr, s->stream); });
+      timed(s, HW_PROF_NODE, [&] { hw::launch_node1d(s->d1, sa, hw::MODE_STAGE, chr, s->stream); });
+    }
   }
   s->cur ^= 1;
 }
@@ -428,17 +438,23 @@ int hw_rk3_step(hw_solver* s, double dt) {
   if (!s->inited) return fail(HW_ERR_STATE, "hw_rk3_step: call hw_init first");
   if (!(dt >= 0) || !(dt < 1e300)) return fail(HW_ERR_ARG, "hw_rk3_step: dt must be finite and >= 0");
   timed(s, HW_PROF_OTHER, [&] { k_set_scalar<<<1, 1, 0, s->stream>>>(s->dt, dt); });
+  const bool fused = fused1d(s);
   for (int k = 1; k <= 3; ++k) {
-    enqueue_alpha(s, false, -1.0);
-    enqueue_stage(s, k);
+    if (k == 1 || !fused) enqueue_alpha(s, false, -1.0);
+    enqueue_stage(s, k, fused && k < 3);
   }
   timed(s, HW_PROF_OTHER, [&] { k_add_time<<<1, 1, 0, s->stream>>>(s->t, s->dt, 0, s->nsteps); });
   CUDA_OK(cudaGetLastError());
   return HW_OK;
 }
 
-// One step with dt computed on the device from U^n (clipped to t_end when t_end > 0).
+// One step with dt computed on the device from U^n (clipped to t_end when t_end > 0). In 1D alpha and the step are
+// on the device already: formed by the step before, or by enqueue_alpha before the first.
 static void enqueue_cfl_step(hw_solver* s, double t_end) {
+  if (fused1d(s)) {
+    for (int k = 1; k <= 3; ++k) enqueue_stage(s, k, true, t_end);
+    return;
+  }
   enqueue_alpha(s, true, t_end);
   enqueue_stage(s, 1);
   for (int k = 2; k <= 3; ++k) {
@@ -462,6 +478,9 @@ int hw_advance(hw_solver* s, int nsteps, double t_end, int use_graph, double* t_
   const bool has_end = t_end > 0.0;
   // A captured graph holds two steps (an even number of stages returns to the same buffer).
   if (s->profiling) use_graph = 0;
+  // small 1D grids: whole chunks of steps in one launch each, no graph
+  const bool run1d = fused1d(s) && hw::run1d_fits(s->d1);
+  if (run1d) use_graph = 0;
   if (use_graph && (!s->graph || s->graph_t_end != t_end || s->cur != 0)) {
     if (s->graph) { cudaGraphExecDestroy(s->graph); s->graph = nullptr; }
     if (s->cur == 0) {
@@ -488,13 +507,25 @@ int hw_advance(hw_solver* s, int nsteps, double t_end, int use_graph, double* t_
   // With an end time the host reads the time back between chunks of steps: two steps at first, then half
   // the steps the last step size leaves to t_end (a step past t_end has size 0 and changes nothing), so a
   // run of n steps waits O(log n) times instead of n/2.
-  int chunk = has_end ? 2 : 1 << 30;
+  int chunk = !has_end ? 1 << 30 : run1d ? 1024 : 2;  // a run's launch ends by itself at t_end
   double t = t0;
+  if (fused1d(s) && nsteps > 0 && !(has_end && t >= t_end)) enqueue_alpha(s, true, t_end);
   while (done < nsteps) {
     if (has_end && t >= t_end) break;
     int todo = std::min(nsteps - done, chunk);
     while (todo > 0) {
-      if (use_graph && s->graph && s->cur == 0 && todo >= 2) {
+      if (run1d) {
+        const int m = std::min(todo, 1024);  // a launch stays within some ten milliseconds
+        bind_state(s, s->state());
+        const hw::Time1D tm{s->amax + 2, s->status, s->alpha, s->dt, s->nsteps, s->params.cfl};
+        int e = 0;
+        timed(s, HW_PROF_NODE, [&] {
+          e = hw::launch_run1d(s->d1, s->base, tm, m, s->params.limiter, t_end, s->params.char_decomp != 0, s->stream);
+        });
+        CUDA_OK((cudaError_t)e);
+        todo -= m;
+        done += m;
+      } else if (use_graph && s->graph && s->cur == 0 && todo >= 2) {
         CUDA_OK(cudaGraphLaunch(s->graph, s->stream));
         todo -= 2;
         done += 2;
@@ -511,7 +542,7 @@ int hw_advance(hw_solver* s, int nsteps, double t_end, int use_graph, double* t_
       CUDA_OK(cudaStreamSynchronize(s->stream));
       t = dt_t[2];
       const double left = dt_t[0] > 0.0 ? (t_end - t) / dt_t[0] : 0.0;
-      chunk = 2 * std::max(1, (int)std::min(0.25 * left, 1e6));
+      chunk = run1d ? chunk : 2 * std::max(1, (int)std::min(0.25 * left, 1e6));
     }
   }
   CUDA_OK(cudaMemcpyAsync(&t, s->t, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
@@ -573,10 +604,14 @@ int hw_rhs(hw_solver* s, double* const* out, int ptr_kind) {
     for (int q = 0; q < 9; ++q) sa.rhs_out[q] = dst[q];
     hw::launch_node2d(s->d2, sa, hw::MODE_RHS, lin, chr, s->stream);
   } else {
-    hw::launch_sweep1d(s->d1, s->alpha, lin, chr, s->stream);
     hw::StageArgs1D sa{};
     for (int q = 0; q < 4; ++q) sa.rhs_out[q] = dst[q];
-    hw::launch_node1d(s->d1, sa, hw::MODE_RHS, lin, chr, s->stream);
+    if (fused1d(s)) {
+      hw::launch_rhs1d(s->d1, sa, s->alpha, chr, s->stream);
+    } else {
+      hw::launch_sweep1d(s->d1, s->alpha, chr, s->stream);
+      hw::launch_node1d(s->d1, sa, hw::MODE_RHS, chr, s->stream);
+    }
   }
   CUDA_OK(cudaGetLastError());
   if (ptr_kind == HW_HOST)

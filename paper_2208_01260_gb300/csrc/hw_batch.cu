@@ -212,7 +212,7 @@ hw::Dev2D dev_of(hw_batch* b, int i, double** S) {
   hw::Dev2D d{};
   d.nx = I.nx; d.ny = I.ny; d.bc_x = I.bc_x; d.bc_y = I.bc_y;
   d.dx = I.dx; d.dy = I.dy; d.inv_dx = I.inv_dx; d.inv_dy = I.inv_dy;
-  hw::set_physics2d(d, b->params.g, b->params.eps_w, b->params.eps_lim);
+  hw::set_physics(d, b->params.g, b->params.eps_w, b->params.eps_lim);
   d.c_bx = I.c_bx; d.c_by = I.c_by; d.c_gx = I.c_gx; d.c_gy = I.c_gy; d.c_mx = I.c_mx; d.c_my = I.c_my;
   for (int q = 0; q < 9; ++q) d.S[q] = S[q] + I.off_n;
   for (int q = 0; q < 3; ++q) d.stat[q] = b->B.stat[q] + I.off_n;
@@ -406,7 +406,7 @@ int hw_batch_create(int n, const hw_grid* grids, const hw_params* params, void* 
   b->B.t = misc + 7 * n;
   b->B.nsteps = (unsigned long long*)(misc + 8 * n);
   b->B.status = (int*)(misc + 9 * n);
-  hw::set_physics2d(b->B, params->g, params->eps_w, params->eps_lim);
+  hw::set_physics(b->B, params->g, params->eps_w, params->eps_lim);
   b->B.cfl = params->cfl;
   b->B.limiter = params->limiter;
   b->B.inst = b->d_inst;

@@ -36,7 +36,7 @@ using Dev2D = Dev2DT<double>;
 
 // g and the weights' epsilons with the constants derived from them.
 template <class D>
-inline void set_physics2d(D& d, double g, double eps_w, double eps_lim) {
+inline void set_physics(D& d, double g, double eps_w, double eps_lim) {
   using R = decltype(d.g);
   d.g = (R)g;
   d.eps_w = (R)eps_w;
@@ -76,6 +76,7 @@ struct Dev1D {
   int nx, bc;
   double dx, inv_dx, g, eps_w, eps_lim;
   double c_b, c_g;   // 1/(2dx), 1/(24dx)
+  double half_g, fx_eps13, fx_eps2, fx_eps13l, fx_eps2l;  // as in Dev2DT
   double* S[4];      // eta, m, dx H, dx M
   double* stat[2];   // b, dx b_x
   double* bx;        // b_x
@@ -130,8 +131,27 @@ int set_last_error(int code, const char* msg);
 void launch_alpha1d(const Dev1D& d, unsigned long long* amax, int* status, cudaStream_t st);
 void launch_finish_alpha1d(const Dev1D& d, const unsigned long long* amax, double* alpha, double* dt_out,
                            double cfl, const double* t_now, double t_end, cudaStream_t st);
-void launch_sweep1d(const Dev1D& d, const double* alpha, bool linear, bool chr, cudaStream_t st);
-void launch_node1d(const Dev1D& d, const StageArgs1D& sa, int mode, bool linear, bool chr, cudaStream_t st);
+// linear weights only (hw_step1d.cu has the scheme's own)
+void launch_sweep1d(const Dev1D& d, const double* alpha, bool chr, cudaStream_t st);
+void launch_node1d(const Dev1D& d, const StageArgs1D& sa, int mode, bool chr, cudaStream_t st);
+// The scheme's 1D right-hand side, and one RK stage (hw_step1d.cu), each one launch with alpha on the device. With
+// next the stage also forms the next stage's alpha and, after stage 3, the time and the next step's size.
+struct Time1D {
+  unsigned long long* slot;  // 4, zero before the first launch
+  int* status;
+  double* alpha;
+  double* dt;  // step, time after it, time
+  unsigned long long* nsteps;
+  double cfl;
+};
+void launch_rhs1d(const Dev1D& d, const StageArgs1D& sa, const double* alpha, bool chr, cudaStream_t st);
+// Up to nsteps whole steps of a small grid (run1d_fits) in one launch, from d.S back into d.S, with alpha and the
+// first step's size on the device; ends early at t_end > 0. Returns the launch's cudaError_t.
+bool run1d_fits(const Dev1D& d);
+int launch_run1d(const Dev1D& d, double* const base[4], const Time1D& tm, int nsteps, int limiter, double t_end, bool chr,
+                 cudaStream_t st);
+void launch_stage1d(const Dev1D& d, const StageArgs1D& sa, const Time1D& tm, bool next, double t_end, bool chr,
+                    cudaStream_t st);
 void launch_init1d(const Dev1D& d, const PhysIn1D& in, int* status, cudaStream_t st);
 void launch_convert1d(const Dev1D& d, const Ptr9& src, const Ptr9& dst, int layout, int dir, cudaStream_t st);
 

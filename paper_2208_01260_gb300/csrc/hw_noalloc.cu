@@ -87,9 +87,7 @@ extern "C" int hw_rhs1d_noalloc(const hw_grid* grid, const hw_params* params, co
   d.bc = grid->bc_x;
   d.dx = dx;
   d.inv_dx = 1.0 / dx;
-  d.g = params->g;
-  d.eps_w = params->eps_w;
-  d.eps_lim = params->eps_lim;
+  hw::set_physics(d, params->g, params->eps_w, params->eps_lim);
   d.c_b = 0.5 / dx;
   d.c_g = 1.0 / (24.0 * dx);
   double* p = base;
@@ -118,10 +116,14 @@ extern "C" int hw_rhs1d_noalloc(const hw_grid* grid, const hw_params* params, co
   hw::launch_alpha1d(d, amax, status, st);
   hw::launch_finish_alpha1d(d, amax, alpha, nullptr, params->cfl, nullptr, -1.0, st);
   const bool lin = params->linear_weights != 0, chr = params->char_decomp != 0;
-  hw::launch_sweep1d(d, alpha, lin, chr, st);
   hw::StageArgs1D sa{};
   for (int q = 0; q < 4; ++q) sa.rhs_out[q] = out[q];
-  hw::launch_node1d(d, sa, hw::MODE_RHS, lin, chr, st);
+  if (lin) {
+    hw::launch_sweep1d(d, alpha, chr, st);
+    hw::launch_node1d(d, sa, hw::MODE_RHS, chr, st);
+  } else {
+    hw::launch_rhs1d(d, sa, alpha, chr, st);
+  }
   e = cudaGetLastError();
   if (e != cudaSuccess)
     return noalloc_fail(HW_ERR_CUDA, (std::string("hw_rhs1d_noalloc: launch failed: ") + cudaGetErrorString(e)).c_str());
