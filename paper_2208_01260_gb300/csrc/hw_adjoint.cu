@@ -706,66 +706,135 @@ struct AdjBuffers {
   int* argmax = nullptr;
   double* lstatic_phys[3] = {};
   unsigned long long* amax = nullptr;  // the forward alpha reduction's keys and scratch (kAlpha2dScratch)
+  // memory of one call (hw_gauge_loss, hw_adjoint_run), kept for the solver's next one up to kKeep bytes each
+  // and freed with the buffers above: allocating and freeing it cost as much as a small run's kernels
+  struct Work {
+    void* p = nullptr;
+    size_t bytes = 0;
+  };
+  std::vector<Work> work;
 };
+constexpr size_t kKeep = (size_t)1 << 31;
+enum { W_SAVE = 0, W_GVALS, W_OBS, W_IDX, W_TAPE, W_SLOT };  // W_SLOT + k: snapshot k
 
 std::mutex g_adj_mu;
 std::vector<AdjBuffers*> g_adj;  // one per live solver that used the adjoint (released by hw_destroy)
 
-// Zeroed on the solver's stream: the static adjoints accumulate into their buffers from the first use on
-// (each use clears them when it is done), so they must start at zero, not at whatever the memory held.
-int adj_alloc(AdjBuffers* B, double** p, size_t cnt, cudaStream_t st) {
+// count planes of cnt doubles, one after the other (so that one memset clears them), zeroed on the solver's
+// stream: the static adjoints accumulate into their buffers from the first use on (each use clears them when it
+// is done), so they must start at zero, not at whatever the memory held.
+int adj_alloc(AdjBuffers* B, double** p, int count, size_t cnt, cudaStream_t st) {
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, cnt * sizeof(double));
+  cudaError_t e = cudaMalloc(&q, count * cnt * sizeof(double));
   if (e != cudaSuccess) return afail(HW_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   B->allocs.push_back(q);
-  *p = (double*)q;
-  e = cudaMemsetAsync(q, 0, cnt * sizeof(double), st);
+  for (int k = 0; k < count; ++k) p[k] = (double*)q + (size_t)k * cnt;
+  e = cudaMemsetAsync(q, 0, count * cnt * sizeof(double), st);
   if (e != cudaSuccess) return afail(HW_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
   return HW_OK;
 }
 
-int get_buffers(hw_solver* s, const hw::SolverView& v, AdjBuffers** out) {
+// The solver's entry, without its planes (created at the first use).
+AdjBuffers* find_entry(hw_solver* s, const hw::SolverView& v) {
   std::lock_guard<std::mutex> lk(g_adj_mu);
   for (AdjBuffers* B : g_adj)
-    if (B->owner == s) {
-      if (B->n != v.n || B->nx != v.d2->nx || B->ny != v.d2->ny)
-        return afail(HW_ERR_STATE, "adjoint: working buffers do not match the solver's grid");
-      *out = B;
-      return HW_OK;
-    }
+    if (B->owner == s) return B;
   AdjBuffers* B = new AdjBuffers();
   B->owner = s;
   B->n = v.n;
   B->nx = v.d2->nx;
   B->ny = v.d2->ny;
+  g_adj.push_back(B);
+  return B;
+}
+
+// At least `bytes` of the entry's memory number k, reused between calls (its contents are not). A call asks in
+// rising order of k; when memory is short, what an earlier call left above k is given back first.
+void* work_get(AdjBuffers* B, int k, size_t bytes) {
+  if (B->work.size() <= (size_t)k) B->work.resize(k + 1);
+  AdjBuffers::Work& w = B->work[k];
+  if (w.bytes >= bytes) return w.p;
+  cudaFree(w.p);
+  w = {};
+  cudaError_t e = cudaMalloc(&w.p, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    for (size_t l = k + 1; l < B->work.size(); ++l) {
+      cudaFree(B->work[l].p);
+      B->work[l] = {};
+    }
+    e = cudaMalloc(&w.p, bytes);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    w.p = nullptr;
+    return nullptr;
+  }
+  w.bytes = bytes;
+  return w.p;
+}
+
+// Gives back what a call needed beyond kKeep (its stream has drained).
+void work_trim(AdjBuffers* B) {
+  size_t held = 0;
+  for (AdjBuffers::Work& w : B->work) {
+    held += w.bytes;
+    if (w.p && held > kKeep) {
+      cudaFree(w.p);
+      held -= w.bytes;
+      w = {};
+    }
+  }
+}
+
+// Bytes held by the memories from number k on.
+size_t work_bytes(const AdjBuffers* B, size_t k) {
+  size_t held = 0;
+  for (; k < B->work.size(); ++k) held += B->work[k].bytes;
+  return held;
+}
+
+int get_buffers(hw_solver* s, const hw::SolverView& v, AdjBuffers** out) {
+  AdjBuffers* B = find_entry(s, v);
+  if (B->n != v.n || B->nx != v.d2->nx || B->ny != v.d2->ny)
+    return afail(HW_ERR_STATE, "adjoint: working buffers do not match the solver's grid");
+  *out = B;
+  if (!B->allocs.empty()) return HW_OK;
   const size_t n = v.n, nxi = (size_t)(B->nx + 1) * B->ny, nyi = (size_t)B->nx * (B->ny + 1);
   int rc = HW_OK;
-  auto A = [&](double** p, size_t c) { if (rc == HW_OK) rc = adj_alloc(B, p, c, v.stream); };
-  for (int k = 0; k < 3; ++k)
-    for (int q = 0; q < 9; ++q) A(&B->stage_in[k][q], n);
-  for (int q = 0; q < 9; ++q) { A(&B->stage_out[q], n); A(&B->lam[0][q], n); A(&B->lam[1][q], n); A(&B->lbase[q], n); A(&B->lR[q], n); }
-  A(&B->alpha_st, 8);
+  auto A = [&](double** p, int count, size_t c) { if (rc == HW_OK) rc = adj_alloc(B, p, count, c, v.stream); };
+  for (int k = 0; k < 3; ++k) A(B->stage_in[k], 9, n);
+  A(B->stage_out, 9, n);
+  A(B->lam[0], 9, n);
+  A(B->lam[1], 9, n);
+  A(B->lbase, 9, n);
+  A(B->lR, 9, n);
+  A(&B->alpha_st, 1, 8);
   for (int k = 0; k < 3; ++k) {
-    for (int c = 0; c < 3; ++c) { A(&B->dbx[k][c], nxi); A(&B->dby[k][c], nyi); }
-    A(&B->fx[k], nxi);
-    A(&B->fy[k], nyi);
+    A(B->dbx[k], 3, nxi);
+    A(B->dby[k], 3, nyi);
+    A(&B->fx[k], 1, nxi);
+    A(&B->fy[k], 1, nyi);
   }
-  for (int q = 0; q < 6; ++q) { A(&B->lmod[q], n); A(&B->lqbx[q], nxi); A(&B->lqby[q], nyi); }
-  for (int f = 0; f < hw::NREC; ++f) { A(&B->lrecx[f], (size_t)(B->nx + 4) * B->ny); A(&B->lrecy[f], (size_t)B->nx * (B->ny + 4)); }
-  for (int q = 0; q < 3; ++q) { A(&B->lstat[q], n); A(&B->lstatic_phys[q], n); }
-  for (int q = 0; q < 2; ++q) { A(&B->lsv[q], n); A(&B->lsq[q], n); }
+  A(B->lmod, 6, n);
+  A(B->lqbx, 6, nxi);
+  A(B->lqby, 6, nyi);
+  A(B->lrecx, hw::NREC, (size_t)(B->nx + 4) * B->ny);
+  A(B->lrecy, hw::NREC, (size_t)B->nx * (B->ny + 4));
+  A(B->lstat, 3, n);
+  A(B->lstatic_phys, 3, n);
+  A(B->lsv, 2, n);
+  A(B->lsq, 2, n);
   double* misc = nullptr;
-  A(&misc, 8);
-  A(reinterpret_cast<double**>(&B->amax), hw::kAlpha2dScratch);
+  A(&misc, 1, 8);
+  A(reinterpret_cast<double**>(&B->amax), 1, hw::kAlpha2dScratch);
   if (rc != HW_OK) {
     for (void* p : B->allocs) cudaFree(p);
-    delete B;
+    B->allocs.clear();
     return rc;
   }
   B->lalpha = misc;
   B->argmax = (int*)(misc + 4);
-  g_adj.push_back(B);
-  *out = B;
   return HW_OK;
 }
 
@@ -776,6 +845,7 @@ void hw::adjoint_release(hw_solver* s) {
   for (size_t k = 0; k < g_adj.size(); ++k)
     if (g_adj[k]->owner == s) {
       for (void* p : g_adj[k]->allocs) cudaFree(p);
+      for (AdjBuffers::Work& w : g_adj[k]->work) cudaFree(w.p);
       delete g_adj[k];
       g_adj.erase(g_adj.begin() + k);
       return;
@@ -792,10 +862,19 @@ double misfit_loss(const double* g, const double* obs, size_t n) {
   return L;
 }
 
+// Clears the planes, those that follow one another in memory by one memset (a stage's reverse clears 36 record
+// planes: 2 launches instead of 36).
 int zero_planes(double* const* p, int count, size_t n, cudaStream_t st) {
-  for (int q = 0; q < count; ++q) ACUDA(cudaMemsetAsync(p[q], 0, n * sizeof(double), st));
+  for (int q = 0; q < count;) {
+    int m = 1;
+    while (q + m < count && p[q + m] == p[q] + (size_t)m * n) ++m;
+    ACUDA(cudaMemsetAsync(p[q], 0, (size_t)m * n * sizeof(double), st));
+    q += m;
+  }
   return HW_OK;
 }
+
+__global__ void k_set_dt(double* p, double v) { *p = v; }
 
 // What the reverse of one step reads: every stage's input, the step's output, the stage alphas, the
 // stages' source interface values 2 bhat and the first components of their fluxes 2 Fhat. Points into AdjBuffers (one step, recomputed from a
@@ -828,7 +907,7 @@ StepTape buffer_tape(AdjBuffers* B) {
 // into the tape); the solver's state is not touched.
 int forward_record(const hw::SolverView& v, AdjBuffers* B, const StepTape& T, double dt) {
   cudaStream_t st = v.stream;
-  ACUDA(cudaMemcpyAsync(v.dt, &dt, sizeof(double), cudaMemcpyHostToDevice, st));
+  k_set_dt<<<1, 1, 0, st>>>(v.dt, dt);
   hw::Dev2D d = *v.d2;
   const bool lin = false, chr = true;
   for (int k = 1; k <= 3; ++k) {
@@ -1146,20 +1225,18 @@ int hw_gauge_loss(hw_solver* s, int nsteps, const double* dts, const int* gauge_
   cudaStream_t st = v.stream;
   double *d_save = nullptr, *d_g = nullptr;
   int* d_idx = nullptr;
-  // every exit after the first allocation frees the working buffers
+  AdjBuffers* B = find_entry(s, v);
   auto check = [&](cudaError_t e, const char* what) {
     if (rc == HW_OK && e != cudaSuccess) rc = afail(HW_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
   };
-  auto alloc = [&](void** p, size_t bytes, const char* what) {
+  auto alloc = [&](void** p, int k, size_t bytes, const char* what) {
     if (rc != HW_OK) return;
-    if (cudaMalloc(p, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      rc = afail(HW_ERR_NOMEM, std::string("hw_gauge_loss: allocation failed: ") + what);
-    }
+    *p = work_get(B, k, bytes);
+    if (!*p) rc = afail(HW_ERR_NOMEM, std::string("hw_gauge_loss: allocation failed: ") + what);
   };
-  alloc((void**)&d_save, 9 * v.n * sizeof(double), "saved state");
-  alloc((void**)&d_g, (size_t)nsteps * ngauge * sizeof(double), "gauge values");
-  alloc((void**)&d_idx, ngauge * sizeof(int), "gauge indices");
+  alloc((void**)&d_save, W_SAVE, 9 * v.n * sizeof(double), "saved state");
+  alloc((void**)&d_g, W_GVALS, (size_t)nsteps * ngauge * sizeof(double), "gauge values");
+  alloc((void**)&d_idx, W_IDX, ngauge * sizeof(int), "gauge indices");
   if (rc == HW_OK) {
     check(cudaMemcpyAsync(d_idx, gauge_idx, ngauge * sizeof(int), cudaMemcpyHostToDevice, st), "cudaMemcpyAsync");
     for (int q = 0; q < 9; ++q)
@@ -1184,9 +1261,7 @@ int hw_gauge_loss(hw_solver* s, int nsteps, const double* dts, const int* gauge_
     rc = hw::solver_set_state_planes(s, src);
   }
   cudaStreamSynchronize(st);
-  cudaFree(d_save);
-  cudaFree(d_g);
-  cudaFree(d_idx);
+  work_trim(B);
   return rc;
 }
 
@@ -1216,7 +1291,7 @@ int hw_adjoint_run(hw_solver* s, int nsteps, const double* dts, const int* gauge
   if (snapshots == HW_ADJ_TAPE || snapshots == HW_ADJ_AUTO) {
     size_t free_b = 0, total_b = 0;
     ACUDA(cudaMemGetInfo(&free_b, &total_b));
-    const double budget = 0.9 * (double)free_b;
+    const double budget = 0.9 * ((double)free_b + (double)work_bytes(B, W_TAPE));  // what is kept is reused or given back
     if ((double)layout.bytes() <= budget) {
       use_tape = true;
     } else if (snapshots == HW_ADJ_TAPE) {
@@ -1237,26 +1312,20 @@ int hw_adjoint_run(hw_solver* s, int nsteps, const double* dts, const int* gauge
   double* tape = nullptr;
   auto cleanup = [&]() {
     cudaStreamSynchronize(st);
-    for (double* p : R.slots) if (p) cudaFree(p);
-    cudaFree(tape);
-    cudaFree(R.d_gvals);
-    cudaFree(d_obs);
-    cudaFree(d_idx);
+    work_trim(B);
     if (forward_steps_out) *forward_steps_out = R.fwd_steps;
   };
-  auto alloc = [&](void** p, size_t bytes, const char* what) {
+  auto alloc = [&](void** p, int k, size_t bytes, const char* what) {
     if (rc != HW_OK) return;
-    if (cudaMalloc(p, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      rc = afail(HW_ERR_NOMEM, std::string("hw_adjoint_run: allocation failed: ") + what);
-    }
+    *p = work_get(B, k, bytes);
+    if (!*p) rc = afail(HW_ERR_NOMEM, std::string("hw_adjoint_run: allocation failed: ") + what);
   };
-  alloc((void**)&R.d_gvals, (size_t)nsteps * ngauge * sizeof(double), "gauge values");
-  alloc((void**)&d_obs, (size_t)nsteps * ngauge * sizeof(double), "observations");
-  alloc((void**)&d_idx, ngauge * sizeof(int), "gauge indices");
-  if (use_tape) alloc((void**)&tape, layout.bytes(), "tape");
+  alloc((void**)&R.d_gvals, W_GVALS, (size_t)nsteps * ngauge * sizeof(double), "gauge values");
+  alloc((void**)&d_obs, W_OBS, (size_t)nsteps * ngauge * sizeof(double), "observations");
+  alloc((void**)&d_idx, W_IDX, ngauge * sizeof(int), "gauge indices");
+  if (use_tape) alloc((void**)&tape, W_TAPE, layout.bytes(), "tape");
   R.slots.assign(use_tape ? 0 : S + 1, nullptr);
-  for (size_t k = 0; k < R.slots.size(); ++k) alloc((void**)&R.slots[k], 9 * v.n * sizeof(double), "snapshot");
+  for (size_t k = 0; k < R.slots.size(); ++k) alloc((void**)&R.slots[k], W_SLOT + (int)k, 9 * v.n * sizeof(double), "snapshot");
   R.d_obs = d_obs;
   R.d_idx = d_idx;
   auto check = [&](cudaError_t e, const char* what) {
