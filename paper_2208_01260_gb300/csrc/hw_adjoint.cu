@@ -909,17 +909,13 @@ int forward_record(const hw::SolverView& v, AdjBuffers* B, const StepTape& T, do
   cudaStream_t st = v.stream;
   k_set_dt<<<1, 1, 0, st>>>(v.dt, dt);
   hw::Dev2D d = *v.d2;
-  const bool lin = false, chr = true;
   for (int k = 1; k <= 3; ++k) {
     for (int q = 0; q < 9; ++q) d.S[q] = T.in[k - 1][q];
     for (int c = 0; c < 3; ++c) { d.X[3 + c] = T.dbx[k - 1][c]; d.Y[3 + c] = T.dby[k - 1][c]; }
     d.X[0] = T.fx[k - 1];
     d.Y[0] = T.fy[k - 1];
-    hw::launch_alpha2d(d, B->amax, (int*)(B->lalpha + 2), st);
-    hw::launch_finish_alpha2d(d, B->amax, T.alpha + 2 * (k - 1), nullptr, v.params->cfl,
-                              nullptr, -1.0, st);
-    hw::launch_sweep_x2d(d, T.alpha + 2 * (k - 1), lin, chr, st);
-    hw::launch_sweep_y2d(d, T.alpha + 2 * (k - 1), lin, chr, st);
+    hw::launch_alpha_finish2d(d, B->amax, (int*)(B->lalpha + 2),
+                              hw::AlphaOut{T.alpha + 2 * (k - 1), v.dt, 0, 0.0, 0.0, 0.0, nullptr, -1.0, nullptr}, st);
     hw::StageArgs sa{};
     sa.k = k;
     sa.limiter = v.params->limiter;
@@ -928,7 +924,7 @@ int forward_record(const hw::SolverView& v, AdjBuffers* B, const StepTape& T, do
       sa.out[q] = k < 3 ? T.in[k][q] : T.out[q];
       sa.base[q] = v.base[q];
     }
-    hw::launch_node2d(d, sa, hw::MODE_STAGE, lin, chr, st);
+    hw::launch_stage_fp64(d, sa, T.alpha + 2 * (k - 1), st);
   }
   ACUDA(cudaGetLastError());
   return HW_OK;
@@ -1143,7 +1139,16 @@ int save_slot(RunCtx& R, int slot) {
   return HW_OK;
 }
 
+// The solver's steps take the recording kernels (hw_forward64.cu) while this lives, so that a recomputed state is
+// the recorded one.
+struct RecordingSteps {
+  hw_solver* s;
+  explicit RecordingSteps(hw_solver* s_) : s(s_) { hw::solver_fp64_stages(s, true); }
+  ~RecordingSteps() { hw::solver_fp64_stages(s, false); }
+};
+
 int advance(RunCtx& R, int from, int steps) {
+  RecordingSteps scope(R.s);
   for (int j = 0; j < steps; ++j) {
     int rc = hw_rk3_step(R.s, R.dts[from + j]);
     if (rc) return rc;
@@ -1243,6 +1248,7 @@ int hw_gauge_loss(hw_solver* s, int nsteps, const double* dts, const int* gauge_
       check(cudaMemcpyAsync(d_save + (size_t)q * v.n, v.state[q], v.n * sizeof(double), cudaMemcpyDeviceToDevice, st),
             "cudaMemcpyAsync");
   }
+  RecordingSteps scope(s);
   for (int j = 0; j < nsteps && rc == HW_OK; ++j) {
     rc = hw_rk3_step(s, dts[j]);
     hw::solver_view(s, &v);
@@ -1352,9 +1358,7 @@ int hw_adjoint_run(hw_solver* s, int nsteps, const double* dts, const int* gauge
   } else if (rc == HW_OK) {
     rc = save_slot(R, 0);
     for (int j = 0; j < nsteps && rc == HW_OK; ++j) {
-      rc = hw_rk3_step(s, dts[j]);
-      hw::solver_view(s, &R.v);
-      ++R.fwd_steps;
+      rc = advance(R, j, 1);
       hw::k_gather_eta<<<(ngauge + 127) / 128, 128, 0, st>>>(R.v.state[0], d_idx, ngauge,
                                                              R.d_gvals + (size_t)j * ngauge);
     }
@@ -1548,8 +1552,6 @@ int dd_adjoint_impl(hw_dd* dd, int nsteps, const double* dts, const int* gauge_i
         const cudaStream_t bs = bl[p].v.stream;
         hw::launch_finish_alpha2d(d, keys + 2 * np, T.alpha + 2 * (k - 1), nullptr, bl[p].v.params->cfl, nullptr, -1.0,
                                   bs);
-        hw::launch_sweep_x2d(d, T.alpha + 2 * (k - 1), false, true, bs);
-        hw::launch_sweep_y2d(d, T.alpha + 2 * (k - 1), false, true, bs);
         hw::StageArgs sa{};
         sa.k = k;
         sa.limiter = bl[p].v.params->limiter;
@@ -1558,7 +1560,7 @@ int dd_adjoint_impl(hw_dd* dd, int nsteps, const double* dts, const int* gauge_i
           sa.out[q] = k < 3 ? T.in[k][q] : T.out[q];
           sa.base[q] = bl[p].v.base[q];
         }
-        hw::launch_node2d(d, sa, hw::MODE_STAGE, false, true, bs);
+        hw::launch_stage_fp64(d, sa, T.alpha + 2 * (k - 1), bs);
       }
       if ((rc = hw::dd_join_blocks(dd, st))) break;
     }
@@ -1851,8 +1853,6 @@ int hw_part_adj_forward_stage(hw_part_adj* a, int j, int k, double dt, const uns
   d.X[0] = T.fx[k - 1];
   d.Y[0] = T.fy[k - 1];
   hw::launch_finish_alpha2d(d, keys, T.alpha + 2 * (k - 1), nullptr, v.params->cfl, nullptr, -1.0, st);
-  hw::launch_sweep_x2d(d, T.alpha + 2 * (k - 1), false, true, st);
-  hw::launch_sweep_y2d(d, T.alpha + 2 * (k - 1), false, true, st);
   hw::StageArgs sa{};
   sa.k = k;
   sa.limiter = v.params->limiter;
@@ -1861,7 +1861,7 @@ int hw_part_adj_forward_stage(hw_part_adj* a, int j, int k, double dt, const uns
     sa.out[q] = k < 3 ? T.in[k][q] : T.out[q];
     sa.base[q] = v.base[q];
   }
-  hw::launch_node2d(d, sa, hw::MODE_STAGE, false, true, st);
+  hw::launch_stage_fp64(d, sa, T.alpha + 2 * (k - 1), st);
   if (k == 3 && a->nloc)
     hw::k_gather_eta_map<<<(a->nloc + 127) / 128, 128, 0, st>>>(T.out[0], a->d_map, a->d_map + a->nloc, a->nloc,
                                                               a->d_gvals + (size_t)j * a->ngauge);

@@ -93,6 +93,7 @@ struct hw_solver {
   // ring of 2 halo nodes, the spacing is the global grid's, and part_info places the block
   bool is_part = false;
   hw_part_info part_info{};
+  bool fp64_stages = false;  // the adjoint's forward pass (hw_forward64.cu)
   // profiling: event pairs recorded around launches, resolved in hw_get_profile
   bool profiling = false;
   std::vector<cudaEvent_t> ev_pool;
@@ -261,7 +262,7 @@ int hw_create(const hw_grid* grid, const hw_params* params, void* cuda_stream, h
   cudaError_t e = cudaStreamCreateWithFlags(&s->cap_stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) { s->cap_stream = nullptr; hw_destroy(s); return fail(HW_ERR_CUDA, cudaGetErrorString(e)); }
   e = cudaMemsetAsync(misc, 0, 16 * sizeof(double), s->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(s->amax + 2, 0, 4 * sizeof(unsigned long long), s->stream);  // 1D alpha slots
+  if (e == cudaSuccess) e = cudaMemsetAsync(s->amax, 0, hw::kAlpha2dScratch * sizeof(unsigned long long), s->stream);
   if (e != cudaSuccess) { hw_destroy(s); return fail(HW_ERR_CUDA, cudaGetErrorString(e)); }
   bind_state(s, s->SA);
   *out = s;
@@ -360,28 +361,39 @@ int hw_init(hw_solver* s, const double* h, const double* hu, const double* hv, c
 static void enqueue_alpha(hw_solver* s, bool with_dt, double t_end) {
   bind_state(s, s->state());
   timed(s, HW_PROF_ALPHA, [&] {
-    if (s->fp32) {
-      hw::launch_alpha2d(s->f2, s->amax, s->status, s->stream);
-      hw::launch_finish_alpha2d(s->d2, s->amax, s->alpha, with_dt ? s->dt : nullptr, s->params.cfl,
-                                with_dt ? s->t : nullptr, t_end, s->stream);
-    } else if (s->is2d()) {
-      hw::launch_alpha2d(s->d2, s->amax, s->status, s->stream);
-      hw::launch_finish_alpha2d(s->d2, s->amax, s->alpha, with_dt ? s->dt : nullptr, s->params.cfl,
-                                with_dt ? s->t : nullptr, t_end, s->stream);
+    if (s->is2d()) {
+      const hw::AlphaOut out{s->alpha, s->dt, with_dt ? 1 : 0, s->params.cfl, s->d2.inv_dx, s->d2.inv_dy,
+                             with_dt ? s->t : nullptr, t_end, s->fp32 ? s->fsc : nullptr};
+      if (s->fp32) hw::launch_alpha_finish2d(s->f2, s->amax, s->status, out, s->stream);
+      else hw::launch_alpha_finish2d(s->d2, s->amax, s->status, out, s->stream);
     } else {
       hw::launch_alpha_finish1d(s->d1, s->amax + 2, s->status, s->alpha, with_dt ? s->dt : nullptr, s->params.cfl,
                                 with_dt ? s->t : nullptr, t_end, s->stream);
     }
-  }, s->is2d() ? (s->fp32 ? 2 : 3) : 1);  // reduction (two passes in 2D double) and finish; one launch in 1D
+  }, s->is2d() && !s->fp32 && s->n > hw::kAlphaOneMax ? 2 : 1);  // two passes on large 2D double grids
 }
 
 // Whether the solver's stages are single launches that also form the next stage's alpha (hw_step1d.cu).
 static bool fused1d(const hw_solver* s) { return !s->is2d() && s->params.linear_weights == 0; }
 
+// The end of a step in stage 3's node update (2D): its time and the count of steps that advanced it.
+enum { CLOCK_NONE = 0, CLOCK_ADD = 1, CLOCK_SNAP = 2 };
+extern "C++" {
+template <class Args>
+static void set_clock(hw_solver* s, Args& sa, int clock) {
+  if (clock == CLOCK_NONE) return;
+  sa.nsteps = s->nsteps;
+  sa.t = s->t;
+  sa.clock = s->dt;
+  sa.snapped = clock == CLOCK_SNAP;
+}
+}
+
 // One stage: sweeps on the current state (alpha already in s->alpha), node kernel into the other
 // buffer, then swap. next (1D): the launch also forms the next stage's alpha and, after stage 3, the time and
-// the next step (clipped to t_end).
-static void enqueue_stage(hw_solver* s, int k, bool next = false, double t_end = -1.0) {
+// the next step (clipped to t_end). clock (2D, stage 3): the time after the step, t + dt or the one recorded
+// next to dt by the CFL step.
+static void enqueue_stage(hw_solver* s, int k, bool next = false, double t_end = -1.0, int clock = CLOCK_NONE) {
   static const char* kNames[4] = {"", "stage 1", "stage 2", "stage 3"};
   Range nvtx_range(kNames[k]);
   double** in = s->state();
@@ -390,19 +402,29 @@ static void enqueue_stage(hw_solver* s, int k, bool next = false, double t_end =
   const bool lin = s->params.linear_weights != 0, chr = s->params.char_decomp != 0;
   if (s->fp32) {
     float** fout = s->fother();
-    timed(s, HW_PROF_OTHER, [&] { hw::launch_scalars_to_float(s->alpha, s->dt, s->fsc, s->stream); });
     timed(s, HW_PROF_SWEEP_X, [&] { hw::launch_sweep_x2d(s->f2, s->fsc, lin, chr, s->stream); });
     timed(s, HW_PROF_SWEEP_Y, [&] { hw::launch_sweep_y2d(s->f2, s->fsc, lin, chr, s->stream); });
     hw::StageArgsT<float> sa{};
     sa.k = k; sa.limiter = s->params.limiter; sa.dt = s->fsc + 2;
     for (int q = 0; q < 9; ++q) { sa.out[q] = fout[q]; sa.base[q] = s->fbase[q]; }
+    set_clock(s, sa, clock);
     timed(s, HW_PROF_NODE, [&] { hw::launch_node2d(s->f2, sa, hw::MODE_STAGE, lin, chr, s->stream); });
   } else if (s->is2d()) {
-    timed(s, HW_PROF_SWEEP_X, [&] { hw::launch_sweep_x2d(s->d2, s->alpha, lin, chr, s->stream); });
-    timed(s, HW_PROF_SWEEP_Y, [&] { hw::launch_sweep_y2d(s->d2, s->alpha, lin, chr, s->stream); });
     hw::StageArgs sa{};
     sa.k = k; sa.limiter = s->params.limiter; sa.dt = s->dt;
     for (int q = 0; q < 9; ++q) { sa.out[q] = out[q]; sa.base[q] = s->base[q]; }
+    set_clock(s, sa, clock);
+    if (s->fp64_stages) {
+      timed(s, HW_PROF_NODE, [&] { hw::launch_stage_fp64(s->d2, sa, s->alpha, s->stream); });
+      s->cur ^= 1;
+      return;
+    }
+    if (s->profiling) {
+      timed(s, HW_PROF_SWEEP_X, [&] { hw::launch_sweep_x2d(s->d2, s->alpha, lin, chr, s->stream); });
+      timed(s, HW_PROF_SWEEP_Y, [&] { hw::launch_sweep_y2d(s->d2, s->alpha, lin, chr, s->stream); });
+    } else {
+      hw::launch_sweeps2d(s->d2, s->alpha, lin, chr, s->stream);
+    }
     timed(s, HW_PROF_NODE, [&] { hw::launch_node2d(s->d2, sa, hw::MODE_STAGE, lin, chr, s->stream); });
   } else {
     hw::StageArgs1D sa{};
@@ -441,9 +463,9 @@ int hw_rk3_step(hw_solver* s, double dt) {
   const bool fused = fused1d(s);
   for (int k = 1; k <= 3; ++k) {
     if (k == 1 || !fused) enqueue_alpha(s, false, -1.0);
-    enqueue_stage(s, k, fused && k < 3);
+    enqueue_stage(s, k, fused && k < 3, -1.0, k == 3 ? CLOCK_ADD : CLOCK_NONE);
   }
-  timed(s, HW_PROF_OTHER, [&] { k_add_time<<<1, 1, 0, s->stream>>>(s->t, s->dt, 0, s->nsteps); });
+  if (!s->is2d()) timed(s, HW_PROF_OTHER, [&] { k_add_time<<<1, 1, 0, s->stream>>>(s->t, s->dt, 0, s->nsteps); });
   CUDA_OK(cudaGetLastError());
   return HW_OK;
 }
@@ -459,9 +481,9 @@ static void enqueue_cfl_step(hw_solver* s, double t_end) {
   enqueue_stage(s, 1);
   for (int k = 2; k <= 3; ++k) {
     enqueue_alpha(s, false, -1.0);
-    enqueue_stage(s, k);
+    enqueue_stage(s, k, false, -1.0, k == 3 ? CLOCK_SNAP : CLOCK_NONE);
   }
-  timed(s, HW_PROF_OTHER, [&] { k_add_time<<<1, 1, 0, s->stream>>>(s->t, s->dt, 1, s->nsteps); });
+  if (!s->is2d()) timed(s, HW_PROF_OTHER, [&] { k_add_time<<<1, 1, 0, s->stream>>>(s->t, s->dt, 1, s->nsteps); });
 }
 
 int hw_advance(hw_solver* s, int nsteps, double t_end, int use_graph, double* t_out, int* steps_out) {
@@ -587,7 +609,6 @@ int hw_rhs(hw_solver* s, double* const* out, int ptr_kind) {
   if (s->fp32) {
     // float right-hand side into the spare state buffer, then widened into the output planes
     float** scratch = s->fother();
-    hw::launch_scalars_to_float(s->alpha, s->dt, s->fsc, s->stream);
     hw::launch_sweep_x2d(s->f2, s->fsc, lin, chr, s->stream);
     hw::launch_sweep_y2d(s->f2, s->fsc, lin, chr, s->stream);
     hw::StageArgsT<float> sa{};
@@ -598,8 +619,7 @@ int hw_rhs(hw_solver* s, double* const* out, int ptr_kind) {
     for (int q = 0; q < 9; ++q) { src[q] = scratch[q]; dd[q] = dst[q]; }
     cast_planes(s, src, dd, 9, 0, s->n);
   } else if (s->is2d()) {
-    hw::launch_sweep_x2d(s->d2, s->alpha, lin, chr, s->stream);
-    hw::launch_sweep_y2d(s->d2, s->alpha, lin, chr, s->stream);
+    hw::launch_sweeps2d(s->d2, s->alpha, lin, chr, s->stream);
     hw::StageArgs sa{};
     for (int q = 0; q < 9; ++q) sa.rhs_out[q] = dst[q];
     hw::launch_node2d(s->d2, sa, hw::MODE_RHS, lin, chr, s->stream);
@@ -713,6 +733,7 @@ cudaStream_t solver_swap_stream(hw_solver* s, cudaStream_t st) {
   return old;
 }
 int solver_cur(hw_solver* s) { return s->cur; }
+void solver_fp64_stages(hw_solver* s, bool on) { s->fp64_stages = on; }
 cudaStream_t solver_stream(hw_solver* s) { return s->stream; }
 const hw_part_info* part_info(hw_solver* s) { return s && s->is_part ? &s->part_info : nullptr; }
 
@@ -819,8 +840,7 @@ int hw_part_stage(hw_solver* s, int k, const unsigned long long* keys, double t_
   bind_state(s, s->state());
   hw::launch_finish_alpha2d(s->d2, keys, s->alpha, k == 1 ? s->dt : nullptr, s->params.cfl, k == 1 ? s->t : nullptr,
                             t_end, s->stream);
-  enqueue_stage(s, k);
-  if (k == 3) k_add_time<<<1, 1, 0, s->stream>>>(s->t, s->dt, 1, s->nsteps);
+  enqueue_stage(s, k, false, -1.0, k == 3 ? CLOCK_SNAP : CLOCK_NONE);
   CUDA_OK(cudaGetLastError());
   return HW_OK;
 }

@@ -56,6 +56,11 @@ struct StageArgsT {
   R* out[9];
   R* base[9];
   R* rhs_out[9];
+  // with nsteps (stage 3): the step's end, *t = clock[1] (snapped) or *t + clock[0], counted if clock[0] > 0
+  unsigned long long* nsteps;
+  double* t;
+  const double* clock;
+  int snapped;
 };
 using StageArgs = StageArgsT<double>;
 
@@ -103,8 +108,27 @@ int set_kernel_attributes2d();
 // reduction (its float maxima, then one slot per tile); the first three are cleared here. The float
 // variant's reduction uses the first three.
 constexpr int kAlpha2dTiles = 152 * 8;
-constexpr int kAlpha2dScratch = 3 + kAlpha2dTiles;
+constexpr int kAlpha2dSlots = 3 + kAlpha2dTiles;      // then the slots of launch_alpha_finish2d (zero between launches)
+constexpr int kAlpha2dScratch = kAlpha2dSlots + 4;
 void launch_alpha2d(const Dev2D& d, unsigned long long* amax, int* status, cudaStream_t st);
+// The reduction with its finish (the last block to end forms alpha; with_dt also the CFL step dt[0], clipped to end
+// at t_end > 0, and the time after it dt[1], from the time *t_now): amax as above, zero before the first launch.
+// fsc (single precision): receives alpha_x, alpha_y and dt rounded to float.
+struct AlphaOut {
+  double* alpha;
+  double* dt;
+  int with_dt;
+  double cfl, inv_dx, inv_dy;
+  const double* t_now;
+  double t_end;
+  float* fsc;
+};
+constexpr size_t kAlphaOneMax = (size_t)1 << 18;  // nodes up to which the double reduction is one launch
+void launch_alpha_finish2d(const Dev2D& d, unsigned long long* amax, int* status, const AlphaOut& out, cudaStream_t st);
+void launch_alpha_finish2d(const Dev2DT<float>& d, unsigned long long* amax, int* status, const AlphaOut& out,
+                           cudaStream_t st);
+// both sweeps (one launch while the grid is small)
+void launch_sweeps2d(const Dev2D& d, const double* alpha, bool linear, bool chr, cudaStream_t st);
 void launch_finish_alpha2d(const Dev2D& d, const unsigned long long* amax, double* alpha, double* dt_out,
                            double cfl, const double* t_now, double t_end, cudaStream_t st);
 void launch_sweep_x2d(const Dev2D& d, const double* alpha, bool linear, bool chr, cudaStream_t st);
@@ -115,14 +139,15 @@ void launch_init2d(const Dev2D& d, const PhysIn& in, int* status, cudaStream_t s
 void launch_static2d(const Dev2D& d, cudaStream_t st);
 void launch_convert2d(const Dev2D& d, const Ptr9& src, const Ptr9& dst, int layout, int dir, cudaStream_t st);
 // single-precision variant of the stage kernels, and plane casts between precisions
-void launch_alpha2d(const Dev2DT<float>& d, unsigned long long* amax, int* status, cudaStream_t st);
 void launch_sweep_x2d(const Dev2DT<float>& d, const float* alpha, bool linear, bool chr, cudaStream_t st);
 void launch_sweep_y2d(const Dev2DT<float>& d, const float* alpha, bool linear, bool chr, cudaStream_t st);
-// alpha[2] and dt of the double scalars, rounded into out[0..2] (once per stage of the float variant)
-void launch_scalars_to_float(const double* alpha, const double* dt, float* out, cudaStream_t st);
 void launch_node2d(const Dev2DT<float>& d, const StageArgsT<float>& sa, int mode, bool linear, bool chr,
                    cudaStream_t st);
 void launch_cast_planes(int nplanes, size_t n, const Ptr12& src, const Ptr12& dst, int to_float, cudaStream_t st);
+
+// One RK stage of the adjoint's forward pass (hw_forward64.cu): sweeps and node update in FP64.
+void launch_stage_fp64(const Dev2D& d, const StageArgs& sa, const double* alpha, cudaStream_t st);
+void solver_fp64_stages(hw_solver* s, bool on);  // this solver's stages (2D double, nonlinear, projected) take it
 
 // record an error message for hw_last_error (hw_api.cu); returns code
 int set_last_error(int code, const char* msg);

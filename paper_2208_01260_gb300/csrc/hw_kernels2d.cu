@@ -49,6 +49,15 @@ __global__ void __launch_bounds__(TILE_T, kYsBlocks) k_sweep_y(Dev2D d, const do
   sweep_y_tile<LINEAR, CHAR, true>(d, alpha[1], blockIdx.x * (TILE_T / YS_C - 3), YS_C, sm);
 }
 
+// Both sweeps in one launch, for grids whose tiles fill the GPU a few times at most: a sweep of few tiles lasts as
+// long as one tile's chain, and each sweep's last wave runs partly empty.
+template <bool CHAR>
+__global__ void __launch_bounds__(TILE_T, kYsBlocks) k_sweep_xy(Dev2D d, const double* __restrict__ alpha, int nxt) {
+  __shared__ double sm[NRECX * TILE_T];
+  if ((int)blockIdx.x < nxt) sweep_x_tile<false, CHAR, true>(d, alpha[0], blockIdx.x * (TILE_T - 3), sm);
+  else sweep_y_tile<false, CHAR, true>(d, alpha[1], (blockIdx.x - nxt) * (TILE_T / YS_C - 3), YS_C, sm);
+}
+
 // Single-precision y-sweep: bound by memory rather than arithmetic, it keeps the column march, whose
 // loads are 32 consecutive nodes of a row: each thread owns one column and marches down `seg`
 // interfaces with the last four node records in a private shared-memory ring (no block barrier and
@@ -89,10 +98,16 @@ __global__ void __launch_bounds__(YS_W, 32) k_sweep_y_col(Dev2DT<float> d, const
   }
 }
 
-template <int MODE, bool LINEAR, bool CHAR, class R>
-__global__ void __launch_bounds__(kNodeT, kNodeBlocks<R>) k_node2d(Dev2DT<R> d, StageArgsT<R> sa) {
+// T threads per block: 256, or 64 for grids that do not fill the GPU with those (their warps then spread over more
+// SMs, and need not spill).
+template <int MODE, bool LINEAR, bool CHAR, class R, int T = kNodeT>
+__global__ void __launch_bounds__(T, T == kNodeT ? kNodeBlocks<R> : 8) k_node2d(Dev2DT<R> d, StageArgsT<R> sa) {
   const int i = blockIdx.x * 32 + threadIdx.x;
-  const int j = blockIdx.y * (kNodeT / 32) + threadIdx.y;
+  const int j = blockIdx.y * (T / 32) + threadIdx.y;
+  if (MODE == MODE_STAGE && sa.nsteps && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
+    *sa.t = sa.snapped ? sa.clock[1] : *sa.t + sa.clock[0];
+    if (sa.clock[0] > 0.0) ++*sa.nsteps;
+  }
   if (i >= d.nx || j >= d.ny) return;
   node_update<MODE, LINEAR, CHAR, kFixed<R>>(d, sa, i, j);
 }
@@ -115,7 +130,7 @@ __device__ __forceinline__ void alpha_tile(size_t n, size_t& begin, size_t& end)
   end = min(n, begin + per);
 }
 
-__global__ void __launch_bounds__(256) k_alpha2d_coarse(Dev2D d, unsigned long long* amax, int* status) {
+__global__ void __launch_bounds__(256) k_alpha2d_coarse(Dev2D d, unsigned int* m32, uint2* tiles, int* status) {
   __shared__ float s_m[2][8];
   __shared__ int s_ex[8];
   size_t begin, end;
@@ -155,54 +170,157 @@ __global__ void __launch_bounds__(256) k_alpha2d_coarse(Dev2D d, unsigned long l
       my = fmaxf(my, s_m[1][k]);
       ex |= s_ex[k];
     }
-    // non-negative floats order as their bit patterns; both maxima share the third 64-bit slot
-    unsigned int* m32 = reinterpret_cast<unsigned int*>(amax + 2);
+    // non-negative floats order as their bit patterns
     atomicMax(m32, __float_as_uint(mx));
     atomicMax(m32 + 1, __float_as_uint(my));
     const unsigned f = ex ? kTileExact : 0u;
-    reinterpret_cast<uint2*>(amax + 3)[blockIdx.x] = make_uint2(__float_as_uint(mx) | f, __float_as_uint(my) | f);
+    tiles[blockIdx.x] = make_uint2(__float_as_uint(mx) | f, __float_as_uint(my) | f);
   }
   if (bad) atomicOr(status, bad);
 }
 
-// The nodes alpha_exact_range would evaluate, in the tiles whose coarse maxima reach the thresholds.
-__global__ void __launch_bounds__(256) k_alpha2d_exact(Dev2D d, unsigned long long* amax, int* status) {
-  const unsigned int* m32 = reinterpret_cast<const unsigned int*>(amax + 2);
+// alpha keys -> doubles; dt = cfl / (alpha_x/dx + alpha_y/dy), optionally clipped to t_end - t.
+__device__ __forceinline__ void finish_alpha(unsigned long long kx, unsigned long long ky, const AlphaOut& f) {
+  const double ax = __longlong_as_double((long long)kx), ay = __longlong_as_double((long long)ky);
+  f.alpha[0] = ax;
+  f.alpha[1] = ay;
+  if (f.with_dt) {
+    double dt = f.cfl / fma(ax, f.inv_dx, ay * f.inv_dy);
+    double t_next = f.t_now ? *f.t_now + dt : 0.0;
+    if (f.t_now && f.t_end > 0.0) {
+      // the step that reaches t_end (within a relative 1e-12) ends exactly on it
+      const double rem = f.t_end - *f.t_now;
+      if (dt >= rem - 1e-12 * f.t_end) {
+        dt = rem > 0.0 ? rem : 0.0;
+        t_next = rem > 0.0 ? f.t_end : *f.t_now;
+      }
+    }
+    f.dt[0] = dt;
+    if (f.t_now) f.dt[1] = t_next;
+  }
+  if (f.fsc) {
+    f.fsc[0] = (float)ax;
+    f.fsc[1] = (float)ay;
+    f.fsc[2] = (float)f.dt[0];
+  }
+}
+
+// The end of a block of a reduction into slots[0..1] (keys; slots[2] scratch, slots[3] the blocks done): called by
+// one thread once the block's maxima are in; the last block finishes and clears the slots. No block waits.
+__device__ __forceinline__ void alpha_block_done(unsigned long long* slots, const AlphaOut& f) {
+  __threadfence();
+  if (atomicAdd(slots + 3, 1ull) != (unsigned long long)gridDim.x - 1) return;
+  __threadfence();
+  finish_alpha(atomicMax(slots, 0ull), atomicMax(slots + 1, 0ull), f);
+  slots[0] = slots[1] = slots[2] = slots[3] = 0;
+}
+
+// The nodes alpha_exact_range would evaluate, in the tiles whose coarse maxima reach the thresholds. keys: the
+// maxima; FINISH: keys are the slots of alpha_block_done.
+template <bool FINISH>
+__global__ void __launch_bounds__(256) k_alpha2d_exact(Dev2D d, const unsigned int* m32, const uint2* tiles,
+                                                       unsigned long long* keys, int* status, AlphaOut f) {
   const float tx = __uint_as_float(m32[0]) * (1.0f - 1e-5f), ty = __uint_as_float(m32[1]) * (1.0f - 1e-5f);
-  const uint2 tile = reinterpret_cast<const uint2*>(amax + 3)[blockIdx.x];
-  if (!((tile.x | tile.y) & kTileExact) && __uint_as_float(tile.x) < tx && __uint_as_float(tile.y) < ty) return;
-  size_t begin, end;
-  alpha_tile((size_t)d.nx * d.ny, begin, end);
-  unsigned long long kx = 0, ky = 0;
-  int bad = 0;
-  for (size_t o0 = begin + threadIdx.x; o0 < end; o0 += kAlphaU * blockDim.x) {
-    float fx[kAlphaU], fy[kAlphaU];
-    bool exact[kAlphaU], neg[kAlphaU], in[kAlphaU];
+  const uint2 tile = tiles[blockIdx.x];
+  if (((tile.x | tile.y) & kTileExact) || !(__uint_as_float(tile.x) < tx && __uint_as_float(tile.y) < ty)) {
+    size_t begin, end;
+    alpha_tile((size_t)d.nx * d.ny, begin, end);
+    unsigned long long kx = 0, ky = 0;
+    int bad = 0;
+    for (size_t o0 = begin + threadIdx.x; o0 < end; o0 += kAlphaU * blockDim.x) {
+      float fx[kAlphaU], fy[kAlphaU];
+      bool exact[kAlphaU], neg[kAlphaU], in[kAlphaU];
 #pragma unroll
-    for (int u = 0; u < kAlphaU; ++u) {
-      in[u] = o0 + u * blockDim.x < end;
-      if (in[u]) alpha_coarse(d, o0 + u * blockDim.x, fx[u], fy[u], exact[u], neg[u]);
+      for (int u = 0; u < kAlphaU; ++u) {
+        in[u] = o0 + u * blockDim.x < end;
+        if (in[u]) alpha_coarse(d, o0 + u * blockDim.x, fx[u], fy[u], exact[u], neg[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < kAlphaU; ++u)
+        if (in[u] && alpha_needs_exact(fx[u], fy[u], exact[u], neg[u], tx, ty))
+          alpha_exact_node(d, o0 + u * blockDim.x, kx, ky, bad);
     }
 #pragma unroll
-    for (int u = 0; u < kAlphaU; ++u)
-      if (in[u] && alpha_needs_exact(fx[u], fy[u], exact[u], neg[u], tx, ty))
-        alpha_exact_node(d, o0 + u * blockDim.x, kx, ky, bad);
+    for (int s = 16; s > 0; s >>= 1) {
+      kx = max(kx, __shfl_xor_sync(0xffffffffu, kx, s));
+      ky = max(ky, __shfl_xor_sync(0xffffffffu, ky, s));
+    }
+    if ((threadIdx.x & 31) == 0) {
+      if (kx) atomicMax(keys, kx);
+      if (ky) atomicMax(keys + 1, ky);
+      if (FINISH) __threadfence();
+    }
+    if (bad) atomicOr(status, bad);
+    if (FINISH) __syncthreads();
   }
+  if (FINISH && threadIdx.x == 0) alpha_block_done(keys, f);
+}
+
+// The whole reduction in one launch, for small grids (kAlphaOneMax): each block takes 256 U nodes, finds their float
+// maxima and evaluates in double its nodes near those (the grid's maximum is one block's, so it is among them).
+// Measured: 3.8 + 4.5 + 2.5 us and a memset in three launches at 64x66 become one of 4.3 us.
+template <int U>
+__global__ void __launch_bounds__(256) k_alpha2d_one(Dev2D d, unsigned long long* slots, int* status, AlphaOut f) {
+  __shared__ float s_m[2][8];
+  __shared__ unsigned long long s_k[2][8];
+  const size_t n = (size_t)d.nx * d.ny, o0 = (size_t)blockIdx.x * (256 * U) + threadIdx.x;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float fx[U], fy[U], mx = 0.0f, my = 0.0f;
+  bool exact[U], neg[U];
+  int bad = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    exact[u] = false;
+    neg[u] = true;  // past the end: skipped
+    fx[u] = fy[u] = 0.0f;
+    if (o0 + u * 256 < n) {
+      alpha_coarse(d, o0 + u * 256, fx[u], fy[u], exact[u], neg[u]);
+      if (neg[u] && !exact[u]) bad |= HW_STATUS_DEPTH;
+    }
+    if (!exact[u] && !neg[u]) {
+      mx = fmaxf(mx, fx[u]);
+      my = fmaxf(my, fy[u]);
+    }
+  }
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
+    my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, s));
+  }
+  if (lane == 0) { s_m[0][w] = mx; s_m[1][w] = my; }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    mx = fmaxf(mx, s_m[0][k]);
+    my = fmaxf(my, s_m[1][k]);
+  }
+  const float tx = mx * (1.0f - 1e-5f), ty = my * (1.0f - 1e-5f);
+  unsigned long long kx = 0, ky = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (o0 + u * 256 < n && alpha_needs_exact(fx[u], fy[u], exact[u], neg[u], tx, ty)) alpha_exact_node(d, o0 + u * 256, kx, ky, bad);
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) {
     kx = max(kx, __shfl_xor_sync(0xffffffffu, kx, s));
     ky = max(ky, __shfl_xor_sync(0xffffffffu, ky, s));
   }
-  if ((threadIdx.x & 31) == 0) {
-    if (kx) atomicMax(amax, kx);
-    if (ky) atomicMax(amax + 1, ky);
-  }
   if (bad) atomicOr(status, bad);
+  if (lane == 0) { s_k[0][w] = kx; s_k[1][w] = ky; }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int k = 1; k < 8; ++k) {
+    kx = max(kx, s_k[0][k]);
+    ky = max(ky, s_k[1][k]);
+  }
+  if (kx) atomicMax(slots, kx);
+  if (ky) atomicMax(slots + 1, ky);
+  alpha_block_done(slots, f);
 }
 
-// Single precision: the maximum in float, widened to a double key once per warp. Each thread keeps the
+// Single precision: the maximum in float, widened to a double key once per block. Each thread keeps the
 // loads of kAlphaU nodes in flight (the pass is bound by memory latency otherwise).
-__global__ void __launch_bounds__(256) k_alpha2d_f32(Dev2DT<float> d, unsigned long long* amax, int* status) {
+__global__ void __launch_bounds__(256) k_alpha2d_f32(Dev2DT<float> d, unsigned long long* slots, int* status, AlphaOut f) {
+  __shared__ float s_m[2][8];
   int bad = 0;
   const size_t n = (size_t)d.nx * d.ny, step = (size_t)gridDim.x * blockDim.x;
   float mx = 0.0f, my = 0.0f;
@@ -239,35 +357,21 @@ __global__ void __launch_bounds__(256) k_alpha2d_f32(Dev2DT<float> d, unsigned l
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
     my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, s));
   }
-  if ((threadIdx.x & 31) == 0) {
-    atomicMax(amax, dkey((double)mx));
-    atomicMax(amax + 1, dkey((double)my));
-  }
   if (bad) atomicOr(status, bad);
+  if ((threadIdx.x & 31) == 0) { s_m[0][threadIdx.x >> 5] = mx; s_m[1][threadIdx.x >> 5] = my; }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int k = 1; k < 8; ++k) {
+    mx = fmaxf(mx, s_m[0][k]);
+    my = fmaxf(my, s_m[1][k]);
+  }
+  atomicMax(slots, dkey((double)mx));
+  atomicMax(slots + 1, dkey((double)my));
+  alpha_block_done(slots, f);
 }
 
-// alpha keys -> doubles; dt = cfl / (alpha_x/dx + alpha_y/dy), optionally clipped to t_end - t.
-__global__ void k_finish_alpha2d(const unsigned long long* amax, double* alpha, double* dt_out, double cfl,
-                                 double inv_dx, double inv_dy, const double* t_now, double t_end) {
-  const double ax = __longlong_as_double((long long)amax[0]);
-  const double ay = __longlong_as_double((long long)amax[1]);
-  alpha[0] = ax;
-  alpha[1] = ay;
-  if (dt_out) {
-    double dt = cfl / fma(ax, inv_dx, ay * inv_dy);
-    double t_next = t_now ? *t_now + dt : 0.0;
-    if (t_now && t_end > 0.0) {
-      // the step that reaches t_end (within a relative 1e-12) ends exactly on it
-      const double rem = t_end - *t_now;
-      if (dt >= rem - 1e-12 * t_end) {
-        dt = rem > 0.0 ? rem : 0.0;
-        t_next = rem > 0.0 ? t_end : *t_now;
-      }
-    }
-    *dt_out = dt;
-    if (t_now) dt_out[1] = t_next;
-  }
-}
+// alpha and dt from keys that a launch of its own found (blocks of a decomposition).
+__global__ void k_finish_alpha2d(const unsigned long long* amax, AlphaOut f) { finish_alpha(amax[0], amax[1], f); }
 
 // ---------------------------------------------------------------------------------------------
 // Initialisation and conversion kernels
@@ -463,8 +567,17 @@ static void launch_sy(const Dev2DT<R>& d, const R* alpha, cudaStream_t st) {
   }
 }
 
+// Nodes up to which the node update runs in blocks of 64 threads: what those hold at once (16 warps per SM).
+constexpr size_t kNodeSmallMax = (size_t)152 * 16 * 32;
+
 template <int MODE, bool L, bool C, class R>
 static void launch_node(const Dev2DT<R>& d, const StageArgsT<R>& sa, cudaStream_t st) {
+  if constexpr (std::is_same<R, double>::value && !L) {
+    if ((size_t)d.nx * d.ny <= kNodeSmallMax) {
+      k_node2d<MODE, L, C, R, 64><<<dim3((d.nx + 31) / 32, (d.ny + 1) / 2), dim3(32, 2), 0, st>>>(d, sa);
+      return;
+    }
+  }
   constexpr int rows = kNodeT / 32;
   dim3 g((d.nx + 31) / 32, (d.ny + rows - 1) / rows);
   k_node2d<MODE, L, C, R><<<g, dim3(32, rows), 0, st>>>(d, sa);
@@ -472,23 +585,42 @@ static void launch_node(const Dev2DT<R>& d, const StageArgsT<R>& sa, cudaStream_
 
 int set_kernel_attributes2d() { return 0; }
 
+static int alpha_blocks(const Dev2D& d) {
+  return (int)std::min<size_t>(((size_t)d.nx * d.ny + 255) / 256, (size_t)kAlpha2dTiles);
+}
 void launch_alpha2d(const Dev2D& d, unsigned long long* amax, int* status, cudaStream_t st) {
   cudaMemsetAsync(amax, 0, 3 * sizeof(unsigned long long), st);
-  const size_t n = (size_t)d.nx * d.ny;
-  const int blocks = (int)std::min<size_t>((n + 255) / 256, (size_t)kAlpha2dTiles);  // tiles: amax[3 ..]
-  k_alpha2d_coarse<<<blocks, 256, 0, st>>>(d, amax, status);
-  k_alpha2d_exact<<<blocks, 256, 0, st>>>(d, amax, status);
+  unsigned int* m32 = reinterpret_cast<unsigned int*>(amax + 2);
+  uint2* tiles = reinterpret_cast<uint2*>(amax + 3);
+  const int blocks = alpha_blocks(d);
+  k_alpha2d_coarse<<<blocks, 256, 0, st>>>(d, m32, tiles, status);
+  k_alpha2d_exact<false><<<blocks, 256, 0, st>>>(d, m32, tiles, amax, status, AlphaOut{});
 }
-void launch_alpha2d(const Dev2DT<float>& d, unsigned long long* amax, int* status, cudaStream_t st) {
-  cudaMemsetAsync(amax, 0, 3 * sizeof(unsigned long long), st);
+void launch_alpha_finish2d(const Dev2D& d, unsigned long long* amax, int* status, const AlphaOut& out, cudaStream_t st) {
+  unsigned long long* slots = amax + kAlpha2dSlots;
   const size_t n = (size_t)d.nx * d.ny;
-  int blocks = (int)std::min<size_t>((n + 255) / 256, (size_t)152 * 8);
-  k_alpha2d_f32<<<blocks, 256, 0, st>>>(d, amax, status);
+  if (n <= (size_t)152 * 256) {
+    k_alpha2d_one<1><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(d, slots, status, out);
+  } else if (n <= kAlphaOneMax) {
+    k_alpha2d_one<4><<<(unsigned)((n + 1023) / 1024), 256, 0, st>>>(d, slots, status, out);
+  } else {
+    unsigned int* m32 = reinterpret_cast<unsigned int*>(slots + 2);
+    uint2* tiles = reinterpret_cast<uint2*>(amax + 3);
+    const int blocks = alpha_blocks(d);
+    k_alpha2d_coarse<<<blocks, 256, 0, st>>>(d, m32, tiles, status);
+    k_alpha2d_exact<true><<<blocks, 256, 0, st>>>(d, m32, tiles, slots, status, out);
+  }
+}
+void launch_alpha_finish2d(const Dev2DT<float>& d, unsigned long long* amax, int* status, const AlphaOut& out,
+                           cudaStream_t st) {
+  const size_t n = (size_t)d.nx * d.ny;
+  const int blocks = (int)std::min<size_t>((n + 255) / 256, (size_t)152 * 8);
+  k_alpha2d_f32<<<blocks, 256, 0, st>>>(d, amax + kAlpha2dSlots, status, out);
 }
 
 void launch_finish_alpha2d(const Dev2D& d, const unsigned long long* amax, double* alpha, double* dt_out,
                            double cfl, const double* t_now, double t_end, cudaStream_t st) {
-  k_finish_alpha2d<<<1, 1, 0, st>>>(amax, alpha, dt_out, cfl, d.inv_dx, d.inv_dy, t_now, t_end);
+  k_finish_alpha2d<<<1, 1, 0, st>>>(amax, AlphaOut{alpha, dt_out, dt_out != nullptr, cfl, d.inv_dx, d.inv_dy, t_now, t_end, nullptr});
 }
 
 template <class R>
@@ -518,6 +650,21 @@ void launch_sweep_x2d(const Dev2D& d, const double* alpha, bool linear, bool chr
 void launch_sweep_y2d(const Dev2D& d, const double* alpha, bool linear, bool chr, cudaStream_t st) {
   sweep_y_impl(d, alpha, linear, chr, st);
 }
+// Tiles of both sweeps up to which they share a launch.
+constexpr unsigned long long kSweepsOneMax = 152 * 4 * 8;
+
+void launch_sweeps2d(const Dev2D& d, const double* alpha, bool linear, bool chr, cudaStream_t st) {
+  constexpr int IX = TILE_T - 3, IY = TILE_T / YS_C - 3;
+  const unsigned long long nxt = ((unsigned long long)d.ny * (d.nx + 4) + IX - 1) / IX;
+  const unsigned long long nyt = ((unsigned long long)((d.nx + YS_C - 1) / YS_C) * (d.ny + 4) + IY - 1) / IY;
+  if (!linear && nxt + nyt <= kSweepsOneMax) {
+    if (chr) k_sweep_xy<true><<<(unsigned)(nxt + nyt), TILE_T, 0, st>>>(d, alpha, (int)nxt);
+    else k_sweep_xy<false><<<(unsigned)(nxt + nyt), TILE_T, 0, st>>>(d, alpha, (int)nxt);
+    return;
+  }
+  launch_sweep_x2d(d, alpha, linear, chr, st);
+  launch_sweep_y2d(d, alpha, linear, chr, st);
+}
 void launch_node2d(const Dev2D& d, const StageArgs& sa, int mode, bool linear, bool chr, cudaStream_t st) {
   node_impl(d, sa, mode, linear, chr, st);
 }
@@ -540,16 +687,6 @@ __global__ void k_cast_planes(int nplanes, size_t n, Ptr12 src, Ptr12 dst, int t
       if (to_float) ((float*)dst.p[q])[o] = (float)((const double*)src.p[q])[o];
       else ((double*)dst.p[q])[o] = (double)((const float*)src.p[q])[o];
     }
-}
-
-__global__ void k_scalars_to_float(const double* alpha, const double* dt, float* out) {
-  out[0] = (float)alpha[0];
-  out[1] = (float)alpha[1];
-  out[2] = (float)*dt;
-}
-
-void launch_scalars_to_float(const double* alpha, const double* dt, float* out, cudaStream_t st) {
-  k_scalars_to_float<<<1, 1, 0, st>>>(alpha, dt, out);
 }
 
 void launch_cast_planes(int nplanes, size_t n, const Ptr12& src, const Ptr12& dst, int to_float, cudaStream_t st) {
