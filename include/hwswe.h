@@ -194,7 +194,7 @@ int hw_batch_get_tiles(hw_batch* b, int i, int* yc);
  * the trial y-tile width yc, over reps repetitions. Changes no state (interface planes are scratch). */
 int hw_batch_time_tiles(hw_batch* b, int nids, const int* ids, int yc, int reps, double* ms_x, double* ms_y);
 /* Launch form of hw_batch_run (no counterpart in the paper). on = 0 (default): each phase of an RK stage
- * is one launch over all grids (12 launches and 3 small key resets per step). on = 1: each step is ONE
+ * is one launch over all grids (12 launches per step). on = 1: each step is ONE
  * cooperative launch of as many blocks as the device holds at once (two small resets before it); its
  * phases (the two alpha passes, the per-grid alpha and dt, both sweeps, the node update; three times) are
  * separated by grid-wide barriers, and sweep tiles and node items are taken from counters. Each barrier

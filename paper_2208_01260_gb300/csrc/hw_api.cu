@@ -727,6 +727,21 @@ int part_planes(hw_solver* s, int set, double** planes, int* nplanes) {
   return HW_OK;
 }
 const Dev2D* part_dev(hw_solver* s) { return &s->d2; }
+void part_block(hw_solver* s, PartBlock* b) {
+  for (int q = 0; q < 9; ++q) { b->S[0][q] = s->SA[q]; b->S[1][q] = s->SB[q]; }
+  b->b = s->d2.stat[0];
+  b->nx = s->part_info.nx;
+  b->ny = s->part_info.ny;
+  for (int f = 0; f < 4; ++f) { b->mode[f] = s->part_info.mode[f]; b->nbr[f] = s->part_info.nbr[f]; }
+  b->alpha = s->alpha;
+  b->dt = s->dt;
+  b->t = s->t;
+  b->status = s->status;
+}
+void part_stage(hw_solver* s, int k) {
+  bind_state(s, s->state());
+  enqueue_stage(s, k, false, -1.0, k == 3 ? CLOCK_SNAP : CLOCK_NONE);
+}
 cudaStream_t solver_swap_stream(hw_solver* s, cudaStream_t st) {
   cudaStream_t old = s->stream;
   s->stream = st;

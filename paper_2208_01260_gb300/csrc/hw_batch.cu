@@ -1,7 +1,7 @@
 // Batched form: many independent 2D grids of uneven sizes advance together, each with its own CFL
 // time step. All instances share pooled planes; every phase of an RK stage (alpha reduction, x-sweep,
 // y-sweep, node update) is ONE launch over a flattened list of work items of every instance (one block
-// per item; the alpha passes loop over theirs), so the launch count per step does not depend on the
+// per item; 12 launches a step), so the launch count per step does not depend on the
 // number of instances and small grids no longer leave the GPU idle. Two steps are captured in a CUDA
 // graph. The sweeps use the single-grid tiles over flattened extended lines (hw_stencil2d.cuh), so no
 // grid size leaves a ragged tile; the y-tile width is per instance, chosen by the autotuner. The
@@ -21,119 +21,79 @@ namespace hw {
 
 constexpr int BN_T = 128;  // nodes per node-kernel item
 
-// ---- alpha per instance in two passes, as the single-grid reduction (a float estimate of every node,
-// the double value only near the float maximum): items (inst, first node, count) ----
-__global__ void __launch_bounds__(256) k_balpha_coarse(BatchDev B, const int4* __restrict__ items, int nitems) {
-  for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
-    const int4 it = items[w];
-    const BInst& I = B.inst[it.x];
-    Dev2D d;
-    make_dev(B, I, d);
-    float mx = 0.0f, my = 0.0f;
-    int bad = 0;
-    const size_t base = (size_t)I.off_n;
-    for (int o = it.y + threadIdx.x; o < it.y + it.z; o += blockDim.x) {
-      float ax, ay;
-      bool exact, neg;
-      alpha_coarse(d, base + o, ax, ay, exact, neg);
-      if (exact) continue;
-      if (neg) { bad |= HW_STATUS_DEPTH; continue; }
-      mx = fmaxf(mx, ax);
-      my = fmaxf(my, ay);
-    }
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) {
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
-      my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, s));
-    }
-    unsigned int* m32 = reinterpret_cast<unsigned int*>(B.amax + 3 * it.x + 2);
-    if ((threadIdx.x & 31) == 0) {
-      atomicMax(m32, __float_as_uint(mx));
-      atomicMax(m32 + 1, __float_as_uint(my));
-    }
-    if (bad) atomicOr(B.status, bad);
-  }
-}
+constexpr int BA_N = 1024;  // nodes per alpha item
 
-__global__ void __launch_bounds__(256) k_balpha_exact(BatchDev B, const int4* __restrict__ items, int nitems) {
-  for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
-    const int4 it = items[w];
-    const BInst& I = B.inst[it.x];
-    Dev2D d;
-    make_dev(B, I, d);
-    const unsigned int* m32 = reinterpret_cast<const unsigned int*>(B.amax + 3 * it.x + 2);
-    unsigned long long kx = 0, ky = 0;
-    int bad = 0;
-    const size_t base = (size_t)I.off_n;
-    alpha_exact_range(d, m32, base + it.y + threadIdx.x, base + it.y + it.z, blockDim.x, kx, ky, bad);
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) {
-      kx = max(kx, __shfl_xor_sync(0xffffffffu, kx, s));
-      ky = max(ky, __shfl_xor_sync(0xffffffffu, ky, s));
-    }
-    if ((threadIdx.x & 31) == 0) {
-      if (kx) atomicMax(B.amax + 3 * it.x, kx);
-      if (ky) atomicMax(B.amax + 3 * it.x + 1, ky);
-    }
-    if (bad) atomicOr(B.status, bad);
-  }
-}
-
-// ---- per instance: alpha from the keys; at a step's start dt = cfl / (ax/dx + ay/dy) ----
-__global__ void k_bfinish(BatchDev B, int n, int with_dt) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double ax = __longlong_as_double((long long)B.amax[3 * i]);
-  const double ay = __longlong_as_double((long long)B.amax[3 * i + 1]);
-  B.alpha[2 * i] = ax;
-  B.alpha[2 * i + 1] = ay;
-  if (with_dt) {
-    const BInst& I = B.inst[i];
+// ---- alpha per instance: items (inst, first node) of BA_N nodes. The last item of an instance to end forms the
+// instance's alpha; at a step's start (k = 1) also dt = cfl / (ax/dx + ay/dy), before its last stage (k = 3) the time
+// after the step. B.done counts the items that ended; keys and counts are zero between launches.
+// Bound by latency: 19.7 us a launch on 24 grids of 911,000 nodes in all (it was a memset, a float pass, a double pass
+// and a finishing kernel). ----
+__global__ void __launch_bounds__(256) k_balpha(const __grid_constant__ BatchDev B, const int4* __restrict__ items) {
+  const int4 it = items[blockIdx.x];
+  const BInst& I = B.inst[it.x];
+  Dev2D d;
+  make_dev(B, I, d);
+  const size_t base = (size_t)I.off_n;
+  const int n = I.nx * I.ny;
+  unsigned long long kx, ky;
+  alpha_block_keys<BA_N / 256>(d, (size_t)it.y + threadIdx.x, (size_t)n, [base](size_t o) { return base + o; }, kx, ky,
+                               B.status);
+  if (threadIdx.x != 0) return;
+  unsigned long long* const key = B.amax + 3 * it.x;
+  if (kx) atomicMax(key, kx);
+  if (ky) atomicMax(key + 1, ky);
+  __threadfence();
+  if (atomicAdd(B.done + it.x, 1u) != (unsigned)((n + BA_N - 1) / BA_N) - 1) return;
+  __threadfence();
+  const double ax = __longlong_as_double((long long)atomicMax(key, 0ull));
+  const double ay = __longlong_as_double((long long)atomicMax(key + 1, 0ull));
+  B.alpha[2 * it.x] = ax;
+  B.alpha[2 * it.x + 1] = ay;
+  if (B.k == 1) {
     const double dt = B.cfl / fma(ax, I.inv_dx, ay * I.inv_dy);
-    B.dt[2 * i] = dt;
-    B.dt[2 * i + 1] = B.t[i] + dt;
+    B.dt[2 * it.x] = dt;
+    B.dt[2 * it.x + 1] = B.t[it.x] + dt;
+  } else if (B.k == 3) {
+    B.t[it.x] = B.dt[2 * it.x + 1];
+    if (B.dt[2 * it.x] > 0.0) ++B.nsteps[it.x];
   }
-}
-
-__global__ void k_btime(BatchDev B, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  B.t[i] = B.dt[2 * i + 1];
-  if (B.dt[2 * i] > 0.0) ++B.nsteps[i];
+  key[0] = key[1] = 0;
+  B.done[it.x] = 0;
 }
 
 // ---- x-sweep: items (inst, first extended node of the tile) over the flattened extended rows ----
 template <bool LINEAR, bool CHAR>
-__global__ void __launch_bounds__(TILE_T, 5) k_bsweep_x(BatchDev B, const int4* __restrict__ items, int nitems) {
+__global__ void __launch_bounds__(TILE_T, 5) k_bsweep_x(const __grid_constant__ BatchDev B, const int4* __restrict__ items, int nitems) {
   __shared__ double sm[NRECX * TILE_T];
   {
     const int4 it = items[blockIdx.x];
     const BInst& I = B.inst[it.x];
     Dev2D d;
     make_dev(B, I, d);
-    sweep_x_tile<LINEAR, CHAR, true>(d, B.alpha[2 * it.x], (unsigned)it.y, sm, (size_t)I.off_n, (size_t)I.off_x);
+    sweep_x_tile<LINEAR, CHAR, true>(d, BatchSource{&B, it.x, false}, B.alpha[2 * it.x], (unsigned)it.y, sm, (size_t)I.off_n, (size_t)I.off_x);
   }
 }
 
 // ---- y-sweep: items (inst, first extended row of the tile) over the flattened column groups ----
 template <bool LINEAR, bool CHAR>
-__global__ void __launch_bounds__(TILE_T, 4) k_bsweep_y(BatchDev B, const int4* __restrict__ items, int nitems) {
+__global__ void __launch_bounds__(TILE_T, 4) k_bsweep_y(const __grid_constant__ BatchDev B, const int4* __restrict__ items, int nitems) {
   __shared__ double sm[NRECX * TILE_T];
   {
     const int4 it = items[blockIdx.x];
     const BInst& I = B.inst[it.x];
     Dev2D d;
     make_dev(B, I, d);
-    sweep_y_tile<LINEAR, CHAR, true>(d, B.alpha[2 * it.x + 1], (unsigned)it.y, I.yc, sm, (size_t)I.off_n,
+    sweep_y_tile<LINEAR, CHAR, true>(d, BatchSource{&B, it.x, false}, B.alpha[2 * it.x + 1], (unsigned)it.y, I.yc, sm, (size_t)I.off_n,
                                      (size_t)I.off_y);
   }
 }
 
 // ---- node update: items (inst, first node) of BN_T consecutive nodes of one grid ----
 // The instance's grid constants come from global memory and take registers that the single-grid kernel keeps
-// in its parameters: 128 registers per thread (16 warps per SM).
+// in its parameters. Two steps of 24 grids of 911,000 nodes, all told, by threads x blocks per SM: 128x4 5115 us, 128x5
+// 5101, 128x6 5062, 256x3 5044, 256x2 5246, 64x8 5196; 128 rather than 256 for less of a small grid's last item.
 template <bool LINEAR, bool CHAR>
-__global__ void __launch_bounds__(BN_T, 4) k_bnode(BatchDev B, const int4* __restrict__ items, int nitems) {
+__global__ void __launch_bounds__(BN_T, 6) k_bnode(const __grid_constant__ BatchDev B, const int4* __restrict__ items, int nitems) {
   {
     const int4 it = items[blockIdx.x];
     const BInst& I = B.inst[it.x];
@@ -152,7 +112,7 @@ __global__ void __launch_bounds__(BN_T, 4) k_bnode(BatchDev B, const int4* __res
       sa.base[q] = B.base[q];
       sa.rhs_out[q] = nullptr;
     }
-    node_update<MODE_STAGE, LINEAR, CHAR, true>(d, sa, i, j, (size_t)I.off_n, (size_t)I.off_x, (size_t)I.off_y);
+    node_update<MODE_STAGE, LINEAR, CHAR, true>(d, BatchSource{&B, it.x, false}, sa, i, j, (size_t)I.off_n, (size_t)I.off_x, (size_t)I.off_y);
   }
 }
 
@@ -192,7 +152,6 @@ struct hw_batch {
   bool persistent = false;
   int bstep_blocks = 0;
   hw::StepSync* d_sync = nullptr;
-  int nb[1] = {1};  // blocks of the alpha passes (resident blocks on the device; they loop over items)
   std::vector<bool> inited;
   bool dirty = false;  // tile shapes changed since the work lists were built
   cudaGraphExec_t graph = nullptr;
@@ -231,7 +190,7 @@ void build_items(const std::vector<hw::BInst>& inst, const std::vector<int>& ids
   for (int i : ids) {
     const hw::BInst& I = inst[i];
     const int n = I.nx * I.ny;
-    for (int o = 0; o < n; o += 4096) out[0].push_back(make_int4(i, o, std::min(4096, n - o), 0));
+    for (int o = 0; o < n; o += hw::BA_N) out[0].push_back(make_int4(i, o, std::min(hw::BA_N, n - o), 0));
     const long long tx = (long long)I.ny * (I.nx + 4);
     for (long long e = 0; e < tx; e += hw::TILE_T - 3) out[1].push_back(make_int4(i, (int)e, 0, 0));
     const int ifs = hw::TILE_T / I.yc - 3;
@@ -254,26 +213,12 @@ int upload_items(hw_batch* b, std::vector<int4> lists[5], int4** dst, int* count
   return HW_OK;
 }
 
-int persistent_blocks(const void* fn, int threads, size_t smem) {
-  int dev = 0, sms = 1, bps = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, threads, smem) != cudaSuccess || bps < 1) bps = 1;
-  return sms * bps;
-}
-
 template <bool L, bool C>
 void launch_phases(hw_batch* b, int which, int4* const* items, const int* counts, cudaStream_t st) {
   // which: bit 0 x-sweep, bit 1 y-sweep, bit 2 node; one block per work item
   if ((which & 1) && counts[1]) hw::k_bsweep_x<L, C><<<counts[1], hw::TILE_T, 0, st>>>(b->B, items[1], counts[1]);
   if ((which & 2) && counts[2]) hw::k_bsweep_y<L, C><<<counts[2], hw::TILE_T, 0, st>>>(b->B, items[2], counts[2]);
   if ((which & 4) && counts[3]) hw::k_bnode<L, C><<<counts[3], hw::BN_T, 0, st>>>(b->B, items[3], counts[3]);
-}
-
-template <bool L, bool C>
-int prime_blocks(hw_batch* b) {
-  b->nb[0] = persistent_blocks((const void*)hw::k_balpha_exact, 256, 0);
-  return 0;
 }
 
 void enqueue_phases(hw_batch* b, int which, int4* const* items, const int* counts, cudaStream_t st) {
@@ -288,13 +233,13 @@ void bind(hw_batch* b) {
   for (int q = 0; q < 9; ++q) { b->B.S[q] = in[q]; b->B.out[q] = out[q]; }
 }
 
-void enqueue_alpha(hw_batch* b, int with_dt, cudaStream_t st) {
-  bind(b);
-  cudaMemsetAsync(b->B.amax, 0, 3 * sizeof(unsigned long long) * b->n, st);
-  const int na = std::min(b->nb[0], b->nitems[0]);
-  hw::k_balpha_coarse<<<na, 256, 0, st>>>(b->B, b->d_items[0], b->nitems[0]);
-  hw::k_balpha_exact<<<na, 256, 0, st>>>(b->B, b->d_items[0], b->nitems[0]);
-  hw::k_bfinish<<<(b->n + 127) / 128, 128, 0, st>>>(b->B, b->n, with_dt);
+void enqueue_alpha(hw_batch* b, cudaStream_t st) {
+  hw::k_balpha<<<b->nitems[0], 256, 0, st>>>(b->B, b->d_items[0]);
+}
+
+// k_balpha expects zero keys; a persistent step that was cut short leaves some.
+cudaError_t clear_keys(hw_batch* b) {
+  return cudaMemset(b->B.amax, 0, 3 * sizeof(unsigned long long) * b->n);
 }
 
 // The persistent step: the keys and the barrier counters start at zero, then one cooperative launch.
@@ -327,13 +272,12 @@ void enqueue_step(hw_batch* b, cudaStream_t st) {
     return;
   }
   for (int k = 1; k <= 3; ++k) {
-    enqueue_alpha(b, k == 1, st);
     b->B.k = k;
     bind(b);
+    enqueue_alpha(b, st);
     enqueue_phases(b, 7, b->d_items, b->nitems, st);
     b->cur ^= 1;
   }
-  hw::k_btime<<<(b->n + 127) / 128, 128, 0, st>>>(b->B, b->n);
 }
 
 int rebuild(hw_batch* b) {
@@ -396,7 +340,7 @@ int hw_batch_create(int n, const hw_grid* grids, const hw_params* params, void* 
   for (int q = 0; q < 2; ++q) { A(&b->B.sv[q], b->tot_n); A(&b->B.sq[q], b->tot_n); }
   for (int q = 0; q < 12; ++q) A(&b->staging[q], b->max_n);
   double* misc = nullptr;
-  A(&misc, (size_t)9 * n + 8);
+  A(&misc, (size_t)10 * n + 8);
   if (rc == HW_OK) rc = balloc(b, (void**)&b->d_inst, sizeof(hw::BInst) * n);
   if (rc == HW_OK) rc = balloc(b, (void**)&b->d_sync, sizeof(hw::StepSync));
   if (rc != HW_OK) { hw_batch_destroy(b); return rc; }
@@ -405,21 +349,16 @@ int hw_batch_create(int n, const hw_grid* grids, const hw_params* params, void* 
   b->B.dt = misc + 5 * n;
   b->B.t = misc + 7 * n;
   b->B.nsteps = (unsigned long long*)(misc + 8 * n);
-  b->B.status = (int*)(misc + 9 * n);
+  b->B.done = (unsigned int*)(misc + 9 * n);
+  b->B.status = (int*)(misc + 10 * n);
   hw::set_physics(b->B, params->g, params->eps_w, params->eps_lim);
   b->B.cfl = params->cfl;
   b->B.limiter = params->limiter;
   b->B.inst = b->d_inst;
   cudaError_t e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) { b->cap_stream = nullptr; hw_batch_destroy(b); return bfail(HW_ERR_CUDA, cudaGetErrorString(e)); }
-  e = cudaMemsetAsync(misc, 0, ((size_t)9 * n + 8) * sizeof(double), b->stream);
+  e = cudaMemsetAsync(misc, 0, ((size_t)10 * n + 8) * sizeof(double), b->stream);
   if (e != cudaSuccess) { hw_batch_destroy(b); return bfail(HW_ERR_CUDA, cudaGetErrorString(e)); }
-  {
-    const bool lin = params->linear_weights != 0, chr = params->char_decomp != 0;
-    const int pr = lin ? (chr ? prime_blocks<true, true>(b) : prime_blocks<true, false>(b))
-                       : (chr ? prime_blocks<false, true>(b) : prime_blocks<false, false>(b));
-    if (pr != 0) { hw_batch_destroy(b); return bfail(HW_ERR_CUDA, "hw_batch_create: kernel attributes"); }
-  }
   rc = rebuild(b);
   if (rc != HW_OK) { hw_batch_destroy(b); return rc; }
   *out = b;
@@ -511,8 +450,10 @@ int hw_batch_run(hw_batch* b, int nsteps, int use_graph) {
   BCUDA(cudaMemcpy(&st, b->B.status, sizeof(int), cudaMemcpyDeviceToHost));
   if (st) {
     BCUDA(cudaMemset(b->B.status, 0, sizeof(int)));
-    if (st & hw::HW_STATUS_TIMEOUT)
+    if (st & hw::HW_STATUS_TIMEOUT) {
+      BCUDA(clear_keys(b));
       return bfail(HW_ERR_TIMEOUT, "hw_batch_run: a grid barrier of the persistent step timed out");
+    }
     return bfail(HW_ERR_DEPTH, "hw_batch_run: non-positive or non-finite depth in some instance");
   }
   return HW_OK;
@@ -551,6 +492,7 @@ int hw_batch_test_barrier_timeout(hw_batch* b) {
   int st = 0;
   BCUDA(cudaMemcpy(&st, b->B.status, sizeof(int), cudaMemcpyDeviceToHost));
   BCUDA(cudaMemset(b->B.status, 0, sizeof(int)));
+  BCUDA(clear_keys(b));
   if (st & hw::HW_STATUS_TIMEOUT) return bfail(HW_ERR_TIMEOUT, "hw_batch_test_barrier_timeout: the barrier wait ran out");
   return HW_OK;
 }

@@ -29,6 +29,7 @@ struct BatchDev {
   double* out[9];
   double* base[9];
   unsigned long long* amax;  // 3 per instance: alpha_x, alpha_y keys, the coarse pass's float maxima
+  unsigned int* done;        // 1 per instance: alpha items that ended (k_balpha)
   double* alpha;             // 2 per instance
   double* dt;                // 2 per instance: step, time after the step
   double* t;                 // 1 per instance
@@ -58,6 +59,27 @@ __device__ __forceinline__ void make_dev(const BatchDev& B, const BInst& I, Dev2
 #pragma unroll
   for (int q = 0; q < 2; ++q) { d.sv[q] = B.sv[q]; d.sq[q] = B.sq[q]; }
 }
+
+// The instance view of stage input planes: B.S (sel = false) or B.out (sel = true).
+__device__ __forceinline__ void make_dev_in(const BatchDev& B, const BInst& I, bool sel, Dev2D& d) {
+  make_dev(B, I, d);
+  if (sel) {
+#pragma unroll
+    for (int q = 0; q < 9; ++q) d.S[q] = B.out[q];
+  }
+}
+
+// The instance's block for a call out of line (GridSource): B is the kernel's parameter.
+struct BatchSource {
+  const BatchDev* B;
+  int inst;
+  bool sel;
+  __device__ __forceinline__ Dev2D dev() const {
+    Dev2D d;
+    make_dev_in(*B, B->inst[inst], sel, d);
+    return d;
+  }
+};
 
 // Barrier and work counters of one persistent step launch (zeroed before the launch).
 struct StepSync {

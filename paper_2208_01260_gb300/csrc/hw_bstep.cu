@@ -72,15 +72,6 @@ __device__ __forceinline__ bool grid_barrier(const StepItems& P, unsigned int& p
   return *s_flag != 0;
 }
 
-// The instance view of stage input planes: B.S (sel = false) or B.out (sel = true).
-__device__ __forceinline__ void make_dev_in(const BatchDev& B, const BInst& I, bool sel, Dev2D& d) {
-  make_dev(B, I, d);
-  if (sel) {
-#pragma unroll
-    for (int q = 0; q < 9; ++q) d.S[q] = B.out[q];
-  }
-}
-
 // Shared memory of a block: two sweep tiles (consecutive tiles alternate, so one barrier per tile
 // suffices) and the block-uniform values the phases pass around.
 struct BStepSmem {
@@ -197,14 +188,14 @@ __device__ __forceinline__ bool bstep_stage(const BatchDev& B, const StepItems& 
       const BInst& I = B.inst[it.x];
       Dev2D d;
       make_dev_in(B, I, sel, d);
-      sweep_x_tile<LINEAR, CHAR, true, true>(d, B.alpha[2 * it.x], (unsigned)it.y, sm, (size_t)I.off_n,
+      sweep_x_tile<LINEAR, CHAR, true, true>(d, BatchSource{&B, it.x, sel}, B.alpha[2 * it.x], (unsigned)it.y, sm, (size_t)I.off_n,
                                              (size_t)I.off_x);
     } else {
       const int4 it = P.y[w - P.n_x];
       const BInst& I = B.inst[it.x];
       Dev2D d;
       make_dev_in(B, I, sel, d);
-      sweep_y_tile<LINEAR, CHAR, true, true>(d, B.alpha[2 * it.x + 1], (unsigned)it.y, I.yc, sm,
+      sweep_y_tile<LINEAR, CHAR, true, true>(d, BatchSource{&B, it.x, sel}, B.alpha[2 * it.x + 1], (unsigned)it.y, I.yc, sm,
                                              (size_t)I.off_n, (size_t)I.off_y);
     }
   }
@@ -233,7 +224,7 @@ __device__ __forceinline__ bool bstep_stage(const BatchDev& B, const StepItems& 
           sa.base[q] = B.base[q];
           sa.rhs_out[q] = nullptr;
         }
-        node_update<MODE_STAGE, LINEAR, CHAR, true, true>(d, sa, ii, j, (size_t)I.off_n, (size_t)I.off_x,
+        node_update<MODE_STAGE, LINEAR, CHAR, true, true>(d, BatchSource{&B, it.x, sel}, sa, ii, j, (size_t)I.off_n, (size_t)I.off_x,
                                                           (size_t)I.off_y);
       }
     }
@@ -246,7 +237,7 @@ __device__ __forceinline__ bool bstep_stage(const BatchDev& B, const StepItems& 
 // (One copy of the stage code selects the input pointers: two inlined copies, one per direction, spill
 // several times more.) Dynamic shared memory: one BStepSmem.
 template <bool LINEAR, bool CHAR>
-__global__ void __launch_bounds__(TILE_T, 4) k_bstep(const BatchDev B, const StepItems P, int cur) {
+__global__ void __launch_bounds__(TILE_T, 4) k_bstep(const __grid_constant__ BatchDev B, const StepItems P, int cur) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BStepSmem& sh = *reinterpret_cast<BStepSmem*>(smem_raw);
   if ((int)blockIdx.x == P.drop_block) return;  // test of the bounded wait: this block never arrives

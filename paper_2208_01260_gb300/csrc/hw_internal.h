@@ -127,6 +127,23 @@ constexpr size_t kAlphaOneMax = (size_t)1 << 18;  // nodes up to which the doubl
 void launch_alpha_finish2d(const Dev2D& d, unsigned long long* amax, int* status, const AlphaOut& out, cudaStream_t st);
 void launch_alpha_finish2d(const Dev2DT<float>& d, unsigned long long* amax, int* status, const AlphaOut& out,
                            cudaStream_t st);
+// One block of a decomposed grid on this device: both state plane sets over its extended (nx + 4) x (ny + 4) nodes,
+// its faces as in hw_part_info, and where its alpha, step and time live.
+struct PartBlock {
+  double* S[2][9];
+  double* b;
+  int nx, ny;
+  int mode[4], nbr[4];
+  double *alpha, *dt;
+  const double* t;
+  int* status;
+};
+// The start of a stage of all blocks (parts: np of them on the device, host: the same on the host), reading plane set
+// cur: ring exchange, alpha, with_dt also the step as AlphaOut. slots: 4, zero before the first launch. d: any block's
+// (spacings and g are common).
+void launch_parts_begin(const PartBlock* parts, const PartBlock* host, int np, int cur, const Dev2D& d, unsigned oddx,
+                        unsigned oddy, unsigned long long* slots, bool with_dt, double cfl, double t_end,
+                        cudaStream_t st);
 // both sweeps (one launch while the grid is small)
 void launch_sweeps2d(const Dev2D& d, const double* alpha, bool linear, bool chr, cudaStream_t st);
 void launch_finish_alpha2d(const Dev2D& d, const unsigned long long* amax, double* alpha, double* dt_out,
@@ -199,6 +216,9 @@ int solver_view(hw_solver* s, SolverView* v);
 // the stream the solver launches on (swapped for graph capture; returns the previous one).
 int part_planes(hw_solver* s, int set, double** planes, int* nplanes);
 const Dev2D* part_dev(hw_solver* s);
+void part_block(hw_solver* s, PartBlock* b);
+// stage k of an initialised block whose ring, alpha and step are in place (launch_parts_begin)
+void part_stage(hw_solver* s, int k);
 cudaStream_t solver_swap_stream(hw_solver* s, cudaStream_t st);
 int solver_cur(hw_solver* s);                  // which of the two state buffers holds the state
 cudaStream_t solver_stream(hw_solver* s);

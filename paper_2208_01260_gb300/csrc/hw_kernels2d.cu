@@ -38,24 +38,24 @@ template <class R>
 constexpr int kNodeBlocks = std::is_same<R, double>::value ? 3 : 5;
 
 template <bool LINEAR, bool CHAR, class R>
-__global__ void __launch_bounds__(kXT<R>, kXsBlocks) k_sweep_x(Dev2DT<R> d, const R* __restrict__ alpha) {
+__global__ void __launch_bounds__(kXT<R>, kXsBlocks) k_sweep_x(const __grid_constant__ Dev2DT<R> d, const R* __restrict__ alpha) {
   __shared__ R sm[kTileRec<R> * kXT<R>];
-  sweep_x_tile<LINEAR, CHAR, kFixed<R>, false, kXT<R>>(d, alpha[0], blockIdx.x * (kXT<R> - 3), sm);
+  sweep_x_tile<LINEAR, CHAR, kFixed<R>, false, kXT<R>>(d, GridSource<R>{&d}, alpha[0], blockIdx.x * (kXT<R> - 3), sm);
 }
 
 template <bool LINEAR, bool CHAR>
-__global__ void __launch_bounds__(TILE_T, kYsBlocks) k_sweep_y(Dev2D d, const double* __restrict__ alpha) {
+__global__ void __launch_bounds__(TILE_T, kYsBlocks) k_sweep_y(const __grid_constant__ Dev2D d, const double* __restrict__ alpha) {
   __shared__ double sm[NRECX * TILE_T];
-  sweep_y_tile<LINEAR, CHAR, true>(d, alpha[1], blockIdx.x * (TILE_T / YS_C - 3), YS_C, sm);
+  sweep_y_tile<LINEAR, CHAR, true>(d, GridSource<double>{&d}, alpha[1], blockIdx.x * (TILE_T / YS_C - 3), YS_C, sm);
 }
 
 // Both sweeps in one launch, for grids whose tiles fill the GPU a few times at most: a sweep of few tiles lasts as
 // long as one tile's chain, and each sweep's last wave runs partly empty.
 template <bool CHAR>
-__global__ void __launch_bounds__(TILE_T, kYsBlocks) k_sweep_xy(Dev2D d, const double* __restrict__ alpha, int nxt) {
+__global__ void __launch_bounds__(TILE_T, kYsBlocks) k_sweep_xy(const __grid_constant__ Dev2D d, const double* __restrict__ alpha, int nxt) {
   __shared__ double sm[NRECX * TILE_T];
-  if ((int)blockIdx.x < nxt) sweep_x_tile<false, CHAR, true>(d, alpha[0], blockIdx.x * (TILE_T - 3), sm);
-  else sweep_y_tile<false, CHAR, true>(d, alpha[1], (blockIdx.x - nxt) * (TILE_T / YS_C - 3), YS_C, sm);
+  if ((int)blockIdx.x < nxt) sweep_x_tile<false, CHAR, true>(d, GridSource<double>{&d}, alpha[0], blockIdx.x * (TILE_T - 3), sm);
+  else sweep_y_tile<false, CHAR, true>(d, GridSource<double>{&d}, alpha[1], (blockIdx.x - nxt) * (TILE_T / YS_C - 3), YS_C, sm);
 }
 
 // Single-precision y-sweep: bound by memory rather than arithmetic, it keeps the column march, whose
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(YS_W, 32) k_sweep_y_col(Dev2DT<float> d, const
 // T threads per block: 256, or 64 for grids that do not fill the GPU with those (their warps then spread over more
 // SMs, and need not spill).
 template <int MODE, bool LINEAR, bool CHAR, class R, int T = kNodeT>
-__global__ void __launch_bounds__(T, T == kNodeT ? kNodeBlocks<R> : 8) k_node2d(Dev2DT<R> d, StageArgsT<R> sa) {
+__global__ void __launch_bounds__(T, T == kNodeT ? kNodeBlocks<R> : 8) k_node2d(const __grid_constant__ Dev2DT<R> d, StageArgsT<R> sa) {
   const int i = blockIdx.x * 32 + threadIdx.x;
   const int j = blockIdx.y * (T / 32) + threadIdx.y;
   if (MODE == MODE_STAGE && sa.nsteps && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(T, T == kNodeT ? kNodeBlocks<R> : 8) k_node2d(
     if (sa.clock[0] > 0.0) ++*sa.nsteps;
   }
   if (i >= d.nx || j >= d.ny) return;
-  node_update<MODE, LINEAR, CHAR, kFixed<R>>(d, sa, i, j);
+  node_update<MODE, LINEAR, CHAR, kFixed<R>>(d, GridSource<R>{&d}, sa, i, j);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -256,65 +256,108 @@ __global__ void __launch_bounds__(256) k_alpha2d_exact(Dev2D d, const unsigned i
   if (FINISH && threadIdx.x == 0) alpha_block_done(keys, f);
 }
 
-// The whole reduction in one launch, for small grids (kAlphaOneMax): each block takes 256 U nodes, finds their float
-// maxima and evaluates in double its nodes near those (the grid's maximum is one block's, so it is among them).
+// The whole reduction in one launch, for small grids (kAlphaOneMax): each block takes 256 U nodes.
 // Measured: 3.8 + 4.5 + 2.5 us and a memset in three launches at 64x66 become one of 4.3 us.
 template <int U>
 __global__ void __launch_bounds__(256) k_alpha2d_one(Dev2D d, unsigned long long* slots, int* status, AlphaOut f) {
-  __shared__ float s_m[2][8];
-  __shared__ unsigned long long s_k[2][8];
-  const size_t n = (size_t)d.nx * d.ny, o0 = (size_t)blockIdx.x * (256 * U) + threadIdx.x;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float fx[U], fy[U], mx = 0.0f, my = 0.0f;
-  bool exact[U], neg[U];
-  int bad = 0;
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    exact[u] = false;
-    neg[u] = true;  // past the end: skipped
-    fx[u] = fy[u] = 0.0f;
-    if (o0 + u * 256 < n) {
-      alpha_coarse(d, o0 + u * 256, fx[u], fy[u], exact[u], neg[u]);
-      if (neg[u] && !exact[u]) bad |= HW_STATUS_DEPTH;
-    }
-    if (!exact[u] && !neg[u]) {
-      mx = fmaxf(mx, fx[u]);
-      my = fmaxf(my, fy[u]);
-    }
-  }
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) {
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
-    my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, s));
-  }
-  if (lane == 0) { s_m[0][w] = mx; s_m[1][w] = my; }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    mx = fmaxf(mx, s_m[0][k]);
-    my = fmaxf(my, s_m[1][k]);
-  }
-  const float tx = mx * (1.0f - 1e-5f), ty = my * (1.0f - 1e-5f);
-  unsigned long long kx = 0, ky = 0;
-#pragma unroll
-  for (int u = 0; u < U; ++u)
-    if (o0 + u * 256 < n && alpha_needs_exact(fx[u], fy[u], exact[u], neg[u], tx, ty)) alpha_exact_node(d, o0 + u * 256, kx, ky, bad);
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) {
-    kx = max(kx, __shfl_xor_sync(0xffffffffu, kx, s));
-    ky = max(ky, __shfl_xor_sync(0xffffffffu, ky, s));
-  }
-  if (bad) atomicOr(status, bad);
-  if (lane == 0) { s_k[0][w] = kx; s_k[1][w] = ky; }
-  __syncthreads();
+  unsigned long long kx, ky;
+  alpha_block_keys<U>(d, (size_t)blockIdx.x * (256 * U) + threadIdx.x, (size_t)d.nx * d.ny, [](size_t o) { return o; },
+                      kx, ky, status);
   if (threadIdx.x != 0) return;
-  for (int k = 1; k < 8; ++k) {
-    kx = max(kx, s_k[0][k]);
-    ky = max(ky, s_k[1][k]);
-  }
   if (kx) atomicMax(slots, kx);
   if (ky) atomicMax(slots + 1, ky);
   alpha_block_done(slots, f);
+}
+
+// The start of a stage of all blocks of a decomposed grid: alpha over the blocks' own nodes (alpha_blocks thread
+// blocks of 1024 nodes per block of the grid) and the exchange of their rings (the other thread blocks). A ring node
+// takes its value through at most one y face and one x face straight from the node it is a copy of; only own nodes
+// are read and only ring nodes written, so the two parts need no order. Bound by latency: 600x512 in 2x2 blocks moves
+// 0.6 MB of rings and reads 10 MB for alpha.
+__global__ void __launch_bounds__(256) k_parts_begin(const PartBlock* __restrict__ parts, int np, int cur, double g,
+                                                     unsigned oddx, unsigned oddy, int alpha_blocks,
+                                                     unsigned long long* slots, AlphaOut f) {
+  const int chunk = (int)(blockIdx.x / (unsigned)np);
+  const PartBlock& P = parts[blockIdx.x - (unsigned)chunk * np];
+  if (chunk < alpha_blocks) {
+    Dev2D d;
+    d.g = g;
+    for (int q = 0; q < 3; ++q) d.S[q] = P.S[cur][q];
+    d.stat[0] = P.b;
+    const unsigned nx = (unsigned)P.nx;
+    unsigned long long kx, ky;
+    alpha_block_keys<4>(d, (size_t)chunk * 1024 + threadIdx.x, (size_t)P.nx * P.ny,
+                        [nx](size_t o) {
+                          const unsigned j = (unsigned)o / nx, i = (unsigned)o - j * nx;
+                          return (size_t)(j + 2) * (nx + 4) + i + 2;
+                        },
+                        kx, ky, P.status);
+    if (threadIdx.x == 0) {
+      if (kx) atomicMax(slots, kx);
+      if (ky) atomicMax(slots + 1, ky);
+    }
+  } else {
+    const int r = (chunk - alpha_blocks) * 256 + threadIdx.x, W = P.nx + 4;
+    if (r < 4 * (W + P.ny)) {
+      // the ring: rows 0, 1, ny + 2, ny + 3 in full width, then columns 0, 1, nx + 2, nx + 3 of the other rows
+      int i, j;
+      if (r < 4 * W) {
+        const int row = r / W;
+        i = r - row * W;
+        j = row < 2 ? row : P.ny + row;
+      } else {
+        const int q = r - 4 * W, c = q & 3;
+        j = 2 + (q >> 2);
+        i = c < 2 ? c : P.nx + c;
+      }
+      // the node's source across a face of block b, in b's direction of length n: coordinate k (0, 1 or n + 2, n + 3)
+      auto cross = [&](const PartBlock*& b, int lo, int n, int n_of_nbr, int& k) {
+        const bool low = k < 2;
+        const int face = low ? lo : lo + 1, c = low ? k : k - (n + 2), mode = b->mode[face];
+        if (mode == HW_HALO_NEIGHBOR) {
+          k = low ? n_of_nbr + c : 2 + c;
+          b = parts + b->nbr[face];
+          return false;
+        }
+        const int sc = mode == HW_HALO_MIRROR ? 1 - c : low ? 0 : 1;
+        k = (low ? 2 : n) + sc;
+        return mode == HW_HALO_MIRROR;
+      };
+      const PartBlock* s = &P;
+      int si = i, sj = j;
+      bool fx = false, fy = false;
+      if (sj < 2 || sj >= s->ny + 2) fy = cross(s, HW_FACE_S, s->ny, parts[s->nbr[sj < 2 ? HW_FACE_S : HW_FACE_N]].ny, sj);
+      if (si < 2 || si >= s->nx + 2) fx = cross(s, HW_FACE_W, s->nx, parts[s->nbr[si < 2 ? HW_FACE_W : HW_FACE_E]].nx, si);
+      const size_t from = (size_t)sj * (s->nx + 4) + si, to = (size_t)j * W + i;
+      double v[9];
+#pragma unroll
+      for (int q = 0; q < 9; ++q) v[q] = s->S[cur][q][from];
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        if (fx && ((oddx >> q) & 1u)) v[q] = -v[q];
+        if (fy && ((oddy >> q) & 1u)) v[q] = -v[q];
+        P.S[cur][q][to] = v[q];
+      }
+    }
+  }
+  // the last thread block to end forms every block's alpha (and dt)
+  __shared__ int s_last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(slots + 3, 1ull) == (unsigned long long)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const unsigned long long ax = atomicMax(slots, 0ull), ay = atomicMax(slots + 1, 0ull);
+  for (int p = threadIdx.x; p < np; p += 256) {
+    f.alpha = parts[p].alpha;
+    f.dt = parts[p].dt;
+    f.t_now = f.with_dt ? parts[p].t : nullptr;
+    finish_alpha(ax, ay, f);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) slots[0] = slots[1] = slots[2] = slots[3] = 0;
 }
 
 // Single precision: the maximum in float, widened to a double key once per block. Each thread keeps the
@@ -616,6 +659,19 @@ void launch_alpha_finish2d(const Dev2DT<float>& d, unsigned long long* amax, int
   const size_t n = (size_t)d.nx * d.ny;
   const int blocks = (int)std::min<size_t>((n + 255) / 256, (size_t)152 * 8);
   k_alpha2d_f32<<<blocks, 256, 0, st>>>(d, amax + kAlpha2dSlots, status, out);
+}
+
+void launch_parts_begin(const PartBlock* parts, const PartBlock* host, int np, int cur, const Dev2D& d, unsigned oddx,
+                        unsigned oddy, unsigned long long* slots, bool with_dt, double cfl, double t_end,
+                        cudaStream_t st) {
+  size_t na = 0, nr = 0;
+  for (int p = 0; p < np; ++p) {
+    na = std::max(na, ((size_t)host[p].nx * host[p].ny + 1023) / 1024);
+    nr = std::max(nr, ((size_t)4 * (host[p].nx + 4 + host[p].ny) + 255) / 256);
+  }
+  k_parts_begin<<<(unsigned)((na + nr) * np), 256, 0, st>>>(
+      parts, np, cur, d.g, oddx, oddy, (int)na, slots,
+      AlphaOut{nullptr, nullptr, with_dt, cfl, d.inv_dx, d.inv_dy, nullptr, t_end, nullptr});
 }
 
 void launch_finish_alpha2d(const Dev2D& d, const unsigned long long* amax, double* alpha, double* dt_out,

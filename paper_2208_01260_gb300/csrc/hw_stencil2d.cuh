@@ -428,11 +428,21 @@ __device__ __forceinline__ bool interface_values_fixed(const double* r0, const d
   return !bad;
 }
 
+// Where the two fallback calls below find their grid: a kernel parameter's address for one grid; the batched kernels,
+// which form a Dev2D per thread, have the call form it again (BatchSource), because a local block whose address went
+// into a call would be written to local memory, all 560 bytes of it, by every thread that never makes the call.
+template <class R>
+struct GridSource {
+  const Dev2DT<R>* p;
+  __device__ __forceinline__ const Dev2DT<R>& dev() const { return *p; }
+};
+
 // An interface whose data does not fit the fixed-point form, from its nodes again on the FP64 pipe: nodes
 // (i - 2 .. i + 1, j) for DIR = 0, (i, j - 2 .. j + 1) for DIR = 1.
-template <int DIR, bool CHAR, bool COH>
-__device__ __noinline__ void interface_fallback(const Dev2D& d, double alpha, int i, int j, size_t on, const double qb[6],
+template <int DIR, bool CHAR, bool COH, class S>
+__device__ __noinline__ void interface_fallback(const S src, double alpha, int i, int j, size_t on, const double qb[6],
                                                 double out[12]) {
+  const Dev2D& d = src.dev();
   double rec[4 * NREC];
 #pragma unroll 1
   for (int s = 0; s < 4; ++s) {
@@ -529,6 +539,65 @@ __device__ __forceinline__ void alpha_exact_range(const Dev2D& d, const unsigned
   }
 }
 
+// alpha keys of one block of 256 threads and 256 U nodes in one pass: float maxima first, then the double values of
+// the block's nodes near those (the grid's maximum is one block's, so it is among them). Node u of a thread has number
+// o0 + 256 u below n and lies at at(number). kx, ky: the block's maxima, in thread 0; status flags go to *status.
+template <int U, class At>
+__device__ __forceinline__ void alpha_block_keys(const Dev2D& d, size_t o0, size_t n, At at, unsigned long long& kx,
+                                                 unsigned long long& ky, int* status) {
+  __shared__ float s_m[2][8];
+  __shared__ unsigned long long s_k[2][8];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float fx[U], fy[U], mx = 0.0f, my = 0.0f;
+  bool exact[U], neg[U];
+  int bad = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    exact[u] = false;
+    neg[u] = true;  // past the end: skipped
+    fx[u] = fy[u] = 0.0f;
+    if (o0 + u * 256 < n) {
+      alpha_coarse(d, at(o0 + u * 256), fx[u], fy[u], exact[u], neg[u]);
+      if (neg[u] && !exact[u]) bad |= HW_STATUS_DEPTH;
+    }
+    if (!exact[u] && !neg[u]) {
+      mx = fmaxf(mx, fx[u]);
+      my = fmaxf(my, fy[u]);
+    }
+  }
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
+    my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, s));
+  }
+  if (lane == 0) { s_m[0][w] = mx; s_m[1][w] = my; }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    mx = fmaxf(mx, s_m[0][k]);
+    my = fmaxf(my, s_m[1][k]);
+  }
+  const float tx = mx * (1.0f - 1e-5f), ty = my * (1.0f - 1e-5f);
+  kx = ky = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (o0 + u * 256 < n && alpha_needs_exact(fx[u], fy[u], exact[u], neg[u], tx, ty))
+      alpha_exact_node(d, at(o0 + u * 256), kx, ky, bad);
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    kx = max(kx, __shfl_xor_sync(0xffffffffu, kx, s));
+    ky = max(ky, __shfl_xor_sync(0xffffffffu, ky, s));
+  }
+  if (bad) atomicOr(status, bad);
+  if (lane == 0) { s_k[0][w] = kx; s_k[1][w] = ky; }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int k = 1; k < 8; ++k) {
+    kx = max(kx, s_k[0][k]);
+    ky = max(ky, s_k[1][k]);
+  }
+}
+
 // ---------------------------------------------------------------------------------------------
 // Sweep tiles over flattened extended lines (shared by the single-grid and the batched kernels).
 // x: extended node E = j (nx + 4) + e stands for node (e - 2, j), e = 0 .. nx + 3 (each row with two halo
@@ -546,8 +615,8 @@ __device__ __forceinline__ void alpha_exact_range(const Dev2D& d, const unsigned
 // ---------------------------------------------------------------------------------------------
 constexpr int TILE_T = 128;
 
-template <bool LINEAR, bool CHAR, bool FIXED, bool COH = false, int T = TILE_T, class R>
-__device__ __forceinline__ void sweep_x_tile(const Dev2DT<R>& d, R ax, unsigned E0, R* sm, size_t on = 0,
+template <bool LINEAR, bool CHAR, bool FIXED, bool COH = false, int T = TILE_T, class S, class R>
+__device__ __forceinline__ void sweep_x_tile(const Dev2DT<R>& d, const S src, R ax, unsigned E0, R* sm, size_t on = 0,
                                              size_t oi = 0) {
   const unsigned W = d.nx + 4, total = (unsigned)d.ny * W;
   const int t = threadIdx.x;
@@ -582,7 +651,7 @@ __device__ __forceinline__ void sweep_x_tile(const Dev2DT<R>& d, R ax, unsigned 
   R out[12];
   if constexpr (FIXED && !LINEAR) {
     if (!interface_values_fixed<0, CHAR>(sm + t, sm + t + 1, sm + t + 2, sm + t + 3, T, qb, d, out))
-      interface_fallback<0, CHAR, COH>(d, ax, (int)k, (int)j, on, qb, out);
+      interface_fallback<0, CHAR, COH>(src, ax, (int)k, (int)j, on, qb, out);
   } else {
       interface_values<0, LINEAR, CHAR>(sm + t, sm + t + 1, sm + t + 2, sm + t + 3, T, qb, R(d.g), R(d.eps_w), out);
   }
@@ -590,8 +659,8 @@ __device__ __forceinline__ void sweep_x_tile(const Dev2DT<R>& d, R ax, unsigned 
   for (int q = 0; q < 12; ++q) d.X[q][o] = out[q];
 }
 
-template <bool LINEAR, bool CHAR, bool FIXED, bool COH = false, class R>
-__device__ __forceinline__ void sweep_y_tile(const Dev2DT<R>& d, R ay, unsigned E0, int yc, R* sm, size_t on = 0,
+template <bool LINEAR, bool CHAR, bool FIXED, bool COH = false, class S, class R>
+__device__ __forceinline__ void sweep_y_tile(const Dev2DT<R>& d, const S src, R ay, unsigned E0, int yc, R* sm, size_t on = 0,
                                              size_t oi = 0) {
   const int rows = TILE_T / yc, ifs = rows - 3;
   const unsigned H = d.ny + 4, total = (unsigned)((d.nx + yc - 1) / yc) * H;
@@ -632,7 +701,7 @@ __device__ __forceinline__ void sweep_y_tile(const Dev2DT<R>& d, R ay, unsigned 
   const R* s0 = sm + t;
   if constexpr (FIXED && !LINEAR) {
     if (!interface_values_fixed<1, CHAR>(s0, s0 + yc, s0 + 2 * yc, s0 + 3 * yc, TILE_T, qb, d, out))
-      interface_fallback<1, CHAR, COH>(d, ay, i, (int)k, on, qb, out);
+      interface_fallback<1, CHAR, COH>(src, ay, i, (int)k, on, qb, out);
   } else {
       interface_values<1, LINEAR, CHAR>(s0, s0 + yc, s0 + 2 * yc, s0 + 3 * yc, TILE_T, qb, R(d.g), R(d.eps_w), out);
   }
@@ -696,8 +765,9 @@ __device__ __forceinline__ void limit_node(const Dev2DT<R>& d, int i, int j, siz
 }
 
 // The same as a call, for the nodes whose data does not fit the fixed-point form.
-template <bool CHAR, bool COH>
-__device__ __noinline__ void limit_node_fallback(const Dev2D& d, int i, int j, size_t on, const double* cur, double* mod) {
+template <bool CHAR, bool COH, class S>
+__device__ __noinline__ void limit_node_fallback(const S src, int i, int j, size_t on, const double* cur, double* mod) {
+  const Dev2D& d = src.dev();
   limit_node<false, CHAR, COH>(d, i, j, on, cur, mod);
 }
 
@@ -803,8 +873,8 @@ __device__ __forceinline__ bool limit_node_fixed(const Dev2D& d, int i, int j, s
 // RHS assembly, limiter and RK combination (or the bare RHS) at node (i, j) of one grid. FIXED: the limiter in
 // fixed point where the node's data fits it. on, oxo, oyo: offsets of the grid in pooled node, x-interface and
 // y-interface planes (0 for one grid). COH: loads of the state, interface and base planes as in ldp.
-template <int MODE, bool LINEAR, bool CHAR, bool FIXED = false, bool COH = false, class R>
-__device__ __forceinline__ void node_update(const Dev2DT<R>& d, const StageArgsT<R>& sa, int i, int j, size_t on = 0,
+template <int MODE, bool LINEAR, bool CHAR, bool FIXED = false, bool COH = false, class S, class R>
+__device__ __forceinline__ void node_update(const Dev2DT<R>& d, const S src, const StageArgsT<R>& sa, int i, int j, size_t on = 0,
                                             size_t oxo = 0, size_t oyo = 0) {
   const size_t o = on + (size_t)j * d.nx + i;
   const size_t ox = oxo + (size_t)j * (d.nx + 1) + i;  // left x-interface; right is ox + 1
@@ -823,7 +893,7 @@ __device__ __forceinline__ void node_update(const Dev2DT<R>& d, const StageArgsT
   if (MODE == MODE_STAGE) {
     if (sa.limiter) {
       if constexpr (FIXED && !LINEAR && std::is_same<R, double>::value) {
-        if (!limit_node_fixed<CHAR, COH>(d, i, j, on, cur, mod)) limit_node_fallback<CHAR, COH>(d, i, j, on, cur, mod);
+        if (!limit_node_fixed<CHAR, COH>(d, i, j, on, cur, mod)) limit_node_fallback<CHAR, COH>(src, i, j, on, cur, mod);
       } else {
         limit_node<LINEAR, CHAR, COH>(d, i, j, on, cur, mod);
       }
