@@ -109,10 +109,11 @@ struct hw_solver {
 };
 
 // Grid spacings and the assembly constants derived from them (a sub-domain takes the global grid's).
-static void set_spacing2d(hw::Dev2D& d, double dx, double dy) {
+static void set_spacing2d(hw::Dev2D& d, double dx, double dy, double g) {
   d.dx = dx; d.dy = dy; d.inv_dx = 1.0 / dx; d.inv_dy = 1.0 / dy;
   d.c_bx = 0.5 / dx; d.c_by = 0.5 / dy; d.c_gx = 1.0 / (24.0 * dx); d.c_gy = 1.0 / (24.0 * dy);
   d.c_mx = 1.0 / (12.0 * dx); d.c_my = 1.0 / (12.0 * dy);
+  hw::set_spacing_products(d, g);
 }
 
 // Bracket the launches enqueued by fn() (kernels of them) with a pair of events when profiling.
@@ -221,7 +222,7 @@ int hw_create(const hw_grid* grid, const hw_params* params, void* cuda_stream, h
     hw::Dev2D& d = s->d2;
     const double dy = (grid->y1 - grid->y0) / ny;
     d.nx = nx; d.ny = ny; d.bc_x = grid->bc_x; d.bc_y = grid->bc_y;
-    set_spacing2d(d, dx, dy);
+    set_spacing2d(d, dx, dy, params->g);
     hw::set_physics(d, params->g, params->eps_w, params->eps_lim);
     for (int q = 0; q < 3; ++q) A(&d.stat[q], s->n);
     for (int q = 0; q < 2; ++q) A(&d.bxy[q], s->n);
@@ -800,7 +801,7 @@ int hw_part_create(const hw_grid* grid, const hw_params* params, int px, int py,
   hw_solver* s = nullptr;
   rc = hw_create(&ext, params, cuda_stream, &s);
   if (rc != HW_OK) return rc;
-  set_spacing2d(s->d2, dx, dy);  // the global spacings exactly (ext.x1 - ext.x0 may round)
+  set_spacing2d(s->d2, dx, dy, s->params.g);  // the global spacings exactly (ext.x1 - ext.x0 may round)
   s->is_part = true;
   s->part_info = info;
   *out = s;

@@ -173,6 +173,7 @@ hw::Dev2D dev_of(hw_batch* b, int i, double** S) {
   d.dx = I.dx; d.dy = I.dy; d.inv_dx = I.inv_dx; d.inv_dy = I.inv_dy;
   hw::set_physics(d, b->params.g, b->params.eps_w, b->params.eps_lim);
   d.c_bx = I.c_bx; d.c_by = I.c_by; d.c_gx = I.c_gx; d.c_gy = I.c_gy; d.c_mx = I.c_mx; d.c_my = I.c_my;
+  d.c_bgx = I.c_bgx; d.c_bgy = I.c_bgy;
   for (int q = 0; q < 9; ++q) d.S[q] = S[q] + I.off_n;
   for (int q = 0; q < 3; ++q) d.stat[q] = b->B.stat[q] + I.off_n;
   for (int q = 0; q < 2; ++q) d.bxy[q] = b->B.bxy[q] + I.off_n;
@@ -321,6 +322,7 @@ int hw_batch_create(int n, const hw_grid* grids, const hw_params* params, void* 
     I.inv_dx = 1.0 / I.dx; I.inv_dy = 1.0 / I.dy;
     I.c_bx = 0.5 / I.dx; I.c_by = 0.5 / I.dy; I.c_gx = 1.0 / (24.0 * I.dx); I.c_gy = 1.0 / (24.0 * I.dy);
     I.c_mx = 1.0 / (12.0 * I.dx); I.c_my = 1.0 / (12.0 * I.dy);
+    hw::set_spacing_products(I, params->g);
     I.off_n = (long long)b->tot_n; I.off_x = (long long)b->tot_x; I.off_y = (long long)b->tot_y;
     I.yc = 2;
     b->tot_n += (size_t)g.nx * g.ny;

@@ -8,7 +8,7 @@ namespace hw {
 
 struct BInst {
   int nx, ny, bc_x, bc_y;
-  double dx, dy, inv_dx, inv_dy, c_bx, c_by, c_gx, c_gy, c_mx, c_my;
+  double dx, dy, inv_dx, inv_dy, c_bx, c_by, c_gx, c_gy, c_mx, c_my, c_bgx, c_bgy;
   long long off_n, off_x, off_y;  // offsets of this grid in the pooled node / x-interface / y-interface planes
   int yc;                          // columns per y-tile group (1, 2 or 4; TILE_T / yc extended rows per tile)
 };
@@ -46,6 +46,7 @@ __device__ __forceinline__ void make_dev(const BatchDev& B, const BInst& I, Dev2
   d.half_g = B.half_g; d.fx_eps13 = B.fx_eps13; d.fx_eps2 = B.fx_eps2;
   d.fx_eps13l = B.fx_eps13l; d.fx_eps2l = B.fx_eps2l;
   d.c_bx = I.c_bx; d.c_by = I.c_by; d.c_gx = I.c_gx; d.c_gy = I.c_gy; d.c_mx = I.c_mx; d.c_my = I.c_my;
+  d.c_bgx = I.c_bgx; d.c_bgy = I.c_bgy;
 #pragma unroll
   for (int q = 0; q < 9; ++q) d.S[q] = B.S[q];
 #pragma unroll

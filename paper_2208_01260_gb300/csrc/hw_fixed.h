@@ -160,6 +160,50 @@ HW_FX double fx_to_double(int64_t x, int u) {
   return x == 0 ? 0.0 : f64_from_words(fx_lo(r), h);
 }
 
+// A positive constant as m 2^u with m in [2^62, 2^63), for fx_to_double_scaled. bad: its exponent is too far from 0
+// for results that stay in the normal range.
+struct FxScale {
+  uint64_t m;
+  int u;
+};
+HW_FX FxScale fx_scale(double c, bool& bad) {
+  uint32_t lo, hi;
+  f64_words(c, lo, hi);
+  const int e = (int)(hi >> 20);  // negative, infinite and NaN: above the range
+  bad |= (unsigned)(e - 1023 + 40) > 80u;
+  FxScale s;
+  s.m = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 42) | ((uint64_t)lo << 10);
+  s.u = e - 1085;
+  return s;
+}
+// x 2^u times the constant, rounded to nearest (the product keeps 60 bits, so within 0.52 units in the last place), for
+// |x| < 2^63. The product costs 9 integer instructions where a multiplication after the conversion costs the FP64 pipe
+// 17 cycles a warp, the time of 40 of them.
+HW_FX double fx_to_double_scaled(int64_t x, int u, FxScale c) {
+  const uint32_t s = (uint32_t)((uint64_t)x >> 63);
+  uint64_t a = ((uint64_t)x ^ (0ull - s)) + s;
+  const bool small = fx_hi(a) == 0;
+  const int n = fx_clz(small ? fx_lo(a) : fx_hi(a)) + (small ? 31 : -1);  // leading bit to 62
+  a = fx_mulhi_u(a << n, c.m);                                            // [2^60, 2^62)
+  const int k = (int)((fx_hi(a) >> 29) ^ 1u);
+  const uint64_t r = ((a << k) + 0x100u) >> 9;
+  const uint32_t h = fx_hi(r) + ((uint32_t)(u + c.u + 1147 - n - k) << 20) + (s << 31);
+  return x == 0 ? 0.0 : f64_from_words(fx_lo(r), h);
+}
+// x / 4, rounded to nearest even where it is subnormal: the exponent field, without the FP64 pipe.
+HW_FX double fx_quarter(double x) {
+  uint32_t lo, hi;
+  f64_words(x, lo, hi);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  if (e <= 2 && (lo | (hi << 1)) != 0u) {
+    const int n = 3 - fx_max(e, 1);
+    const uint64_t m = ((uint64_t)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo;
+    const uint64_t r = (m + ((1ull << (n - 1)) - 1) + ((m >> n) & 1)) >> n;
+    return f64_from_words(fx_lo(r), fx_hi(r) | (hi & 0x80000000u));
+  }
+  return e == 0 || e == 0x7ff ? x : f64_from_words(lo, hi - 0x200000u);
+}
+
 // ---- nonlinear weights ----------------------------------------------------------------------
 // Positive quantities of their own scale: q 2^x (x relative to a scale common to the three).
 HW_FX uint64_t fx_shr(uint64_t a, int n) { return a >> fx_min(n, 63); }

@@ -20,6 +20,7 @@ struct Dev2DT {
   // assembly constants: 1/(2dx), 1/(2dy), 1/(24dx), 1/(24dy), 1/(12dx), 1/(12dy)
   R c_bx, c_by, c_gx, c_gy, c_mx, c_my;
   R half_g;            // g / 2
+  R c_bgx, c_bgy;      // g / (2dx), g / (2dy) (double grids; set_spacing_products)
   R fx_eps13, fx_eps2;    // the weights' epsilon of the fixed-point sweeps: (160/781) g eps_w, (80/781) eps_w
   R fx_eps13l, fx_eps2l;  // and of the limiter: (12/13) g eps_lim, (3/13) eps_lim
   R* S[9];      // current state (eta, m, w, dx V, dy Q)
@@ -46,6 +47,14 @@ inline void set_physics(D& d, double g, double eps_w, double eps_lim) {
   d.fx_eps2 = (R)((80.0 / 781.0) * eps_w);
   d.fx_eps13l = (R)((12.0 / 13.0) * eps_lim * g);
   d.fx_eps2l = (R)((3.0 / 13.0) * eps_lim);
+}
+
+// g c_b, rounded once from c_g = c_b / 12: the interface values carry c_g (fluxes) and this (bottom), whose quotient
+// decides how well the two balance at rest.
+template <class D>
+inline void set_spacing_products(D& d, double g) {
+  d.c_bgx = (double)(12.0L * (long double)g * (long double)d.c_gx);
+  d.c_bgy = (double)(12.0L * (long double)g * (long double)d.c_gy);
 }
 
 template <class R>

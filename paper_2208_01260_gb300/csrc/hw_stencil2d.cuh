@@ -152,9 +152,28 @@ __device__ __forceinline__ void node_record_fixed(const Node12& n, double g, dou
 // ---------------------------------------------------------------------------------------------
 // One interface from the four stencil records (nodes i-1, i, i+1, i+2 along the sweep).
 // Outputs (12): 2 Fhat, 2 bhat, 24 dS Ghat (derivative-equation flux), 12 dT Mhat (mixed term),
-// where dS is the spacing along the sweep and dT the spacing across it.
+// where dS is the spacing along the sweep and dT the spacing across it. In double the first three carry the factors
+// the node update would apply to their differences (interface_scales): there each costs the FP64 pipe an operation per
+// difference, here most are part of the fixed-point form's conversions.
 // qb[6] = source candidates q_1..q_3 of (b, dS b_s) for the '+' side then the mirrored '-' side.
 // ---------------------------------------------------------------------------------------------
+// Factors of the double interface values of sweep DIR: cf of 2 Fhat is 12 c_g = 1/(2dS), cb of 2 bhat is g/(2dS), cg of
+// 24 dS Ghat is 1/(24dS).
+template <int DIR>
+__device__ __forceinline__ double scale_g(const Dev2D& d) { return DIR == 0 ? d.c_gx : d.c_gy; }
+template <int DIR>
+__device__ __forceinline__ double scale_b(const Dev2D& d) { return DIR == 0 ? d.c_bgx : d.c_bgy; }
+template <int DIR>
+__device__ __forceinline__ void interface_scales(const Dev2D& d, double out[12]) {
+  const double cg = scale_g<DIR>(d), cf = 12.0 * cg, cb = scale_b<DIR>(d);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    out[c] *= cf;
+    out[3 + c] *= cb;
+    out[6 + c] *= cg;
+  }
+}
+
 template <int DIR, bool LINEAR, bool CHAR, class R>
 __device__ __forceinline__ void interface_values(const R* r0, const R* r1, const R* r2,
                                                    const R* r3, int stride, const R qb[6], R g,
@@ -290,6 +309,7 @@ __device__ __forceinline__ bool interface_values_fixed(const double* r0, const d
   const double upc = fma(gh, rs, un), umc = fma(-gh, rs, un);
   const FxEps eps2 = fx_eps(d.fx_eps2, bad);
   const FxEps eps13 = CHAR ? fx_eps(d.fx_eps13 * hs, bad) : eps2;
+  const FxScale kg = fx_scale(scale_g<DIR>(d), bad), kb = fx_scale(scale_b<DIR>(d), bad);
   // units of the fields' data (below 2^57): field k is its component (normal, tangential, normal) plus c_k F_0,
   // c = (-(un + c), -ut, -(un - c)); a coefficient's shift brings its products to the field's unit
   int U02 = 0, U1 = 0;
@@ -393,21 +413,21 @@ __device__ __forceinline__ bool interface_values_fixed(const double* r0, const d
   // the source values) a factor 1/2
   const int ub_ = eb - 1082;
   if (CHAR) {
-    const double ic2 = 0.5 * rs;
-    const double A = fx_to_double(G[2] - G[0], U02) * ((1.0 / 6.0) * ic2);
+    // 2 Fhat = (A, un A + (G2 + G0)/12, ut A + G1/6) with A = (G2 - G0) / (12 c), times 12 c_g
+    const double A = fx_to_double(G[2] - G[0], U02) * (scale_g<DIR>(d) * rs);
     out[0] = A;
-    out[cn] = fma(un, A, (1.0 / 12.0) * fx_to_double(G[2] + G[0], U02));
-    out[ct] = fma(ut, A, (1.0 / 6.0) * fx_to_double(G[1], U1));
-    const double Bs = fx_to_double(BA, ub_) * rs;
+    out[cn] = fma(un, A, fx_to_double_scaled(G[2] + G[0], U02, kg));
+    out[ct] = fma(ut, A, fx_to_double_scaled(G[1], U1 + 1, kg));
+    const double Bs = fx_to_double(BA, ub_) * (scale_b<DIR>(d) * rs);
     out[3] = Bs;
-    out[3 + cn] = fma(un, Bs, fx_to_double(BD, ub_));
+    out[3 + cn] = fma(un, Bs, fx_to_double_scaled(BD, ub_, kb));
     out[3 + ct] = ut * Bs;
   } else {
-    out[0] = (1.0 / 6.0) * fx_to_double(G[0], m0 - 1078);
-    out[cn] = (1.0 / 6.0) * fx_to_double(G[1], mn - 1078);
-    out[ct] = (1.0 / 6.0) * fx_to_double(G[2], mt - 1078);
+    out[0] = fx_to_double_scaled(G[0], m0 - 1077, kg);
+    out[cn] = fx_to_double_scaled(G[1], mn - 1077, kg);
+    out[ct] = fx_to_double_scaled(G[2], mt - 1077, kg);
     out[3] = 0.0;
-    out[3 + cn] = fx_to_double(BD, ub_);
+    out[3 + cn] = fx_to_double_scaled(BD, ub_, kb);
     out[3 + ct] = 0.0;
   }
   // derivative-equation flux and mixed term
@@ -418,9 +438,9 @@ __device__ __forceinline__ bool interface_values_fixed(const double* r0, const d
     const int64_t f1[3] = {load(3, R_FM), load(2, R_FM), load(1, R_FM)}, p1[3] = {load(3, R_GM), load(2, R_GM), load(1, R_GM)};
     Q[2] = quintic(f0, p0) - quintic(f1, p1);
   }
-  out[6] = fx_to_double(Q[0], m0 - 1078);
-  out[6 + cn] = fx_to_double(Q[1], CHAR ? U02 : mn - 1078);
-  out[6 + ct] = fx_to_double(Q[2], mt - 1078);
+  out[6] = fx_to_double_scaled(Q[0], m0 - 1078, kg);
+  out[6 + cn] = fx_to_double_scaled(Q[1], CHAR ? U02 : mn - 1078, kg);
+  out[6 + ct] = fx_to_double_scaled(Q[2], mt - 1078, kg);
 #pragma unroll
   for (int c = 0; c < 3; ++c)
     out[9 + c] = fma(7.0, RV(r1, R_MIX + c) + RV(r2, R_MIX + c), -(RV(r0, R_MIX + c) + RV(r3, R_MIX + c)));
@@ -451,6 +471,7 @@ __device__ __noinline__ void interface_fallback(const S src, double alpha, int i
     node_record<DIR>(n, d.g, alpha, rec + s * NREC);
   }
   interface_values<DIR, false, CHAR>(rec, rec + NREC, rec + 2 * NREC, rec + 3 * NREC, 1, qb, d.g, d.eps_w, out);
+  interface_scales<DIR>(d, out);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -654,6 +675,7 @@ __device__ __forceinline__ void sweep_x_tile(const Dev2DT<R>& d, const S src, R 
       interface_fallback<0, CHAR, COH>(src, ax, (int)k, (int)j, on, qb, out);
   } else {
       interface_values<0, LINEAR, CHAR>(sm + t, sm + t + 1, sm + t + 2, sm + t + 3, T, qb, R(d.g), R(d.eps_w), out);
+      if constexpr (std::is_same<R, double>::value) interface_scales<0>(d, out);
   }
 #pragma unroll
   for (int q = 0; q < 12; ++q) d.X[q][o] = out[q];
@@ -704,6 +726,7 @@ __device__ __forceinline__ void sweep_y_tile(const Dev2DT<R>& d, const S src, R 
       interface_fallback<1, CHAR, COH>(src, ay, i, (int)k, on, qb, out);
   } else {
       interface_values<1, LINEAR, CHAR>(s0, s0 + yc, s0 + 2 * yc, s0 + 3 * yc, TILE_T, qb, R(d.g), R(d.eps_w), out);
+      if constexpr (std::is_same<R, double>::value) interface_scales<1>(d, out);
   }
 #pragma unroll
   for (int q = 0; q < 12; ++q) d.Y[q][o] = out[q];
@@ -903,45 +926,65 @@ __device__ __forceinline__ void node_update(const Dev2DT<R>& d, const S src, con
     }
   }
   // ---- RHS (eq. swe-form-2d-dis) in scaled units: R_U, dx R_V, dy R_Q ----
+  // In double: of the negative, whose 50 operations bound this part (64 with the factors applied here, 3 more per node in
+  // the RK combination; node kernel at 2048^2 1.04 -> 0.94 ms, the sweeps within 2% of what they were).
   const R eta = cur[0], H1 = cur[3], H2 = cur[6];
   const R g = R(d.g);
-  // grid constants in the working precision
-  const R c_bx = R(d.c_bx), c_by = R(d.c_by), c_gx = R(d.c_gx), c_gy = R(d.c_gy), c_mx = R(d.c_mx),
-          c_my = R(d.c_my);
+  const R c_mx = R(d.c_mx), c_my = R(d.c_my);
   const R ge = g * eta;
   R Rv[9];
+  if constexpr (std::is_same<R, double>::value) {
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const R dFx = ldp<COH>(d.X[c] + ox + 1) - ldp<COH>(d.X[c] + ox);
-    const R dFy = ldp<COH>(d.Y[c] + oy + d.nx) - ldp<COH>(d.Y[c] + oy);
-    const R dbx = ldp<COH>(d.X[3 + c] + ox + 1) - ldp<COH>(d.X[3 + c] + ox);
-    const R dby = ldp<COH>(d.Y[3 + c] + oy + d.nx) - ldp<COH>(d.Y[3 + c] + oy);
-    const R dGx = ldp<COH>(d.X[6 + c] + ox + 1) - ldp<COH>(d.X[6 + c] + ox);
-    const R dGy = ldp<COH>(d.Y[6 + c] + oy + d.nx) - ldp<COH>(d.Y[6 + c] + oy);
-    const R dMx = ldp<COH>(d.X[9 + c] + ox + 1) - ldp<COH>(d.X[9 + c] + ox);
-    const R dMy = ldp<COH>(d.Y[9 + c] + oy + d.nx) - ldp<COH>(d.Y[9 + c] + oy);
-    const R db = fma(c_bx, dbx, c_by * dby);  // [b~]_x/dx + [b-]_y/dy
-    Rv[c] = fma(-ge, db, fma(-c_bx, dFx, -(c_by * dFy)));
-    R rv = fma(-c_gx, dGx, -(c_my * dMy));
-    R rq = fma(-c_mx, dMx, -(c_gy * dGy));
-    if (c > 0) {
-      rv = fma(-ge, __ldg(d.sv[c - 1] + o), rv);
-      rq = fma(-ge, __ldg(d.sq[c - 1] + o), rq);
+    for (int c = 0; c < 3; ++c) {
+      auto dx_ = [&](int q) { return ldp<COH>(d.X[q + c] + ox + 1) - ldp<COH>(d.X[q + c] + ox); };
+      auto dy_ = [&](int q) { return ldp<COH>(d.Y[q + c] + oy + d.nx) - ldp<COH>(d.Y[q + c] + oy); };
+      const R db = dx_(3) + dy_(3);  // g ([b~]_x/dx + [b-]_y/dy)
+      Rv[c] = fma(eta, db, dx_(0) + dy_(0));
+      R rv = fma(H1, db, fma(c_my, dy_(9), dx_(6)));
+      R rq = fma(H2, db, fma(c_mx, dx_(9), dy_(6)));
+      if (c > 0) {
+        rv = fma(ge, __ldg(d.sv[c - 1] + o), rv);
+        rq = fma(ge, __ldg(d.sq[c - 1] + o), rq);
+      }
+      Rv[3 + c] = rv;
+      Rv[6 + c] = rq;
     }
-    Rv[3 + c] = fma(-(g * H1), db, rv);
-    Rv[6 + c] = fma(-(g * H2), db, rq);
+  } else {
+    const R c_bx = d.c_bx, c_by = d.c_by, c_gx = d.c_gx, c_gy = d.c_gy;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const R dFx = ldp<COH>(d.X[c] + ox + 1) - ldp<COH>(d.X[c] + ox);
+      const R dFy = ldp<COH>(d.Y[c] + oy + d.nx) - ldp<COH>(d.Y[c] + oy);
+      const R dbx = ldp<COH>(d.X[3 + c] + ox + 1) - ldp<COH>(d.X[3 + c] + ox);
+      const R dby = ldp<COH>(d.Y[3 + c] + oy + d.nx) - ldp<COH>(d.Y[3 + c] + oy);
+      const R dGx = ldp<COH>(d.X[6 + c] + ox + 1) - ldp<COH>(d.X[6 + c] + ox);
+      const R dGy = ldp<COH>(d.Y[6 + c] + oy + d.nx) - ldp<COH>(d.Y[6 + c] + oy);
+      const R dMx = ldp<COH>(d.X[9 + c] + ox + 1) - ldp<COH>(d.X[9 + c] + ox);
+      const R dMy = ldp<COH>(d.Y[9 + c] + oy + d.nx) - ldp<COH>(d.Y[9 + c] + oy);
+      const R db = fma(c_bx, dbx, c_by * dby);  // [b~]_x/dx + [b-]_y/dy
+      Rv[c] = fma(-ge, db, fma(-c_bx, dFx, -(c_by * dFy)));
+      R rv = fma(-c_gx, dGx, -(c_my * dMy));
+      R rq = fma(-c_mx, dMx, -(c_gy * dGy));
+      if (c > 0) {
+        rv = fma(-ge, __ldg(d.sv[c - 1] + o), rv);
+        rq = fma(-ge, __ldg(d.sq[c - 1] + o), rq);
+      }
+      Rv[3 + c] = fma(-(g * H1), db, rv);
+      Rv[6 + c] = fma(-(g * H2), db, rq);
+    }
   }
   if (MODE == MODE_RHS) {
     // physical units: R_V = (dx R_V)/dx, R_Q = (dy R_Q)/dy
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
       const R s = q < 3 ? R(1.0) : R(q < 6 ? d.inv_dx : d.inv_dy);
-      sa.rhs_out[q][o] = Rv[q] * s;
+      const R r = q < 3 ? Rv[q] : Rv[q] * s;
+      sa.rhs_out[q][o] = std::is_same<R, double>::value ? flip_sign(r, 0x80000000u) : r;
     }
     return;
   }
   // ---- SSP-RK3 combination (eq. RK) ----
-  const R dt = R(*sa.dt);
+  const R dt = std::is_same<R, double>::value ? -R(*sa.dt) : R(*sa.dt);
   if (sa.k == 1) {
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
@@ -949,7 +992,19 @@ __device__ __forceinline__ void node_update(const Dev2DT<R>& d, const S src, con
       if (sa.base) sa.base[q][o] = cq;
       sa.out[q][o] = fma(dt, Rv[q], cq);
     }
-  } else {
+    return;
+  }
+  if constexpr (std::is_same<R, double>::value) {
+    if (sa.k == 2) {  // (3 base + cq + dt R) / 4: two operations on the FP64 pipe
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const R cq = q < 3 ? cur[q] : mod[q - 3];
+        sa.out[q][o] = fx_quarter(fma(dt, Rv[q], fma(3.0, ldp<COH>(sa.base[q] + o), cq)));
+      }
+      return;
+    }
+  }
+  {
     const R a = sa.k == 2 ? R(0.75) : R(1.0) / R(3.0);
     const R b = sa.k == 2 ? R(0.25) : R(2.0) / R(3.0);
 #pragma unroll
