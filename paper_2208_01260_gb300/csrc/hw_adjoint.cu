@@ -4,7 +4,7 @@
 // Reverse of one RK stage (eq. RK with the right-hand side of eq. swe-form-2d-dis):
 //   k_adj_node_pre   RK combination, node-local terms of the assembly (g eta, g H1, g H2 times the
 //                    source differences), the adjoint of the limited derivatives
-//   k_adj_sweep_x/y  adjoint of each interface's 12 values (from the two neighbouring nodes), reverse
+//   k_adj_sweeps    adjoint of each interface's 12 values (from the two neighbouring nodes), reverse
 //                    of the reconstruction (Sec. 2.1 Steps 1-2, eq. mixed) into the four stencil records
 //   k_adj_records    reverse of the per-node records (fluxes, chain-rule derivatives, LF split), ghost
 //                    records mapped back to the mirrored or periodic node with the parity table
@@ -37,7 +37,7 @@ struct AdjDev {
   const double* lout[9];  // adjoint of the stage output
   double* lin[9];         // adjoint of the stage input (written)
   double* lbase[9];       // adjoint of the step base (accumulated over stages 3, 2; consumed at stage 1)
-  double* lR[9];          // adjoint of the right-hand side (scratch)
+  double* lR[12];         // adjoint of the right-hand side, and g (eta lR_c + H1 lR_3+c + H2 lR_6+c) (scratch)
   double* lmod[6];        // adjoint of the limited derivatives (scratch)
   double* lrecx[NREC];    // record adjoints, x: rows of nx + 4 (raw index -2 .. nx+1)
   double* lrecy[NREC];    // record adjoints, y: ny + 4 rows of nx
@@ -85,12 +85,17 @@ __device__ __forceinline__ double block_sum(double v) {
   return v;  // lane 0 of each warp holds the warp sum
 }
 
+// Threads per block of the node kernels and the records, over nodes (records) one after the other: small blocks, so that
+// the small grids this runs on spread their FP64 work over all SMs (150 x 97 nodes are 57 blocks of 256).
+constexpr int A_NT = 64;
+
 // ---- 1. node pre-pass ----
-__global__ void __launch_bounds__(256) k_adj_node_pre(AdjDev A) {
-  const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y;
+__global__ void __launch_bounds__(A_NT) k_adj_node_pre(const __grid_constant__ AdjDev A) {
   const Dev2D& d = A.d;
-  if (i >= d.nx || j >= d.ny) return;
-  const size_t o = (size_t)j * d.nx + i;
+  const unsigned tid = blockIdx.x * A_NT + threadIdx.x;
+  const int j = (int)(tid / (unsigned)d.nx), i = (int)(tid - (unsigned)j * d.nx);
+  if (j >= d.ny) return;
+  const size_t o = tid;
   double lc[9], lR[9];
 #pragma unroll
   for (int q = 0; q < 9; ++q) {
@@ -142,186 +147,150 @@ __global__ void __launch_bounds__(256) k_adj_node_pre(AdjDev A) {
   A.lin[6][o] += lH2;
 #pragma unroll
   for (int q = 0; q < 9; ++q) A.lR[q][o] = lR[q];
+  const double gH1 = g * d.S[3][o], gH2 = g * d.S[6][o];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) A.lR[9 + c][o] = fma(ge, lR[c], fma(gH1, lR[3 + c], gH2 * lR[6 + c]));
 }
 
-// adjoint of the 12 values of the x-interface k of row j (from nodes k-1 and k)
-__device__ __forceinline__ void interface_adjoint_x(const AdjDev& A, int k, int j, double lX[12]) {
+// adjoint of an interface's 12 values: differences over its two nodes (entries o0 and o1 of the planes; off the grid,
+// has0 or has1 false, a node counts zero) times cb (fluxes and bottom), cg (derivative flux) and cm (mixed term)
+template <int DIR>
+__device__ __forceinline__ void interface_adjoint(const AdjDev& A, size_t o0, size_t o1, bool has0, bool has1, double lX[12]) {
   const Dev2D& d = A.d;
-  for (int q = 0; q < 12; ++q) lX[q] = 0.0;
+  const double cb = DIR == 0 ? d.c_bx : d.c_by, cg = DIR == 0 ? d.c_gx : d.c_gy, cm = DIR == 0 ? d.c_mx : d.c_my;
+  auto diff = [&](int q) { return (has1 ? A.lR[q][o1] : 0.0) - (has0 ? A.lR[q][o0] : 0.0); };
 #pragma unroll
-  for (int side = 0; side < 2; ++side) {
-    const int p = side == 0 ? k - 1 : k;  // node seeing k as its right (side 0) or left (side 1) interface
-    if (p < 0 || p >= d.nx) continue;
-    const double sgn = side == 0 ? -1.0 : 1.0;
-    const size_t o = (size_t)j * d.nx + p;
-    const double g = d.g, ge = g * d.S[0][o], gH1 = g * d.S[3][o], gH2 = g * d.S[6][o];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const double lu = A.lR[c][o], lv = A.lR[3 + c][o], lq = A.lR[6 + c][o];
-      lX[c] += sgn * d.c_bx * lu;
-      lX[3 + c] += sgn * d.c_bx * (ge * lu + gH1 * lv + gH2 * lq);
-      lX[6 + c] += sgn * d.c_gx * lv;
-      lX[9 + c] += sgn * d.c_mx * lq;
-    }
+  for (int c = 0; c < 3; ++c) {
+    lX[c] = cb * diff(c);
+    lX[3 + c] = cb * diff(9 + c);
+    // along x the derivative flux feeds the V equations and the mixed term the Q equations, along y the reverse
+    lX[6 + c] = cg * diff(DIR == 0 ? 3 + c : 6 + c);
+    lX[9 + c] = cm * diff(DIR == 0 ? 6 + c : 3 + c);
   }
 }
 
-__device__ __forceinline__ void interface_adjoint_y(const AdjDev& A, int i, int k, double lY[12]) {
-  const Dev2D& d = A.d;
-  for (int q = 0; q < 12; ++q) lY[q] = 0.0;
+// The sum over a record's interfaces of entry f's adjoints: stencil position s of the interface s before the record's
+// own, for the positions that write the entry (FP, GP: 0..2; FM, GM: 1..3; mixed: all; state: 1, 2). at(s): the slab
+// entry (s, f), false ok(s): outside the block.
+template <class At, class Ok>
+__device__ __forceinline__ double record_sum(int f, const At& at, const Ok& ok) {
+  const int lo = f < R_FM ? 0 : f < R_GP ? 1 : f < R_GM ? 0 : f < R_MIX ? 1 : f < R_H ? 0 : 1;
+  const int hi = f < R_FM ? 2 : f < R_GP ? 3 : f < R_GM ? 2 : f < R_H ? 3 : 2;
+  double acc = ok(lo) ? at(lo) : 0.0;
 #pragma unroll
-  for (int side = 0; side < 2; ++side) {
-    const int p = side == 0 ? k - 1 : k;
-    if (p < 0 || p >= d.ny) continue;
-    const double sgn = side == 0 ? -1.0 : 1.0;
-    const size_t o = (size_t)p * d.nx + i;
-    const double g = d.g, ge = g * d.S[0][o], gH1 = g * d.S[3][o], gH2 = g * d.S[6][o];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const double lu = A.lR[c][o], lv = A.lR[3 + c][o], lq = A.lR[6 + c][o];
-      lY[c] += sgn * d.c_by * lu;
-      lY[3 + c] += sgn * d.c_by * (ge * lu + gH1 * lv + gH2 * lq);
-      lY[6 + c] += sgn * d.c_gy * lq;  // Psi2 hat feeds the Q equations
-      lY[9 + c] += sgn * d.c_my * lv;  // mixed Phi2 hat feeds the V equations
-    }
-  }
+  for (int s = 1; s < 4; ++s)
+    if (s > lo && s <= hi && ok(s)) acc += at(s);
+  return acc;
 }
 
-// ---- 2. x-interfaces (a block of AX_T threads: AX_I = AX_T - 3 consecutive interfaces of one row and
-// their AX_N = AX_T node records, one per thread) ----
-// The four record adjoints of each interface collect in a shared-memory slab; after the block has
-// finished, each record sums its (up to) four contributions, so only the three records a block shares
-// with each neighbour are added atomically.
-constexpr int AX_T = 64;
-constexpr int AX_I = AX_T - 3;
-constexpr int AX_N = AX_T;
+// ---- 2. interfaces of both sweeps, over the flattened extended lines of hw_stencil2d.cuh ----
+// A block of AT threads reverses AX_I consecutive x-interfaces (their AT records, one per thread), or AY_R y-interfaces
+// of AY_C adjacent columns. The four record adjoints of each interface collect in a shared-memory slab; after the block
+// has finished, each record sums its contributions, so only the three records (rows of records) a block shares with
+// each neighbour are added atomically.
+//
+// Bound by the FP64 pipe, at 255 registers a thread: 8 warps per SM, in whatever blocks. Both sweeps are one launch of
+// small blocks because the grids this runs on are small: as two launches, with 256 threads a y-block, a grid of 150 x 97
+// had 291 and 65 blocks (the y-sweep on 65 of 152 SMs, as long as two of its warps per partition take), and one of
+// 256^2 ran 2.1 and 1.7 waves in 3 and 2. Measured with the reverse's fewer operations (hw_adjoint.cuh): 271 us a stage for
+// both sweeps at 256^2, 75 us at 150 x 97; the whole gradient 11.9 -> 10.2 ms and 15.4 -> 13.1 ms.
+constexpr int AT = 64;
+constexpr int AX_I = AT - 3;
+constexpr int AY_C = 4, AY_R = AT / AY_C, AY_NR = AY_R + 3;
+constexpr int A_NREC = AY_NR * AY_C;  // records held (an x-block's AT are fewer)
 
-__global__ void __launch_bounds__(AX_T) k_adj_sweep_x(AdjDev A) {
-  __shared__ double sm[NREC * AX_N];
-  __shared__ double slab[4 * NREC * AX_T];
+__global__ void __launch_bounds__(AT) k_adj_sweeps(const __grid_constant__ AdjDev A, unsigned nxt) {
+  __shared__ double recs[NREC * A_NREC];
+  __shared__ double slab[4 * NREC * AT];
   const Dev2D& d = A.d;
-  const int j = blockIdx.y, k0 = blockIdx.x * AX_I;
-  const double ax = A.alpha[0];
   const int t = threadIdx.x;
-  for (int u = t; u < AX_N; u += AX_T) {
-    const int i = k0 - 2 + u;
-    if (i > d.nx + 1) break;
-    Node12 n;
-    load_node(d, i, j, n);
-    double rec[NREC];
-    node_record<0>(n, d.g, ax, rec);
+  if (blockIdx.x < nxt) {
+    const unsigned W = d.nx + 4, total = (unsigned)d.ny * W, E = blockIdx.x * AX_I + t, j = E / W, e = E - j * W;
+    if (E < total) {
+      Node12 n;
+      load_node(d, (int)e - 2, (int)j, n);
+      double rec[NREC];
+      node_record<0>(n, d.g, A.alpha[0], rec);
 #pragma unroll
-    for (int f = 0; f < NREC; ++f) sm[f * AX_N + u] = rec[f];
-  }
-  __syncthreads();
-  const int k = k0 + t;
-  if (t < AX_I && k <= d.nx) {
-    const size_t o = (size_t)j * (d.nx + 1) + k;
-    double qb[6];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) qb[q] = d.qbx[q][o];
-    double lX[12];
-    interface_adjoint_x(A, k, j, lX);
-    double lqb[6] = {0, 0, 0, 0, 0, 0};
-    interface_values_rev<0>(sm + t, 1, AX_N, qb, A.fax[o], A.dbx[0][o], d.g, d.eps_w, lX,
-                            SlabAcc{slab + t, AX_T}, lqb);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) A.lqbx[q][o] += lqb[q];
-  } else {
-    for (int e = 0; e < 4 * NREC; ++e) slab[e * AX_T + t] = 0.0;  // no interface (tile or row end)
-  }
-  __syncthreads();
-  const size_t row = (size_t)j * (d.nx + 4);
-  for (int u = t; u < AX_N; u += AX_T) {
-    const int r = k0 - 2 + u;  // raw record index, -2 .. nx+1
-    if (r > d.nx + 1) break;
-    const bool shared_slot = u < 3 || u >= AX_I;
-    for (int f = 0; f < NREC; ++f) {
-      double acc = 0.0;
-#pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        const int tt = u - s;
-        if (tt >= 0 && tt < AX_T) acc += slab[(s * NREC + f) * AX_T + tt];
-      }
-      double* dst = A.lrecx[f] + row + (r + 2);
-      if (shared_slot) {
-        if (acc != 0.0) atomicAdd(dst, acc);
-      } else {
-        *dst = acc;
-      }
+      for (int f = 0; f < NREC; ++f) recs[f * A_NREC + t] = rec[f];
     }
-  }
-}
-
-// ---- 2'. y-interfaces (a block: AY_R interface rows of 32 columns; records of AY_R + 3 node rows) ----
-constexpr int AY_R = 8;
-constexpr int AY_NR = AY_R + 3;
-constexpr int AY_T = 32 * AY_R;
-constexpr size_t AY_SMEM = (size_t)(NREC * AY_NR * 32 + 4 * NREC * AY_T) * sizeof(double);
-
-__global__ void __launch_bounds__(AY_T) k_adj_sweep_y(AdjDev A) {
-  extern __shared__ double ysm[];
-  double* recs = ysm;                      // [NREC][AY_NR][32]
-  double* slab = ysm + NREC * AY_NR * 32;  // [4][NREC][AY_T]
-  const Dev2D& d = A.d;
-  const int i0 = blockIdx.x * 32, k0 = blockIdx.y * AY_R;
-  const int tid = threadIdx.x, c = tid & 31, ty = tid >> 5;
-  const double ay = A.alpha[1];
-  for (int idx = tid; idx < AY_NR * 32; idx += AY_T) {
-    const int u = idx >> 5, cc = idx & 31;
-    const int i = i0 + cc, r = k0 - 2 + u;
-    if (i >= d.nx || r > d.ny + 1) continue;
-    Node12 n;
-    load_node(d, i, r, n);
-    double rec[NREC];
-    node_record<1>(n, d.g, ay, rec);
+    __syncthreads();
+    if (t < AX_I && E < total && e <= (unsigned)d.nx) {
+      const size_t o = (size_t)j * (d.nx + 1) + e, on = (size_t)j * d.nx + e;
+      double qb[6], lX[12], lqb[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
-    for (int f = 0; f < NREC; ++f) recs[(f * AY_NR + u) * 32 + cc] = rec[f];
-  }
-  __syncthreads();
-  const int i = i0 + c, k = k0 + ty;
-  if (i < d.nx && k <= d.ny) {
-    const size_t o = (size_t)k * d.nx + i;
-    double qb[6];
+      for (int q = 0; q < 6; ++q) qb[q] = d.qbx[q][o];
+      interface_adjoint<0>(A, on - 1, on, e > 0, e < (unsigned)d.nx, lX);
+      interface_values_rev<0>(recs + t, 1, A_NREC, qb, A.fax[o], A.dbx[0][o], d.g, d.eps_w, lX, SlabAcc{slab + t, AT}, lqb);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) qb[q] = d.qby[q][o];
-    double lY[12];
-    interface_adjoint_y(A, i, k, lY);
-    double lqb[6] = {0, 0, 0, 0, 0, 0};
-    const double* r0 = recs + ty * 32 + c;
-    interface_values_rev<1>(r0, 32, AY_NR * 32, qb, A.fay[o], A.dby[0][o], d.g, d.eps_w, lY,
-                            SlabAcc{slab + tid, AY_T}, lqb);
+      for (int q = 0; q < 6; ++q) A.lqbx[q][o] += lqb[q];
+    } else {
+      for (int q = 0; q < 4 * NREC; ++q) slab[q * AT + t] = 0.0;  // no interface
+    }
+    __syncthreads();
+    if (E >= total) return;
+    const bool shared_slot = t < 3 || t >= AX_I;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) A.lqby[q][o] += lqb[q];
-  } else {
-    for (int e = 0; e < 4 * NREC; ++e) slab[e * AY_T + tid] = 0.0;  // past the grid's edge
-  }
-  __syncthreads();
-  for (int idx = tid; idx < AY_NR * 32; idx += AY_T) {
-    const int u = idx >> 5, cc = idx & 31;
-    const int ii = i0 + cc, r = k0 - 2 + u;  // raw record row, -2 .. ny+1
-    if (ii >= d.nx || r > d.ny + 1) continue;
-    const bool shared_row = u < 3 || u >= AY_R;
-    const size_t pos = (size_t)(r + 2) * d.nx + ii;
     for (int f = 0; f < NREC; ++f) {
-      double acc = 0.0;
+      const double acc = record_sum(
+          f, [&](int s) { return slab[(s * NREC + f) * AT + t - s]; }, [&](int s) { return t >= s; });
+      double* dst = A.lrecx[f] + E;
+      if (!shared_slot) *dst = acc;
+      else if (acc != 0.0) atomicAdd(dst, acc);
+    }
+  } else {
+    const unsigned H = d.ny + 4, total = (unsigned)((d.nx + AY_C - 1) / AY_C) * H, E0 = (blockIdx.x - nxt) * AY_R;
+    // record (or interface) idx of the block: extended row E0 + idx / AY_C, column idx % AY_C of the row's group
+    auto place = [&](int idx, int& i, int& e) {
+      const unsigned E = E0 + idx / AY_C, g = E / H;
+      e = (int)(E - g * H);
+      i = (int)g * AY_C + idx % AY_C;
+      return E < total && i < d.nx;
+    };
+    int i, e;
+    for (int idx = t; idx < A_NREC; idx += AT) {
+      if (!place(idx, i, e)) continue;
+      Node12 n;
+      load_node(d, i, e - 2, n);
+      double rec[NREC];
+      node_record<1>(n, d.g, A.alpha[1], rec);
 #pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        const int uu = u - s;
-        if (uu >= 0 && uu < AY_R) acc += slab[(s * NREC + f) * AY_T + uu * 32 + cc];
-      }
-      double* dst = A.lrecy[f] + pos;
-      if (shared_row) {
-        if (acc != 0.0) atomicAdd(dst, acc);
-      } else {
-        *dst = acc;
+      for (int f = 0; f < NREC; ++f) recs[f * A_NREC + idx] = rec[f];
+    }
+    __syncthreads();
+    if (place(t, i, e) && e <= d.ny) {
+      const size_t o = (size_t)e * d.nx + i;
+      double qb[6], lY[12], lqb[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll
+      for (int q = 0; q < 6; ++q) qb[q] = d.qby[q][o];
+      interface_adjoint<1>(A, o - d.nx, o, e > 0, e < d.ny, lY);
+      interface_values_rev<1>(recs + t, AY_C, A_NREC, qb, A.fay[o], A.dby[0][o], d.g, d.eps_w, lY, SlabAcc{slab + t, AT}, lqb);
+#pragma unroll
+      for (int q = 0; q < 6; ++q) A.lqby[q][o] += lqb[q];
+    } else {
+      for (int q = 0; q < 4 * NREC; ++q) slab[q * AT + t] = 0.0;
+    }
+    __syncthreads();
+    for (int idx = t; idx < A_NREC; idx += AT) {
+      if (!place(idx, i, e)) continue;
+      const int u = idx / AY_C;
+      const bool shared_row = u < 3 || u >= AY_R;
+      const size_t pos = (size_t)e * d.nx + i;
+#pragma unroll
+      for (int f = 0; f < NREC; ++f) {
+        const double acc = record_sum(
+            f, [&](int s) { return slab[(s * NREC + f) * AT + idx - s * AY_C]; },
+            [&](int s) { return u >= s && u - s < AY_R; });
+        double* dst = A.lrecy[f] + pos;
+        if (!shared_row) *dst = acc;
+        else if (acc != 0.0) atomicAdd(dst, acc);
       }
     }
   }
 }
 
 // ---- 3. records: raw x-records (r = -2..nx+1, row j) and raw y-records (column i, r = -2..ny+1) ----
-__global__ void __launch_bounds__(256) k_adj_records(AdjDev A) {
+__global__ void __launch_bounds__(A_NT) k_adj_records(const __grid_constant__ AdjDev A) {
   const Dev2D& d = A.d;
   const int nxr = (d.nx + 4) * d.ny, nyr = d.nx * (d.ny + 4);
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -372,11 +341,12 @@ __global__ void __launch_bounds__(256) k_adj_records(AdjDev A) {
 }
 
 // ---- 4. limiter ----
-__global__ void __launch_bounds__(256) k_adj_limiter(AdjDev A) {
-  const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y;
+__global__ void __launch_bounds__(A_NT) k_adj_limiter(const __grid_constant__ AdjDev A) {
   const Dev2D& d = A.d;
-  if (i >= d.nx || j >= d.ny) return;
-  const size_t o = (size_t)j * d.nx + i;
+  const unsigned tid = blockIdx.x * A_NT + threadIdx.x;
+  const int j = (int)(tid / (unsigned)d.nx), i = (int)(tid - (unsigned)j * d.nx);
+  if (j >= d.ny) return;
+  const size_t o = tid;
   double cur[9];
 #pragma unroll
   for (int q = 0; q < 9; ++q) cur[q] = d.S[q][o];
@@ -399,7 +369,7 @@ __global__ void __launch_bounds__(256) k_adj_limiter(AdjDev A) {
     load_node(d, im, jm, nm);
     load_node(d, ip, jp, np);
     const int qd = dir == 0 ? 3 : 6;
-    double lUm[3] = {}, lU0[3] = {}, lUp[3] = {}, lDm[3] = {}, lDp[3] = {};
+    double lUm[3], lU0[3], lUp[3], lDm[3], lDp[3];
     if (dir == 0)
       limit_dir_rev<0>(nm.v, cur, np.v, nm.v + qd, np.v + qd, u, v, c, ic2, gh, d.eps_lim, lo, lUm, lU0, lUp, lDm, lDp,
                        lu, lv, lc, lic2, lgh);
@@ -693,7 +663,7 @@ struct AdjBuffers {
   double* fy[3] = {};
   double* lam[2][9] = {};
   double* lbase[9] = {};
-  double* lR[9] = {};
+  double* lR[12] = {};
   double* lmod[6] = {};
   double* lrecx[hw::NREC] = {};
   double* lrecy[hw::NREC] = {};
@@ -808,7 +778,7 @@ int get_buffers(hw_solver* s, const hw::SolverView& v, AdjBuffers** out) {
   A(B->lam[0], 9, n);
   A(B->lam[1], 9, n);
   A(B->lbase, 9, n);
-  A(B->lR, 9, n);
+  A(B->lR, 12, n);
   A(&B->alpha_st, 1, 8);
   for (int k = 0; k < 3; ++k) {
     A(B->dbx[k], 3, nxi);
@@ -948,8 +918,8 @@ hw::AdjDev stage_args(const hw::SolverView& v, AdjBuffers* B, const StepTape& T,
     A.lout[q] = B->lam[cur][q];
     A.lin[q] = B->lam[cur ^ 1][q];
     A.lbase[q] = B->lbase[q];
-    A.lR[q] = B->lR[q];
   }
+  for (int q = 0; q < 12; ++q) A.lR[q] = B->lR[q];
   for (int q = 0; q < 6; ++q) { A.lmod[q] = B->lmod[q]; A.lqbx[q] = B->lqbx[q]; A.lqby[q] = B->lqby[q]; }
   for (int f = 0; f < hw::NREC; ++f) { A.lrecx[f] = B->lrecx[f]; A.lrecy[f] = B->lrecy[f]; }
   for (int q = 0; q < 3; ++q) { A.lstat[q] = B->lstat[q]; A.dbx[q] = T.dbx[k - 1][q]; A.dby[q] = T.dby[k - 1][q]; }
@@ -969,13 +939,14 @@ int reverse_stage_body(const hw::SolverView& v, AdjBuffers* B, const hw::AdjDev&
   const hw::Dev2D& d = A.d;
   if ((rc = zero_planes(B->lrecx, hw::NREC, (size_t)(d.nx + 4) * d.ny, st))) return rc;
   if ((rc = zero_planes(B->lrecy, hw::NREC, (size_t)d.nx * (d.ny + 4), st))) return rc;
-  const dim3 gn((d.nx + 31) / 32, (d.ny + 7) / 8), bn(32, 8);
-  hw::k_adj_node_pre<<<gn, bn, 0, st>>>(A);
-  hw::k_adj_sweep_x<<<dim3((d.nx + 1 + hw::AX_I - 1) / hw::AX_I, d.ny), hw::AX_T, 0, st>>>(A);
-  hw::k_adj_sweep_y<<<dim3((d.nx + 31) / 32, (d.ny + 1 + hw::AY_R - 1) / hw::AY_R), hw::AY_T, hw::AY_SMEM, st>>>(A);
+  const unsigned gn = ((unsigned)d.nx * d.ny + hw::A_NT - 1) / hw::A_NT;
+  hw::k_adj_node_pre<<<gn, hw::A_NT, 0, st>>>(A);
+  const unsigned nxt = ((unsigned)d.ny * (d.nx + 4) + hw::AX_I - 1) / hw::AX_I;
+  const unsigned nyt = ((unsigned)((d.nx + hw::AY_C - 1) / hw::AY_C) * (d.ny + 4) + hw::AY_R - 1) / hw::AY_R;
+  hw::k_adj_sweeps<<<nxt + nyt, hw::AT, 0, st>>>(A, nxt);
   const int nrec = (d.nx + 4) * d.ny + d.nx * (d.ny + 4);
-  hw::k_adj_records<<<(nrec + 255) / 256, 256, 0, st>>>(A);
-  if (A.limiter) hw::k_adj_limiter<<<gn, bn, 0, st>>>(A);
+  hw::k_adj_records<<<(nrec - 1) / hw::A_NT + 1, hw::A_NT, 0, st>>>(A);
+  if (A.limiter) hw::k_adj_limiter<<<gn, hw::A_NT, 0, st>>>(A);
   ACUDA(cudaGetLastError());
   return HW_OK;
 }
@@ -984,7 +955,6 @@ int reverse_stage_body(const hw::SolverView& v, AdjBuffers* B, const hw::AdjDev&
 // on return (in lam[*cur]); static adjoints accumulate.
 int reverse_recorded(const hw::SolverView& v, AdjBuffers* B, const StepTape& T, double dt, int* cur) {
   int rc = HW_OK;
-  ACUDA(cudaFuncSetAttribute(hw::k_adj_sweep_y, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hw::AY_SMEM));
   cudaStream_t st = v.stream;
   const size_t n = v.n;
   if ((rc = zero_planes(B->lbase, 9, n, st))) return rc;
@@ -1452,7 +1422,6 @@ int dd_adjoint_impl(hw_dd* dd, int nsteps, const double* dts, const int* gauge_i
     if ((rc = check_adjoint_solver(parts[p], &bl[p].v))) return rc;
     if ((rc = get_buffers(parts[p], bl[p].v, &bl[p].B))) return rc;
   }
-  ACUDA(cudaFuncSetAttribute(hw::k_adj_sweep_y, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hw::AY_SMEM));
   std::vector<RunTape> layout;
   for (int p = 0; p < np; ++p) layout.emplace_back(bl[p].v, nsteps);
   // gauges by owner block: local extended node and global slot
@@ -1781,8 +1750,8 @@ int hw_part_adj_create(hw_solver* s, int nsteps, int ngauge, int nloc, const int
   alloc((void**)&a->keys, hw::kAlpha2dScratch * sizeof(double));
   if (rc) { pa_free(a); return rc; }
   cudaStream_t st = a->v.stream;
-  cudaError_t e = cudaFuncSetAttribute(hw::k_adj_sweep_y, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hw::AY_SMEM);
-  if (e == cudaSuccess && nloc) e = cudaMemcpyAsync(a->d_map, map.data(), map.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+  cudaError_t e = cudaSuccess;
+  if (nloc) e = cudaMemcpyAsync(a->d_map, map.data(), map.size() * sizeof(int), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(a->d_gvals, 0, gb, st);
   const StepTape T0 = a->layout->step(a->tape, 0);
   for (int q = 0; q < 9 && e == cudaSuccess; ++q)
