@@ -403,13 +403,17 @@ static void enqueue_stage(hw_solver* s, int k, bool next = false, double t_end =
   const bool lin = s->params.linear_weights != 0, chr = s->params.char_decomp != 0;
   if (s->fp32) {
     float** fout = s->fother();
-    timed(s, HW_PROF_SWEEP_X, [&] { hw::launch_sweep_x2d(s->f2, s->fsc, lin, chr, s->stream); });
-    timed(s, HW_PROF_SWEEP_Y, [&] { hw::launch_sweep_y2d(s->f2, s->fsc, lin, chr, s->stream); });
     hw::StageArgsT<float> sa{};
     sa.k = k; sa.limiter = s->params.limiter; sa.dt = s->fsc + 2;
     for (int q = 0; q < 9; ++q) { sa.out[q] = fout[q]; sa.base[q] = s->fbase[q]; }
     set_clock(s, sa, clock);
-    timed(s, HW_PROF_NODE, [&] { hw::launch_node2d(s->f2, sa, hw::MODE_STAGE, lin, chr, s->stream); });
+    if (lin || s->profiling) {  // linear weights; a profile takes the phases apart
+      timed(s, HW_PROF_SWEEP_X, [&] { hw::launch_sweep_x2d(s->f2, s->fsc, lin, chr, s->stream); });
+      timed(s, HW_PROF_SWEEP_Y, [&] { hw::launch_sweep_y2d(s->f2, s->fsc, lin, chr, s->stream); });
+      timed(s, HW_PROF_NODE, [&] { hw::launch_node2d(s->f2, sa, hw::MODE_STAGE, lin, chr, s->stream); });
+    } else {
+      hw::launch_stage2d_f32(s->f2, sa, s->fsc, chr, s->stream);
+    }
   } else if (s->is2d()) {
     hw::StageArgs sa{};
     sa.k = k; sa.limiter = s->params.limiter; sa.dt = s->dt;

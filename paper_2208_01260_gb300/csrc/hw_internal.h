@@ -169,6 +169,8 @@ void launch_sweep_x2d(const Dev2DT<float>& d, const float* alpha, bool linear, b
 void launch_sweep_y2d(const Dev2DT<float>& d, const float* alpha, bool linear, bool chr, cudaStream_t st);
 void launch_node2d(const Dev2DT<float>& d, const StageArgsT<float>& sa, int mode, bool linear, bool chr,
                    cudaStream_t st);
+// a stage of the single-precision variant in one launch, nonlinear weights (hw_stage32.cu)
+void launch_stage2d_f32(const Dev2DT<float>& d, const StageArgsT<float>& sa, const float* alpha, bool chr, cudaStream_t st);
 void launch_cast_planes(int nplanes, size_t n, const Ptr12& src, const Ptr12& dst, int to_float, cudaStream_t st);
 
 // One RK stage of the adjoint's forward pass (hw_forward64.cu): sweeps and node update in FP64.

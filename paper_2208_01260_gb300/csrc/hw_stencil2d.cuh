@@ -770,20 +770,21 @@ __device__ __forceinline__ void limit_dir(const R Um[3], const R U0[3], const R 
 }
 
 // The limiter of both directions at node (i, j) on the FP64 pipe: scaled V and Q of the node into mod.
-template <bool LINEAR, bool CHAR, bool COH, class R>
-__device__ __forceinline__ void limit_node(const Dev2DT<R>& d, int i, int j, size_t on, const R cur[9], R mod[6]) {
-  const R h = cur[0] - __ldg(d.stat[0] + on + (size_t)j * d.nx + i);
+// b: the node's bottom; at(di, dj, n): its neighbours.
+template <bool LINEAR, bool CHAR, class R, class At>
+__device__ __forceinline__ void limit_node(const Dev2DT<R>& d, R b, const R cur[9], R mod[6], const At& at) {
+  const R h = cur[0] - b;
   const R gh = R(d.g) * h;
   const R rh = fast_rcp(h);
   const R u = cur[1] * rh, v = cur[2] * rh;
   const R rs = fast_rsqrt(gh);
   const R c = gh * rs, ic2 = R(0.5) * rs;
   Node12T<R> nm, np;
-  load_node<COH>(d, i - 1, j, nm, on);
-  load_node<COH>(d, i + 1, j, np, on);
+  at(-1, 0, nm);
+  at(1, 0, np);
   limit_dir<0, LINEAR, CHAR>(nm.v, cur, np.v, nm.v + 3, np.v + 3, u, v, c, ic2, gh, R(d.eps_lim), mod);
-  load_node<COH>(d, i, j - 1, nm, on);
-  load_node<COH>(d, i, j + 1, np, on);
+  at(0, -1, nm);
+  at(0, 1, np);
   limit_dir<1, LINEAR, CHAR>(nm.v, cur, np.v, nm.v + 6, np.v + 6, u, v, c, ic2, gh, R(d.eps_lim), mod + 3);
 }
 
@@ -791,7 +792,8 @@ __device__ __forceinline__ void limit_node(const Dev2DT<R>& d, int i, int j, siz
 template <bool CHAR, bool COH, class S>
 __device__ __noinline__ void limit_node_fallback(const S src, int i, int j, size_t on, const double* cur, double* mod) {
   const Dev2D& d = src.dev();
-  limit_node<false, CHAR, COH>(d, i, j, on, cur, mod);
+  limit_node<false, CHAR>(d, __ldg(d.stat[0] + on + (size_t)j * d.nx + i), cur, mod,
+                          [&](int di, int dj, Node12& n) { load_node<COH>(d, i + di, j + dj, n, on); });
 }
 
 // The same in fixed point (hw_fixed.h): the node and its four neighbours as integers of one unit per component,
@@ -893,18 +895,29 @@ __device__ __forceinline__ bool limit_node_fixed(const Dev2D& d, int i, int j, s
   return true;
 }
 
-// RHS assembly, limiter and RK combination (or the bare RHS) at node (i, j) of one grid. FIXED: the limiter in
-// fixed point where the node's data fits it. on, oxo, oyo: offsets of the grid in pooled node, x-interface and
-// y-interface planes (0 for one grid). COH: loads of the state, interface and base planes as in ldp.
-template <int MODE, bool LINEAR, bool CHAR, bool FIXED = false, bool COH = false, class S, class R>
-__device__ __forceinline__ void node_update(const Dev2DT<R>& d, const S src, const StageArgsT<R>& sa, int i, int j, size_t on = 0,
-                                            size_t oxo = 0, size_t oyo = 0) {
+// What the update of node (i, j) reads of the grid, from the planes: its state, bottom and neighbours, and the differences
+// of interface value q over it along x and y. o, ox, oy: the node, its left x-interface and its lower y-interface.
+template <bool COH, class R>
+struct PlaneFaces {
+  const Dev2DT<R>& d;
+  const int i, j;
+  const size_t on, o, ox, oy;
+  __device__ __forceinline__ R state(int q) const { return ldp<COH>(d.S[q] + o); }
+  __device__ __forceinline__ R bottom() const { return __ldg(d.stat[0] + o); }
+  __device__ __forceinline__ void neighbour(int di, int dj, Node12T<R>& n) const { load_node<COH>(d, i + di, j + dj, n, on); }
+  __device__ __forceinline__ R x(int q) const { return ldp<COH>(d.X[q] + ox + 1) - ldp<COH>(d.X[q] + ox); }
+  __device__ __forceinline__ R y(int q) const { return ldp<COH>(d.Y[q] + oy + d.nx) - ldp<COH>(d.Y[q] + oy); }
+};
+
+// RHS assembly, limiter and RK combination (or the bare RHS) at node (i, j) of one grid, read through faces. FIXED: the limiter in fixed point where the node's data fits it. on: offset of the grid in pooled
+// node planes (0 for one grid). COH: loads of the state and base planes as in ldp.
+template <int MODE, bool LINEAR, bool CHAR, bool FIXED, bool COH, class S, class R, class Faces>
+__device__ __forceinline__ void node_update_faces(const Dev2DT<R>& d, const S src, const StageArgsT<R>& sa, int i, int j, size_t on,
+                                                  const Faces& faces) {
   const size_t o = on + (size_t)j * d.nx + i;
-  const size_t ox = oxo + (size_t)j * (d.nx + 1) + i;  // left x-interface; right is ox + 1
-  const size_t oy = oyo + (size_t)j * d.nx + i;        // lower y-interface; upper is oy + nx
   R cur[9];
 #pragma unroll
-  for (int q = 0; q < 9; ++q) cur[q] = ldp<COH>(d.S[q] + o);
+  for (int q = 0; q < 9; ++q) cur[q] = faces.state(q);
   if (MODE == MODE_STAGE && !(*sa.dt > 0.0)) {
     // a step of size 0 (e.g. clipped at the end time) leaves the state unchanged
 #pragma unroll
@@ -918,7 +931,7 @@ __device__ __forceinline__ void node_update(const Dev2DT<R>& d, const S src, con
       if constexpr (FIXED && !LINEAR && std::is_same<R, double>::value) {
         if (!limit_node_fixed<CHAR, COH>(d, i, j, on, cur, mod)) limit_node_fallback<CHAR, COH>(src, i, j, on, cur, mod);
       } else {
-        limit_node<LINEAR, CHAR, COH>(d, i, j, on, cur, mod);
+        limit_node<LINEAR, CHAR>(d, faces.bottom(), cur, mod, [&](int di, int dj, Node12T<R>& n) { faces.neighbour(di, dj, n); });
       }
     } else {
 #pragma unroll
@@ -936,12 +949,10 @@ __device__ __forceinline__ void node_update(const Dev2DT<R>& d, const S src, con
   if constexpr (std::is_same<R, double>::value) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      auto dx_ = [&](int q) { return ldp<COH>(d.X[q + c] + ox + 1) - ldp<COH>(d.X[q + c] + ox); };
-      auto dy_ = [&](int q) { return ldp<COH>(d.Y[q + c] + oy + d.nx) - ldp<COH>(d.Y[q + c] + oy); };
-      const R db = dx_(3) + dy_(3);  // g ([b~]_x/dx + [b-]_y/dy)
-      Rv[c] = fma(eta, db, dx_(0) + dy_(0));
-      R rv = fma(H1, db, fma(c_my, dy_(9), dx_(6)));
-      R rq = fma(H2, db, fma(c_mx, dx_(9), dy_(6)));
+      const R db = faces.x(3 + c) + faces.y(3 + c);  // g ([b~]_x/dx + [b-]_y/dy)
+      Rv[c] = fma(eta, db, faces.x(c) + faces.y(c));
+      R rv = fma(H1, db, fma(c_my, faces.y(9 + c), faces.x(6 + c)));
+      R rq = fma(H2, db, fma(c_mx, faces.x(9 + c), faces.y(6 + c)));
       if (c > 0) {
         rv = fma(ge, __ldg(d.sv[c - 1] + o), rv);
         rq = fma(ge, __ldg(d.sq[c - 1] + o), rq);
@@ -953,14 +964,8 @@ __device__ __forceinline__ void node_update(const Dev2DT<R>& d, const S src, con
     const R c_bx = d.c_bx, c_by = d.c_by, c_gx = d.c_gx, c_gy = d.c_gy;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const R dFx = ldp<COH>(d.X[c] + ox + 1) - ldp<COH>(d.X[c] + ox);
-      const R dFy = ldp<COH>(d.Y[c] + oy + d.nx) - ldp<COH>(d.Y[c] + oy);
-      const R dbx = ldp<COH>(d.X[3 + c] + ox + 1) - ldp<COH>(d.X[3 + c] + ox);
-      const R dby = ldp<COH>(d.Y[3 + c] + oy + d.nx) - ldp<COH>(d.Y[3 + c] + oy);
-      const R dGx = ldp<COH>(d.X[6 + c] + ox + 1) - ldp<COH>(d.X[6 + c] + ox);
-      const R dGy = ldp<COH>(d.Y[6 + c] + oy + d.nx) - ldp<COH>(d.Y[6 + c] + oy);
-      const R dMx = ldp<COH>(d.X[9 + c] + ox + 1) - ldp<COH>(d.X[9 + c] + ox);
-      const R dMy = ldp<COH>(d.Y[9 + c] + oy + d.nx) - ldp<COH>(d.Y[9 + c] + oy);
+      const R dFx = faces.x(c), dFy = faces.y(c), dbx = faces.x(3 + c), dby = faces.y(3 + c);
+      const R dGx = faces.x(6 + c), dGy = faces.y(6 + c), dMx = faces.x(9 + c), dMy = faces.y(9 + c);
       const R db = fma(c_bx, dbx, c_by * dby);  // [b~]_x/dx + [b-]_y/dy
       Rv[c] = fma(-ge, db, fma(-c_bx, dFx, -(c_by * dFy)));
       R rv = fma(-c_gx, dGx, -(c_my * dMy));
@@ -1013,6 +1018,15 @@ __device__ __forceinline__ void node_update(const Dev2DT<R>& d, const S src, con
       sa.out[q][o] = fma(a, ldp<COH>(sa.base[q] + o), b * fma(dt, Rv[q], cq));
     }
   }
+}
+
+// The same from the interface planes; oxo, oyo: the grid's offsets in pooled ones. COH: their loads too.
+template <int MODE, bool LINEAR, bool CHAR, bool FIXED = false, bool COH = false, class S, class R>
+__device__ __forceinline__ void node_update(const Dev2DT<R>& d, const S src, const StageArgsT<R>& sa, int i, int j, size_t on = 0,
+                                            size_t oxo = 0, size_t oyo = 0) {
+  const size_t o = (size_t)j * d.nx + i;
+  const PlaneFaces<COH, R> faces{d, i, j, on, on + o, oxo + o + j, oyo + o};
+  node_update_faces<MODE, LINEAR, CHAR, FIXED, COH>(d, src, sa, i, j, on, faces);
 }
 
 }  // namespace hw
