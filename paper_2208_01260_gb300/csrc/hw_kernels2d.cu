@@ -21,7 +21,7 @@ constexpr int YS_C = 2;  // columns per y-tile group of the double y-sweep (meas
 
 // The double kernels run the nonlinear reconstruction and the limiter in fixed point (hw_fixed.h): on the FP64
 // pipe alone these kernels took 2.80 (x), 2.85 (y) and 2.03 ms (node) per stage at 2048^2, its operations at the
-// pipe's rate; now 0.78, 0.84 and 0.94 ms. What bounds the sweeps is the sum of what is left on the FP64 pipe (69
+// pipe's rate; now 0.78, 0.84 and 0.87 ms. What bounds the sweeps is the sum of what is left on the FP64 pipe (69
 // operations per x-interface, 58% busy) and integer work (4110 instructions per warp, 54% of the issue slots, the integer
 // pipe 60% busy); the node kernel the FP64 pipe (99 operations, 70% busy) with the latency of its loads.
 template <class R>

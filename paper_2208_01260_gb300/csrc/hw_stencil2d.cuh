@@ -796,43 +796,16 @@ __device__ __noinline__ void limit_node_fallback(const S src, int i, int j, size
                           [&](int di, int dj, Node12& n) { load_node<COH>(d, i + di, j + dj, n, on); });
 }
 
-// The same in fixed point (hw_fixed.h): the node and its four neighbours as integers of one unit per component,
-// the differences and derivatives projected and limited field by field. False (mod unspecified) when an operand
-// does not fit.
+// The same in fixed point (hw_fixed.h), direction by direction: the node and its two neighbours as integers of one unit
+// per component (mass, normal, tangential), the differences and derivatives projected and limited field by field. One
+// copy of the code for both directions, each with its own loads and units: with both directions' 27 values loaded
+// first the node kernel spilled 380 bytes a thread at 80 registers, whose write-back was half of its DRAM writes (now about 90 bytes; a
+// job of two steps at 2048^2 15.97 -> 15.55 ms).
+// False (mod unspecified) when an operand does not fit.
 template <bool CHAR, bool COH>
 __device__ __forceinline__ bool limit_node_fixed(const Dev2D& d, int i, int j, size_t on, const double cur[9],
                                                  double mod[6]) {
-  // U of the node, then of the neighbours W, E, S, N; their derivatives along x (W, E) or y (S, N)
-  double U[5][3], D[4][3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) U[0][c] = cur[c];
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    bool fx, fy;
-    const int ii = map_index(s == 0 ? i - 1 : s == 1 ? i + 1 : i, d.nx, d.bc_x, fx);
-    const int jj = map_index(s == 2 ? j - 1 : s == 3 ? j + 1 : j, d.ny, d.bc_y, fy);
-    const size_t o = on + (size_t)jj * d.nx + ii;
-    const uint32_t m = (s < 2 ? fx : fy) ? 0x80000000u : 0u;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int q = (s < 2 ? 3 : 6) + c;
-      U[s + 1][c] = flip_sign(ldp<COH>(d.S[c] + o), (s < 2 ? par_x2d(c) : par_y2d(c)) < 0 ? m : 0u);
-      D[s][c] = flip_sign(ldp<COH>(d.S[q] + o), (s < 2 ? par_x2d(q) : par_y2d(q)) < 0 ? m : 0u);
-    }
-  }
   bool bad = false;
-  int em[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    uint32_t w = 0, any = 0;
-#pragma unroll
-    for (int s = 0; s < 5; ++s) { w = max(w, fx_absw(U[s][c])); any |= fx_any(U[s][c]); }
-#pragma unroll
-    for (int s = 0; s < 4; ++s) { w = max(w, fx_absw(D[s][c])); any |= fx_any(D[s][c]); }
-    em[c] = (int)(w >> 20);
-    bad |= (em[c] > kFxExpMax) | ((em[c] < kFxExpMin) & (any != 0u));
-    em[c] = max(em[c], kFxExpMin);
-  }
   const double h = cur[0] - __ldg(d.stat[0] + on + (size_t)j * d.nx + i);
   const double gh = d.g * h;
   const double rh = fast_rcp(h);
@@ -840,35 +813,62 @@ __device__ __forceinline__ bool limit_node_fixed(const Dev2D& d, int i, int j, s
   const double rs = fast_rsqrt(gh);
   const FxEps eps2 = fx_eps(d.fx_eps2l, bad);
   const FxEps eps13 = CHAR ? fx_eps(d.fx_eps13l * h, bad) : eps2;
-  if (bad) return false;
-  int64_t c0[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) c0[c] = fx_from_double(U[0][c], em[c]);
-#pragma unroll
+#pragma unroll 1
   for (int dir = 0; dir < 2; ++dir) {
-    const int cn = dir == 0 ? 1 : 2, ct = dir == 0 ? 2 : 1;
+    // planes of (mass, normal, tangential) and of their derivatives along the direction; across a wall the normal
+    // component and the others' derivatives change sign
+    const double* const pu[3] = {d.S[0], dir == 0 ? d.S[1] : d.S[2], dir == 0 ? d.S[2] : d.S[1]};
+    const double* const pd[3] = {dir == 0 ? d.S[3] : d.S[6], dir == 0 ? d.S[4] : d.S[8], dir == 0 ? d.S[5] : d.S[7]};
+    double U[3][3], D[2][3];
+    U[0][0] = cur[0];
+    U[0][1] = dir == 0 ? cur[1] : cur[2];
+    U[0][2] = dir == 0 ? cur[2] : cur[1];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      bool fx, fy;
+      const int ii = map_index(dir == 0 ? i - 1 + 2 * s : i, d.nx, d.bc_x, fx);
+      const int jj = map_index(dir == 0 ? j : j - 1 + 2 * s, d.ny, d.bc_y, fy);
+      const size_t o = on + (size_t)jj * d.nx + ii;
+      const uint32_t m = (dir == 0 ? fx : fy) ? 0x80000000u : 0u;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        U[s + 1][c] = flip_sign(ldp<COH>(pu[c] + o), c == 1 ? m : 0u);
+        D[s][c] = flip_sign(ldp<COH>(pd[c] + o), c == 1 ? 0u : m);
+      }
+    }
+    int em[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const uint32_t w = max(max(max(fx_absw(U[0][c]), fx_absw(U[1][c])), fx_absw(U[2][c])), max(fx_absw(D[0][c]), fx_absw(D[1][c])));
+      const uint32_t any = fx_any(U[0][c]) | fx_any(U[1][c]) | fx_any(U[2][c]) | fx_any(D[0][c]) | fx_any(D[1][c]);
+      em[c] = (int)(w >> 20);
+      bad |= (em[c] > kFxExpMax) | ((em[c] < kFxExpMin) & (any != 0u));
+      em[c] = max(em[c], kFxExpMin);
+    }
+    if (bad) return false;
     // differences to the two neighbours and their derivatives, below 2^61
     int64_t a[4][3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      a[0][c] = c0[c] - fx_from_double(U[1 + 2 * dir][c], em[c]);
-      a[1][c] = fx_from_double(U[2 + 2 * dir][c], em[c]) - c0[c];
-      a[2][c] = fx_from_double(D[2 * dir][c], em[c]);
-      a[3][c] = fx_from_double(D[2 * dir + 1][c], em[c]);
+      const int64_t c0 = fx_from_double(U[0][c], em[c]);
+      a[0][c] = c0 - fx_from_double(U[1][c], em[c]);
+      a[1][c] = fx_from_double(U[2][c], em[c]) - c0;
+      a[2][c] = fx_from_double(D[0][c], em[c]);
+      a[3][c] = fx_from_double(D[1][c], em[c]);
     }
-    double* const out = mod + 3 * dir;
+    double out[3];
     if (CHAR) {
-      const double un = dir == 0 ? u : v, ut = dir == 0 ? v : u;
       // rows (-(un + c), 1, 0), (-ut, 0, 1), (-(un - c), 1, 0) on (mass, normal, tangential)
+      const double un = dir == 0 ? u : v, ut = dir == 0 ? v : u;
       const double upc = fma(gh, rs, un), umc = fma(-gh, rs, un);
       int up, um, uv;
       const int64_t xp = fx_mantissa(-upc, up), xm = fx_mantissa(-umc, um), xv = fx_mantissa(-ut, uv);
       const int u0 = em[0] - 1082 + 64;
-      const int U02 = max(max(max(up, um) + u0 + 2, em[cn] - 1078), -900), U1 = max(max(uv + u0 + 2, em[ct] - 1078), -900);
+      const int U02 = max(max(max(up, um) + u0 + 2, em[1] - 1078), -900), U1 = max(max(uv + u0 + 2, em[2] - 1078), -900);
       if (max(U02, U1) > 900) return false;
       const FxS kp = fx_split(xp >> min(U02 - up - u0, 63)), km = fx_split(xm >> min(U02 - um - u0, 63)),
                 kv = fx_split(xv >> min(U1 - uv - u0, 63));
-      const int sn = min(U02 + 1082 - em[cn], 63), st = min(U1 + 1082 - em[ct], 63);
+      const int sn = min(U02 + 1082 - em[1], 63), st = min(U1 + 1082 - em[2], 63);
       int64_t nu[3];
       FxS x[4];
 #pragma unroll
@@ -878,18 +878,23 @@ __device__ __forceinline__ bool limit_node_fixed(const Dev2D& d, int i, int j, s
         const FxS kk = k == 0 ? kp : k == 1 ? kv : km;
         int64_t f[4];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) f[s] = fx_mulhi(x[s], kk, k == 1 ? a[s][ct] >> st : a[s][cn] >> sn);
+        for (int s = 0; s < 4; ++s) f[s] = fx_mulhi(x[s], kk, k == 1 ? a[s][2] >> st : a[s][1] >> sn);
         nu[k] = fx_limiter_field(f[0], f[1], f[2], f[3], k == 1 ? eps2 : eps13, k == 1 ? U1 : U02);
       }
       const double A = fx_to_double(nu[2] - nu[0], U02 - 1) * (0.5 * rs);
       out[0] = A;
-      out[cn] = fma(un, A, fx_to_double(nu[2] + nu[0], U02 - 2));
-      out[ct] = fma(ut, A, fx_to_double(nu[1], U1 - 1));
+      out[1] = fma(un, A, fx_to_double(nu[2] + nu[0], U02 - 2));
+      out[2] = fma(ut, A, fx_to_double(nu[1], U1 - 1));
     } else {
 #pragma unroll
       for (int c = 0; c < 3; ++c)
         out[c] = fx_to_double(fx_limiter_field(a[0][c] >> 3, a[1][c] >> 3, a[2][c] >> 3, a[3][c] >> 3, eps2, em[c] - 1079),
                               em[c] - 1080);
+    }
+    if (dir == 0) {
+      mod[0] = out[0]; mod[1] = out[1]; mod[2] = out[2];
+    } else {
+      mod[3] = out[0]; mod[4] = out[2]; mod[5] = out[1];
     }
   }
   return true;
