@@ -274,8 +274,10 @@ __device__ __forceinline__ void interface_values(const R* r0, const R* r1, const
 }
 
 // The same interface with the reconstruction and the derivative flux in fixed point (hw_fixed.h), from four
-// records of node_record_fixed. Returns false, with out unspecified, when an operand does not fit.
-template <int DIR, bool CHAR>
+// records of node_record_fixed. Returns false, with out unspecified, when an operand does not fit. PAIR: the lanes 2k
+// and 2k + 1 share one interface, each forms the side of its lowest bit, and both return the result (the sums over the
+// sides are of integers, so it is the same).
+template <int DIR, bool CHAR, bool PAIR = false>
 __device__ __forceinline__ bool interface_values_fixed(const double* r0, const double* r1, const double* r2,
                                                        const double* r3, int stride, const double qb[6],
                                                        const Dev2D& d, double out[12]) {
@@ -342,8 +344,9 @@ __device__ __forceinline__ bool interface_values_fixed(const double* r0, const d
   auto quintic = [](const int64_t f[3], const int64_t p[3]) {
     return 3 * ((f[0] - f[1]) - 7 * (f[1] - f[2])) + (p[0] - 2 * p[1] - 5 * p[2]);
   };
+  const int own = PAIR ? (int)(threadIdx.x & 1) : 0;
 #pragma unroll 1
-  for (int side = 1; side >= 0; --side) {
+  for (int side = PAIR ? own : 1; side >= own; --side) {
     // '+': nodes 0, 1, 2 of (F+, G+); '-': nodes 3, 2, 1 of (F-, -G-)
     const double* const q = side == 0 ? r0 : r3 + R_FM * stride;
     const int step = side == 0 ? (int)(r1 - r0) : -(int)(r1 - r0);
@@ -408,6 +411,20 @@ __device__ __forceinline__ bool interface_values_fixed(const double* r0, const d
         }
       }
     }
+  }
+  if constexpr (PAIR) {
+    const unsigned pair = 3u << (threadIdx.x & 30);
+    auto other = [&](int64_t x) { return (int64_t)__shfl_xor_sync(pair, (long long)x, 1); };
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      G[k] += other(G[k]);
+      if (k < 2 || !CHAR) {
+        const int64_t q = other(Q[k]);
+        Q[k] = own == 0 ? Q[k] - q : q - Q[k];
+      }
+    }
+    BA += other(BA);
+    BD += other(BD);
   }
   // back to physical components: G carries a factor 6, BA and BD (the sums over fields 1 and 3 of -+ and of
   // the source values) a factor 1/2
@@ -801,96 +818,119 @@ __device__ __noinline__ void limit_node_fallback(const S src, int i, int j, size
 // copy of the code for both directions, each with its own loads and units: with both directions' 27 values loaded
 // first the node kernel spilled 380 bytes a thread at 80 registers, whose write-back was half of its DRAM writes (now about 90 bytes; a
 // job of two steps at 2048^2 15.97 -> 15.55 ms).
-// False (mod unspecified) when an operand does not fit.
+// False (out unspecified) when an operand does not fit.
+struct LimitNode {  // the node's velocities, g h, 1/sqrt(g h) and the weights' epsilons
+  double u, v, gh, rs;
+  FxEps eps2, eps13;
+  bool bad;
+  template <bool CHAR>
+  __device__ __forceinline__ void form(const Dev2D& d, double b, const double cur[9]) {
+    bad = false;
+    const double h = cur[0] - b;
+    gh = d.g * h;
+    const double rh = fast_rcp(h);
+    u = cur[1] * rh;
+    v = cur[2] * rh;
+    rs = fast_rsqrt(gh);
+    eps2 = fx_eps(d.fx_eps2l, bad);
+    eps13 = CHAR ? fx_eps(d.fx_eps13l * h, bad) : eps2;
+  }
+};
+
+// out: mass, normal, tangential.
+template <bool CHAR, bool COH>
+__device__ __forceinline__ bool limit_dir_fixed(const Dev2D& d, int i, int j, size_t on, const double cur[9], const LimitNode& L,
+                                                int dir, double out[3]) {
+  const double u = L.u, v = L.v, gh = L.gh, rs = L.rs;
+  const FxEps eps2 = L.eps2, eps13 = L.eps13;
+  bool bad = L.bad;
+  // planes of (mass, normal, tangential) and of their derivatives along the direction; across a wall the normal
+  // component and the others' derivatives change sign
+  const double* const pu[3] = {d.S[0], dir == 0 ? d.S[1] : d.S[2], dir == 0 ? d.S[2] : d.S[1]};
+  const double* const pd[3] = {dir == 0 ? d.S[3] : d.S[6], dir == 0 ? d.S[4] : d.S[8], dir == 0 ? d.S[5] : d.S[7]};
+  double U[3][3], D[2][3];
+  U[0][0] = cur[0];
+  U[0][1] = dir == 0 ? cur[1] : cur[2];
+  U[0][2] = dir == 0 ? cur[2] : cur[1];
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    bool fx, fy;
+    const int ii = map_index(dir == 0 ? i - 1 + 2 * s : i, d.nx, d.bc_x, fx);
+    const int jj = map_index(dir == 0 ? j : j - 1 + 2 * s, d.ny, d.bc_y, fy);
+    const size_t o = on + (size_t)jj * d.nx + ii;
+    const uint32_t m = (dir == 0 ? fx : fy) ? 0x80000000u : 0u;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      U[s + 1][c] = flip_sign(ldp<COH>(pu[c] + o), c == 1 ? m : 0u);
+      D[s][c] = flip_sign(ldp<COH>(pd[c] + o), c == 1 ? 0u : m);
+    }
+  }
+  int em[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const uint32_t w = max(max(max(fx_absw(U[0][c]), fx_absw(U[1][c])), fx_absw(U[2][c])), max(fx_absw(D[0][c]), fx_absw(D[1][c])));
+    const uint32_t any = fx_any(U[0][c]) | fx_any(U[1][c]) | fx_any(U[2][c]) | fx_any(D[0][c]) | fx_any(D[1][c]);
+    em[c] = (int)(w >> 20);
+    bad |= (em[c] > kFxExpMax) | ((em[c] < kFxExpMin) & (any != 0u));
+    em[c] = max(em[c], kFxExpMin);
+  }
+  if (bad) return false;
+  // differences to the two neighbours and their derivatives, below 2^61
+  int64_t a[4][3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int64_t c0 = fx_from_double(U[0][c], em[c]);
+    a[0][c] = c0 - fx_from_double(U[1][c], em[c]);
+    a[1][c] = fx_from_double(U[2][c], em[c]) - c0;
+    a[2][c] = fx_from_double(D[0][c], em[c]);
+    a[3][c] = fx_from_double(D[1][c], em[c]);
+  }
+  if (CHAR) {
+    // rows (-(un + c), 1, 0), (-ut, 0, 1), (-(un - c), 1, 0) on (mass, normal, tangential)
+    const double un = dir == 0 ? u : v, ut = dir == 0 ? v : u;
+    const double upc = fma(gh, rs, un), umc = fma(-gh, rs, un);
+    int up, um, uv;
+    const int64_t xp = fx_mantissa(-upc, up), xm = fx_mantissa(-umc, um), xv = fx_mantissa(-ut, uv);
+    const int u0 = em[0] - 1082 + 64;
+    const int U02 = max(max(max(up, um) + u0 + 2, em[1] - 1078), -900), U1 = max(max(uv + u0 + 2, em[2] - 1078), -900);
+    if (max(U02, U1) > 900) return false;
+    const FxS kp = fx_split(xp >> min(U02 - up - u0, 63)), km = fx_split(xm >> min(U02 - um - u0, 63)),
+              kv = fx_split(xv >> min(U1 - uv - u0, 63));
+    const int sn = min(U02 + 1082 - em[1], 63), st = min(U1 + 1082 - em[2], 63);
+    int64_t nu[3];
+    FxS x[4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) x[s] = fx_split(a[s][0]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const FxS kk = k == 0 ? kp : k == 1 ? kv : km;
+      int64_t f[4];
+#pragma unroll
+      for (int s = 0; s < 4; ++s) f[s] = fx_mulhi(x[s], kk, k == 1 ? a[s][2] >> st : a[s][1] >> sn);
+      nu[k] = fx_limiter_field(f[0], f[1], f[2], f[3], k == 1 ? eps2 : eps13, k == 1 ? U1 : U02);
+    }
+    const double A = fx_to_double(nu[2] - nu[0], U02 - 1) * (0.5 * rs);
+    out[0] = A;
+    out[1] = fma(un, A, fx_to_double(nu[2] + nu[0], U02 - 2));
+    out[2] = fma(ut, A, fx_to_double(nu[1], U1 - 1));
+  } else {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      out[c] = fx_to_double(fx_limiter_field(a[0][c] >> 3, a[1][c] >> 3, a[2][c] >> 3, a[3][c] >> 3, eps2, em[c] - 1079),
+                            em[c] - 1080);
+  }
+  return true;
+}
+
 template <bool CHAR, bool COH>
 __device__ __forceinline__ bool limit_node_fixed(const Dev2D& d, int i, int j, size_t on, const double cur[9],
                                                  double mod[6]) {
-  bool bad = false;
-  const double h = cur[0] - __ldg(d.stat[0] + on + (size_t)j * d.nx + i);
-  const double gh = d.g * h;
-  const double rh = fast_rcp(h);
-  const double u = cur[1] * rh, v = cur[2] * rh;
-  const double rs = fast_rsqrt(gh);
-  const FxEps eps2 = fx_eps(d.fx_eps2l, bad);
-  const FxEps eps13 = CHAR ? fx_eps(d.fx_eps13l * h, bad) : eps2;
+  LimitNode L;
+  L.form<CHAR>(d, __ldg(d.stat[0] + on + (size_t)j * d.nx + i), cur);
 #pragma unroll 1
   for (int dir = 0; dir < 2; ++dir) {
-    // planes of (mass, normal, tangential) and of their derivatives along the direction; across a wall the normal
-    // component and the others' derivatives change sign
-    const double* const pu[3] = {d.S[0], dir == 0 ? d.S[1] : d.S[2], dir == 0 ? d.S[2] : d.S[1]};
-    const double* const pd[3] = {dir == 0 ? d.S[3] : d.S[6], dir == 0 ? d.S[4] : d.S[8], dir == 0 ? d.S[5] : d.S[7]};
-    double U[3][3], D[2][3];
-    U[0][0] = cur[0];
-    U[0][1] = dir == 0 ? cur[1] : cur[2];
-    U[0][2] = dir == 0 ? cur[2] : cur[1];
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      bool fx, fy;
-      const int ii = map_index(dir == 0 ? i - 1 + 2 * s : i, d.nx, d.bc_x, fx);
-      const int jj = map_index(dir == 0 ? j : j - 1 + 2 * s, d.ny, d.bc_y, fy);
-      const size_t o = on + (size_t)jj * d.nx + ii;
-      const uint32_t m = (dir == 0 ? fx : fy) ? 0x80000000u : 0u;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        U[s + 1][c] = flip_sign(ldp<COH>(pu[c] + o), c == 1 ? m : 0u);
-        D[s][c] = flip_sign(ldp<COH>(pd[c] + o), c == 1 ? 0u : m);
-      }
-    }
-    int em[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const uint32_t w = max(max(max(fx_absw(U[0][c]), fx_absw(U[1][c])), fx_absw(U[2][c])), max(fx_absw(D[0][c]), fx_absw(D[1][c])));
-      const uint32_t any = fx_any(U[0][c]) | fx_any(U[1][c]) | fx_any(U[2][c]) | fx_any(D[0][c]) | fx_any(D[1][c]);
-      em[c] = (int)(w >> 20);
-      bad |= (em[c] > kFxExpMax) | ((em[c] < kFxExpMin) & (any != 0u));
-      em[c] = max(em[c], kFxExpMin);
-    }
-    if (bad) return false;
-    // differences to the two neighbours and their derivatives, below 2^61
-    int64_t a[4][3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int64_t c0 = fx_from_double(U[0][c], em[c]);
-      a[0][c] = c0 - fx_from_double(U[1][c], em[c]);
-      a[1][c] = fx_from_double(U[2][c], em[c]) - c0;
-      a[2][c] = fx_from_double(D[0][c], em[c]);
-      a[3][c] = fx_from_double(D[1][c], em[c]);
-    }
     double out[3];
-    if (CHAR) {
-      // rows (-(un + c), 1, 0), (-ut, 0, 1), (-(un - c), 1, 0) on (mass, normal, tangential)
-      const double un = dir == 0 ? u : v, ut = dir == 0 ? v : u;
-      const double upc = fma(gh, rs, un), umc = fma(-gh, rs, un);
-      int up, um, uv;
-      const int64_t xp = fx_mantissa(-upc, up), xm = fx_mantissa(-umc, um), xv = fx_mantissa(-ut, uv);
-      const int u0 = em[0] - 1082 + 64;
-      const int U02 = max(max(max(up, um) + u0 + 2, em[1] - 1078), -900), U1 = max(max(uv + u0 + 2, em[2] - 1078), -900);
-      if (max(U02, U1) > 900) return false;
-      const FxS kp = fx_split(xp >> min(U02 - up - u0, 63)), km = fx_split(xm >> min(U02 - um - u0, 63)),
-                kv = fx_split(xv >> min(U1 - uv - u0, 63));
-      const int sn = min(U02 + 1082 - em[1], 63), st = min(U1 + 1082 - em[2], 63);
-      int64_t nu[3];
-      FxS x[4];
-#pragma unroll
-      for (int s = 0; s < 4; ++s) x[s] = fx_split(a[s][0]);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const FxS kk = k == 0 ? kp : k == 1 ? kv : km;
-        int64_t f[4];
-#pragma unroll
-        for (int s = 0; s < 4; ++s) f[s] = fx_mulhi(x[s], kk, k == 1 ? a[s][2] >> st : a[s][1] >> sn);
-        nu[k] = fx_limiter_field(f[0], f[1], f[2], f[3], k == 1 ? eps2 : eps13, k == 1 ? U1 : U02);
-      }
-      const double A = fx_to_double(nu[2] - nu[0], U02 - 1) * (0.5 * rs);
-      out[0] = A;
-      out[1] = fma(un, A, fx_to_double(nu[2] + nu[0], U02 - 2));
-      out[2] = fma(ut, A, fx_to_double(nu[1], U1 - 1));
-    } else {
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        out[c] = fx_to_double(fx_limiter_field(a[0][c] >> 3, a[1][c] >> 3, a[2][c] >> 3, a[3][c] >> 3, eps2, em[c] - 1079),
-                              em[c] - 1080);
-    }
+    if (!limit_dir_fixed<CHAR, COH>(d, i, j, on, cur, L, dir, out)) return false;
     if (dir == 0) {
       mod[0] = out[0]; mod[1] = out[1]; mod[2] = out[2];
     } else {
@@ -914,43 +954,15 @@ struct PlaneFaces {
   __device__ __forceinline__ R y(int q) const { return ldp<COH>(d.Y[q] + oy + d.nx) - ldp<COH>(d.Y[q] + oy); }
 };
 
-// RHS assembly, limiter and RK combination (or the bare RHS) at node (i, j) of one grid, read through faces. FIXED: the limiter in fixed point where the node's data fits it. on: offset of the grid in pooled
-// node planes (0 for one grid). COH: loads of the state and base planes as in ldp.
-template <int MODE, bool LINEAR, bool CHAR, bool FIXED, bool COH, class S, class R, class Faces>
-__device__ __forceinline__ void node_update_faces(const Dev2DT<R>& d, const S src, const StageArgsT<R>& sa, int i, int j, size_t on,
-                                                  const Faces& faces) {
-  const size_t o = on + (size_t)j * d.nx + i;
-  R cur[9];
-#pragma unroll
-  for (int q = 0; q < 9; ++q) cur[q] = faces.state(q);
-  if (MODE == MODE_STAGE && !(*sa.dt > 0.0)) {
-    // a step of size 0 (e.g. clipped at the end time) leaves the state unchanged
-#pragma unroll
-    for (int q = 0; q < 9; ++q) sa.out[q][o] = cur[q];
-    return;
-  }
-  // ---- limiter (Sec. R(2.2), dimension by dimension) ----
-  R mod[6];
-  if (MODE == MODE_STAGE) {
-    if (sa.limiter) {
-      if constexpr (FIXED && !LINEAR && std::is_same<R, double>::value) {
-        if (!limit_node_fixed<CHAR, COH>(d, i, j, on, cur, mod)) limit_node_fallback<CHAR, COH>(src, i, j, on, cur, mod);
-      } else {
-        limit_node<LINEAR, CHAR>(d, faces.bottom(), cur, mod, [&](int di, int dj, Node12T<R>& n) { faces.neighbour(di, dj, n); });
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < 6; ++q) mod[q] = cur[3 + q];
-    }
-  }
-  // ---- RHS (eq. swe-form-2d-dis) in scaled units: R_U, dx R_V, dy R_Q ----
+// RHS (eq. swe-form-2d-dis) in scaled units: R_U, dx R_V, dy R_Q, of node o with state cur.
+template <class R, class Faces>
+__device__ __forceinline__ void right_hand_side(const Dev2DT<R>& d, size_t o, const R cur[9], const Faces& faces, R Rv[9]) {
   // In double: of the negative, whose 50 operations bound this part (64 with the factors applied here, 3 more per node in
   // the RK combination; node kernel at 2048^2 1.04 -> 0.94 ms, the sweeps within 2% of what they were).
   const R eta = cur[0], H1 = cur[3], H2 = cur[6];
   const R g = R(d.g);
   const R c_mx = R(d.c_mx), c_my = R(d.c_my);
   const R ge = g * eta;
-  R Rv[9];
   if constexpr (std::is_same<R, double>::value) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -983,6 +995,39 @@ __device__ __forceinline__ void node_update_faces(const Dev2DT<R>& d, const S sr
       Rv[6 + c] = fma(-(g * H2), db, rq);
     }
   }
+}
+
+// RHS assembly, limiter and RK combination (or the bare RHS) at node (i, j) of one grid, read through faces. FIXED: the limiter in fixed point where the node's data fits it. on: offset of the grid in pooled
+// node planes (0 for one grid). COH: loads of the state and base planes as in ldp.
+template <int MODE, bool LINEAR, bool CHAR, bool FIXED, bool COH, class S, class R, class Faces>
+__device__ __forceinline__ void node_update_faces(const Dev2DT<R>& d, const S src, const StageArgsT<R>& sa, int i, int j, size_t on,
+                                                  const Faces& faces) {
+  const size_t o = on + (size_t)j * d.nx + i;
+  R cur[9];
+#pragma unroll
+  for (int q = 0; q < 9; ++q) cur[q] = faces.state(q);
+  if (MODE == MODE_STAGE && !(*sa.dt > 0.0)) {
+    // a step of size 0 (e.g. clipped at the end time) leaves the state unchanged
+#pragma unroll
+    for (int q = 0; q < 9; ++q) sa.out[q][o] = cur[q];
+    return;
+  }
+  // ---- limiter (Sec. R(2.2), dimension by dimension) ----
+  R mod[6];
+  if (MODE == MODE_STAGE) {
+    if (sa.limiter) {
+      if constexpr (FIXED && !LINEAR && std::is_same<R, double>::value) {
+        if (!limit_node_fixed<CHAR, COH>(d, i, j, on, cur, mod)) limit_node_fallback<CHAR, COH>(src, i, j, on, cur, mod);
+      } else {
+        limit_node<LINEAR, CHAR>(d, faces.bottom(), cur, mod, [&](int di, int dj, Node12T<R>& n) { faces.neighbour(di, dj, n); });
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 6; ++q) mod[q] = cur[3 + q];
+    }
+  }
+  R Rv[9];
+  right_hand_side<R>(d, o, cur, faces, Rv);
   if (MODE == MODE_RHS) {
     // physical units: R_V = (dx R_V)/dx, R_Q = (dy R_Q)/dy
 #pragma unroll
