@@ -240,6 +240,89 @@ __device__ __forceinline__ void interface_m(const double* r0, const double* r1, 
 #undef RV
 }
 
+// ---- the same interface shared out over lanes and warps (small grids), operation for operation ----
+// Eigenvectors of the interface between the records r1 and r2.
+template <int DIR>
+struct Eigen {
+  double un, ut, upc, umc, ic2, eps2, eps13;
+  template <class M>
+  __device__ __forceinline__ void form(const double* r1, const double* r2, int stride, double g, double eps_w, M& mul) {
+    const double hs = r1[R_H * stride] + r2[R_H * stride];
+    const double rhs = mul.rcp(hs);
+    const double ub = mul(r1[R_M * stride] + r2[R_M * stride], rhs);
+    const double vb = mul(r1[R_W * stride] + r2[R_W * stride], rhs);
+    const double gh = mul(mul.k(0.5, g), hs);
+    const double rs = fast_rsqrt(gh);
+    ic2 = mul.k(0.5, rs);
+    un = DIR == 0 ? ub : vb;
+    ut = DIR == 0 ? vb : ub;
+    upc = fma(gh, rs, un);
+    umc = fma(-gh, rs, un);
+    eps2 = mul.k(4.0, eps_w);
+    eps13 = mul(mul(mul.k(8.0, g), eps_w), hs);
+  }
+};
+
+// One upwind side: q, step = its first record's split data and the way to the next (side 1 from the far end, its
+// derivatives negated by mask): the three fields' values and the source with the weights of fields 1 and 3.
+template <int DIR, class M>
+__device__ __forceinline__ void side_values(const Eigen<DIR>& E, const double* q, int step, int stride, uint32_t mask,
+                                            const double qbs[3], double v[3], double& b1, double& b3, M& mul) {
+  const int cn = DIR == 0 ? 1 : 2, ct = DIR == 0 ? 2 : 1;
+  double f[3][3], p[3][3];
+#pragma unroll
+  for (int t = 0; t < 3; ++t) {
+    const double* r = q + t * step;
+    const double F0 = r[0], Fn = r[cn * stride], Ft = r[ct * stride];
+    const double G0 = flip_sign(r[R_GP * stride], mask), Gn = flip_sign(r[(R_GP + cn) * stride], mask),
+                 Gt = flip_sign(r[(R_GP + ct) * stride], mask);
+    f[0][t] = fma(E.upc, F0, -Fn);
+    f[1][t] = fma(-E.ut, F0, Ft);
+    f[2][t] = fma(-E.umc, F0, Fn);
+    p[0][t] = fma(E.upc, G0, -Gn);
+    p[1][t] = fma(-E.ut, G0, Gt);
+    p[2][t] = fma(-E.umc, G0, Gn);
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    WeightsT W;
+    v[k] = side_value(f[k][0], f[k][1], f[k][2], p[k][0], p[k][1], p[k][2], k == 1 ? E.eps2 : E.eps13, W, mul);
+    if (k == 0) b1 = weighted_value(W, qbs[0], qbs[1], qbs[2], mul);
+    if (k == 2) b3 = weighted_value(W, qbs[0], qbs[1], qbs[2], mul);
+  }
+}
+
+// Back to physical components from the sums over both sides: the first six interface values.
+template <int DIR, class M>
+__device__ __forceinline__ void back_values(const Eigen<DIR>& E, const double G[3], double GB1, double GB3, double out[6], M& mul) {
+  const int cn = DIR == 0 ? 1 : 2, ct = DIR == 0 ? 2 : 1;
+  const double A = mul(G[0] + G[2], E.ic2);
+  out[0] = A;
+  out[cn] = fma(E.un, A, mul.k(0.5, G[2] - G[0]));
+  out[ct] = fma(E.ut, A, G[1]);
+  const double Bs = mul(GB1 + GB3, E.ic2);
+  out[3] = Bs;
+  out[3 + cn] = fma(E.un, Bs, mul.k(0.5, GB3 - GB1));
+  out[3 + ct] = mul(E.ut, Bs);
+}
+
+// The derivative flux and the mixed term: the other six.
+__device__ __forceinline__ void linear_values(const double* r0, int sstep, int stride, double out[6]) {
+  const double *r1 = r0 + sstep, *r2 = r1 + sstep, *r3 = r2 + sstep;
+#define RV(r, f) (r)[(f) * stride]
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double fpart =
+        fma(7.0, RV(r2, R_FP + c) - RV(r1, R_FM + c),
+            fma(8.0, RV(r2, R_FM + c) - RV(r1, R_FP + c), RV(r0, R_FP + c) - RV(r3, R_FM + c)));
+    const double gpart = fma(-5.0, RV(r2, R_GP + c) + RV(r1, R_GM + c),
+                             fma(-2.0, RV(r1, R_GP + c) + RV(r2, R_GM + c), RV(r0, R_GP + c) + RV(r3, R_GM + c)));
+    out[c] = fma(3.0, fpart, gpart);
+    out[3 + c] = fma(7.0, RV(r1, R_MIX + c) + RV(r2, R_MIX + c), -(RV(r0, R_MIX + c) + RV(r3, R_MIX + c)));
+  }
+#undef RV
+}
+
 template <int DIR, class M>
 __device__ __forceinline__ void limit_along(const double Um[3], const double U0[3], const double Up[3],
                                           const double Dm[3], const double Dp[3], double u, double v, double c,
@@ -264,27 +347,16 @@ __device__ __forceinline__ void limit_along(const double Um[3], const double U0[
   out[ct] = fma(ut, A, nu[1]);
 }
 
+// RHS (eq. swe-form-2d-dis) in scaled units: R_U, dx R_V, dy R_Q, of the node at o with the left x-interface ox and
+// the lower y-interface oy.
 template <class M>
-__device__ __forceinline__ void node_update_m(const Dev2D& d, const StageArgs& sa, int i, int j, M& mul) {
-  const size_t o = (size_t)j * d.nx + i;
-  const size_t ox = (size_t)j * (d.nx + 1) + i;  // left x-interface; right is ox + 1
-  const size_t oy = (size_t)j * d.nx + i;             // lower y-interface; upper is oy + nx
-  double cur[9];
-#pragma unroll
-  for (int q = 0; q < 9; ++q) cur[q] = __ldg(d.S[q] + o);
-  if (!(*sa.dt > 0.0)) {
-    // a step of size 0 (e.g. clipped at the end time) leaves the state unchanged
-#pragma unroll
-    for (int q = 0; q < 9; ++q) sa.out[q][o] = cur[q];
-    return;
-  }
+__device__ __forceinline__ void right_hand_side(const Dev2D& d, const double cur[9], size_t o, size_t ox, size_t oy, double Rv[9],
+                                                M& mul) {
   const double eta = cur[0], H1 = cur[3], H2 = cur[6];
   const double g = d.g;
   const double c_bx = d.c_bx, c_by = d.c_by, c_gx = d.c_gx, c_gy = d.c_gy, c_mx = d.c_mx,
           c_my = d.c_my;
   const double ge = mul(g, eta);
-  // ---- RHS (eq. swe-form-2d-dis) in scaled units: R_U, dx R_V, dy R_Q ----
-  double Rv[9];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const double dFx = __ldg(d.X[c] + ox + 1) - __ldg(d.X[c] + ox);
@@ -306,16 +378,44 @@ __device__ __forceinline__ void node_update_m(const Dev2D& d, const StageArgs& s
     Rv[3 + c] = fma(-mul(g, H1), db, rv);
     Rv[6 + c] = fma(-mul(g, H2), db, rq);
   }
+}
+
+// The node's velocities, wave speed c, 1/(2c) and g h.
+template <class M>
+__device__ __forceinline__ void node_speeds(const Dev2D& d, const double cur[9], size_t o, double& u, double& v, double& c,
+                                            double& ic2, double& gh, M& mul) {
+  const double b0 = __ldg(d.stat[0] + o);
+  const double h = cur[0] - b0;
+  gh = mul(d.g, h);
+  const double rh = mul.rcp(h);
+  u = mul(cur[1], rh);
+  v = mul(cur[2], rh);
+  const double rs = fast_rsqrt(gh);
+  c = mul(gh, rs);
+  ic2 = mul.k(0.5, rs);
+}
+
+template <class M>
+__device__ __forceinline__ void node_update_m(const Dev2D& d, const StageArgs& sa, int i, int j, M& mul) {
+  const size_t o = (size_t)j * d.nx + i;
+  const size_t ox = (size_t)j * (d.nx + 1) + i;  // left x-interface; right is ox + 1
+  const size_t oy = (size_t)j * d.nx + i;             // lower y-interface; upper is oy + nx
+  double cur[9];
+#pragma unroll
+  for (int q = 0; q < 9; ++q) cur[q] = __ldg(d.S[q] + o);
+  if (!(*sa.dt > 0.0)) {
+    // a step of size 0 (e.g. clipped at the end time) leaves the state unchanged
+#pragma unroll
+    for (int q = 0; q < 9; ++q) sa.out[q][o] = cur[q];
+    return;
+  }
+  double Rv[9];
+  right_hand_side(d, cur, o, ox, oy, Rv, mul);
   // ---- limiter (Sec. 2.2, dimension by dimension) ----
   double mod[6];
   if (sa.limiter) {
-    const double b0 = __ldg(d.stat[0] + o);
-    const double h = eta - b0;
-    const double gh = mul(g, h);
-    const double rh = mul.rcp(h);
-    const double u = mul(cur[1], rh), v = mul(cur[2], rh);
-    const double rs = fast_rsqrt(gh);
-    const double c = mul(gh, rs), ic2 = mul.k(0.5, rs);
+    double u, v, c, ic2, gh;
+    node_speeds(d, cur, o, u, v, c, ic2, gh, mul);
     Node12 nm, np;
     // x neighbours
     load_node(d, i - 1, j, nm);
@@ -419,6 +519,185 @@ __global__ void __launch_bounds__(FT, 3) k_sweeps_fp64(Dev2D d, const double* __
   }
 }
 
+// The same for small grids, where a tile's time is one warp's chain of dependent operations: SR - 3 x-interfaces per tile, each
+// side a lane's (pairs of lanes exchange their sums), the derivative flux and the mixed term other warps': 60 -> 39 us a
+// stage at 150 x 97. The sums keep their order, so the values are those of k_sweeps_fp64 bit for bit.
+constexpr int SR = 64, ST = 3 * SR;  // records and threads per tile
+
+template <int DIR>
+__device__ __forceinline__ void sweep_split(const Dev2D& d, const double* sm, int rs, int u, bool valid, size_t o) {
+  // u: the interface's first record; rs: records to the next one of its line
+  double* const* P = DIR == 0 ? d.X : d.Y;
+  if (threadIdx.x < 2 * SR) {
+    const int side = threadIdx.x & 1;
+    double v[3] = {}, b1 = 0.0, b3 = 0.0, qbs[3];
+    Int<false> mi;
+    const double* r0 = sm + u;
+    Eigen<DIR> E{};
+    if (valid) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) qbs[q] = __ldg((DIR == 0 ? d.qbx : d.qby)[3 * side + q] + o);
+      E.form(r0 + rs, r0 + 2 * rs, SR, d.g, d.eps_w, mi);
+      side_values<DIR>(E, side ? r0 + 3 * rs + R_FM * SR : r0, side ? -rs : rs, SR, side ? 0x80000000u : 0u, qbs, v, b1, b3, mi);
+    }
+    double w[3], c1, c3;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) w[k] = __shfl_xor_sync(0xffffffffu, v[k], 1);
+    c1 = __shfl_xor_sync(0xffffffffu, b1, 1);
+    c3 = __shfl_xor_sync(0xffffffffu, b3, 1);
+    bool bad = mi.bad;
+    bad |= __shfl_xor_sync(0xffffffffu, (int)bad, 1) != 0;
+    if (valid && side == 0) {
+      double out[12];
+      if (!bad) {
+        const double G[3] = {v[0] + w[0], v[1] + w[1], v[2] + w[2]};
+        const double GB1 = (0.0 - b1) - c1, GB3 = (0.0 + b3) + c3;
+        back_values<DIR>(E, G, GB1, GB3, out, mi);
+        bad = mi.bad;
+      }
+      if (bad) {
+        double qb[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) qb[q] = __ldg((DIR == 0 ? d.qbx : d.qby)[q] + o);
+        Fp64 mf;
+        interface_m<DIR>(r0, r0 + rs, r0 + 2 * rs, r0 + 3 * rs, SR, qb, d.g, d.eps_w, out, mf);
+      }
+#pragma unroll
+      for (int q = 0; q < 6; ++q) P[q][o] = out[q];
+    }
+  } else if (valid) {
+    double out[6];
+    linear_values(sm + u, rs, SR, out);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) P[6 + q][o] = out[q];
+  }
+}
+
+__global__ void __launch_bounds__(ST, 2) k_sweeps_fp64_split(const __grid_constant__ Dev2D d, const double* __restrict__ alpha,
+                                                             unsigned nxt) {
+  __shared__ double sm[NREC * SR];
+  const int t = threadIdx.x, u = t < 2 * SR ? t >> 1 : t - 2 * SR;  // the thread's interface
+  Fp64 mf;
+  if (blockIdx.x < nxt) {
+    const unsigned W = d.nx + 4, total = (unsigned)d.ny * W, E0 = blockIdx.x * (SR - 3);
+    if (t < SR && E0 + t < total) {
+      const unsigned j = (E0 + t) / W;
+      Node12 n;
+      load_node(d, (int)(E0 + t - j * W) - 2, (int)j, n);
+      double rec[NREC];
+      record<0>(n, d.g, alpha[0], rec, mf);
+#pragma unroll
+      for (int f = 0; f < NREC; ++f) sm[f * SR + t] = rec[f];
+    }
+    __syncthreads();
+    const unsigned E = E0 + u, j = E / W, e = E - j * W;
+    sweep_split<0>(d, sm, 1, u, u < SR - 3 && E < total && e <= (unsigned)d.nx, (size_t)j * (d.nx + 1) + e);
+  } else {
+    constexpr int yc = 2, ifs = SR / yc - 3;
+    const unsigned H = d.ny + 4, total = (unsigned)((d.nx + yc - 1) / yc) * H, E0 = (blockIdx.x - nxt) * ifs;
+    if (t < SR) {
+      const unsigned E = E0 + t / yc, g = E / H;
+      const int i = (int)g * yc + t % yc;
+      if (E < total && i < d.nx) {
+        Node12 n;
+        load_node(d, i, (int)(E - g * H) - 2, n);
+        double rec[NREC];
+        record<1>(n, d.g, alpha[1], rec, mf);
+#pragma unroll
+        for (int f = 0; f < NREC; ++f) sm[f * SR + t] = rec[f];
+      }
+    }
+    __syncthreads();
+    const unsigned E = E0 + u / yc, g = E / H, e = E - g * H;
+    const int i = (int)g * yc + u % yc;
+    sweep_split<1>(d, sm, yc, u, u / yc < ifs && E < total && e <= (unsigned)d.ny && i < d.nx, (size_t)e * d.nx + i);
+  }
+}
+
+// The node update of small grids: 64 nodes a block, their right-hand sides, x-limiters and y-limiters two warps' each, the
+// RK combination of three planes likewise: 46 -> 30 us a stage at 150 x 97, the values those of k_node_fp64.
+__global__ void __launch_bounds__(192, 3) k_node_fp64_split(const __grid_constant__ Dev2D d, StageArgs sa) {
+  __shared__ double s_mod[6 * 64], s_R[9 * 64];
+  __shared__ int s_bad[64];
+  const int t = threadIdx.x & 63, role = threadIdx.x >> 6;
+  if (sa.nsteps && blockIdx.x == 0 && threadIdx.x == 0) {
+    *sa.t = sa.snapped ? sa.clock[1] : *sa.t + sa.clock[0];
+    if (sa.clock[0] > 0.0) ++*sa.nsteps;
+  }
+  const unsigned o = blockIdx.x * 64 + t;
+  const int j = (int)(o / (unsigned)d.nx), i = (int)(o - (unsigned)j * d.nx);
+  const bool in = j < d.ny;
+  if (!(*sa.dt > 0.0)) {  // a step of size 0
+    if (in)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) sa.out[3 * role + q][o] = __ldg(d.S[3 * role + q] + o);
+    return;
+  }
+  if (role == 0) s_bad[t] = 0;
+  __syncthreads();
+  Int<true> mi;
+  if (in) {
+    double cur[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) cur[q] = __ldg(d.S[q] + o);
+    if (role == 0) {
+      double Rv[9];
+      right_hand_side(d, cur, o, (size_t)j * (d.nx + 1) + i, o, Rv, mi);
+#pragma unroll
+      for (int q = 0; q < 9; ++q) s_R[q * 64 + t] = Rv[q];
+    } else {
+      double mod[3];
+      if (sa.limiter) {
+        double u, v, c, ic2, gh;
+        node_speeds(d, cur, o, u, v, c, ic2, gh, mi);
+        Node12 nm, np;
+        if (role == 1) {
+          load_node(d, i - 1, j, nm);
+          load_node(d, i + 1, j, np);
+          limit_along<0>(nm.v, cur, np.v, nm.v + 3, np.v + 3, u, v, c, ic2, gh, d.eps_lim, mod, mi);
+        } else {
+          load_node(d, i, j - 1, nm);
+          load_node(d, i, j + 1, np);
+          limit_along<1>(nm.v, cur, np.v, nm.v + 6, np.v + 6, u, v, c, ic2, gh, d.eps_lim, mod, mi);
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) mod[q] = role == 1 ? cur[3 + q] : cur[6 + q];
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) s_mod[(3 * (role - 1) + q) * 64 + t] = mod[q];
+    }
+    if (mi.bad) s_bad[t] = 1;
+  }
+  __syncthreads();
+  double cq[3], res[3];
+  if (in) {
+    const double dt = *sa.dt, a = sa.k == 2 ? 0.75 : 1.0 / 3.0, b = sa.k == 2 ? 0.25 : 2.0 / 3.0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const double R = s_R[(3 * role + q) * 64 + t];
+      cq[q] = role == 0 ? __ldg(d.S[q] + o) : s_mod[(3 * (role - 1) + q) * 64 + t];
+      res[q] = fma(dt, R, cq[q]);
+      if (sa.k != 1) res[q] = fma(a, __ldg(sa.base[3 * role + q] + o), mi(b, res[q]));
+    }
+    if (mi.bad) s_bad[t] = 1;
+  }
+  __syncthreads();
+  if (!in) return;
+  if (s_bad[t]) {
+    if (role == 0) {
+      Fp64 mf;
+      node_update_m(d, sa, i, j, mf);
+    }
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (sa.k == 1 && sa.base) sa.base[3 * role + q][o] = cq[q];
+    sa.out[3 * role + q][o] = res[q];
+  }
+}
+
 template <int T>
 __global__ void __launch_bounds__(T, T == 256 ? 3 : 8) k_node_fp64(Dev2D d, StageArgs sa) {
   const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * (T / 32) + threadIdx.y;
@@ -437,12 +716,21 @@ __global__ void __launch_bounds__(T, T == 256 ? 3 : 8) k_node_fp64(Dev2D d, Stag
 
 }  // namespace
 
+// Nodes up to which the sweeps are split over lanes and warps, and the node update is: the split sweeps are the faster form as
+// long as the tiles fill the GPU a few times at most (129 against 141 us a stage at 256^2, 39 against 60 at 150 x 97), the
+// split node update while its blocks are resident at once (59 against 51 us at 256^2, 30 against 46 at 150 x 97).
+constexpr size_t kSweepSplitMax = (size_t)152 * 16 * 32, kNodeSplitMax = (size_t)152 * 3 * 64;
+
 void launch_stage_fp64(const Dev2D& d, const StageArgs& sa, const double* alpha, cudaStream_t st) {
-  constexpr int IX = FT - 3, IY = FT / 2 - 3;
+  const size_t n = (size_t)d.nx * d.ny;
+  const bool split = n <= kSweepSplitMax;
+  const int IX = (split ? SR : FT) - 3, IY = (split ? SR : FT) / 2 - 3;
   const unsigned long long nxt = ((unsigned long long)d.ny * (d.nx + 4) + IX - 1) / IX;
   const unsigned long long nyt = ((unsigned long long)((d.nx + 1) / 2) * (d.ny + 4) + IY - 1) / IY;
-  k_sweeps_fp64<<<(unsigned)(nxt + nyt), FT, 0, st>>>(d, alpha, (unsigned)nxt);
-  if ((size_t)d.nx * d.ny <= (size_t)152 * 16 * 32)
+  if (split) k_sweeps_fp64_split<<<(unsigned)(nxt + nyt), ST, 0, st>>>(d, alpha, (unsigned)nxt);
+  else k_sweeps_fp64<<<(unsigned)(nxt + nyt), FT, 0, st>>>(d, alpha, (unsigned)nxt);
+  if (n <= kNodeSplitMax) k_node_fp64_split<<<(unsigned)((n + 63) / 64), 192, 0, st>>>(d, sa);
+  else if (n <= (size_t)152 * 16 * 32)
     k_node_fp64<64><<<dim3((d.nx + 31) / 32, (d.ny + 1) / 2), dim3(32, 2), 0, st>>>(d, sa);
   else
     k_node_fp64<256><<<dim3((d.nx + 31) / 32, (d.ny + 7) / 8), dim3(32, 8), 0, st>>>(d, sa);
