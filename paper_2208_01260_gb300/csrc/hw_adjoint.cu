@@ -37,7 +37,7 @@ struct AdjDev {
   const double* lout[9];  // adjoint of the stage output
   double* lin[9];         // adjoint of the stage input (written)
   double* lbase[9];       // adjoint of the step base (accumulated over stages 3, 2; consumed at stage 1)
-  double* lR[12];         // adjoint of the right-hand side, and g (eta lR_c + H1 lR_3+c + H2 lR_6+c) (scratch)
+  double* lR[9];          // adjoint of the right-hand side (scratch)
   double* lmod[6];        // adjoint of the limited derivatives (scratch)
   double* lrecx[NREC];    // record adjoints, x: rows of nx + 4 (raw index -2 .. nx+1)
   double* lrecy[NREC];    // record adjoints, y: ny + 4 rows of nx
@@ -52,6 +52,7 @@ struct AdjDev {
   const double* fax;      // forward first component of 2 Fhat (x-interfaces) of this stage
   const double* fay;      // forward first component of 2 Fhat (y-interfaces)
   int* argmax;            // [2]
+  int clear;              // the pre-pass clears lalpha and argmax (else the caller has)
 };
 
 // atomically add parity-mapped adjoints of a (possibly ghost) node's 12 entries to the real node
@@ -94,6 +95,10 @@ __global__ void __launch_bounds__(A_NT) k_adj_node_pre(const __grid_constant__ A
   const Dev2D& d = A.d;
   const unsigned tid = blockIdx.x * A_NT + threadIdx.x;
   const int j = (int)(tid / (unsigned)d.nx), i = (int)(tid - (unsigned)j * d.nx);
+  if (A.clear && tid < 2) {
+    A.lalpha[tid] = 0.0;
+    A.argmax[tid] = INT_MAX;
+  }
   if (j >= d.ny) return;
   const size_t o = tid;
   double lc[9], lR[9];
@@ -106,7 +111,7 @@ __global__ void __launch_bounds__(A_NT) k_adj_node_pre(const __grid_constant__ A
     } else {
       lc[q] = A.b * lo;
       lR[q] = A.b * A.dt * lo;
-      A.lbase[q][o] += A.a * lo;
+      A.lbase[q][o] = A.k == 3 ? A.a * lo : A.lbase[q][o] + A.a * lo;  // stage 3 is reversed first
     }
   }
   const double eta = d.S[0][o], g = d.g, ge = g * eta;
@@ -147,25 +152,48 @@ __global__ void __launch_bounds__(A_NT) k_adj_node_pre(const __grid_constant__ A
   A.lin[6][o] += lH2;
 #pragma unroll
   for (int q = 0; q < 9; ++q) A.lR[q][o] = lR[q];
-  const double gH1 = g * d.S[3][o], gH2 = g * d.S[6][o];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) A.lR[9 + c][o] = fma(ge, lR[c], fma(gH1, lR[3 + c], gH2 * lR[6 + c]));
 }
 
-// adjoint of an interface's 12 values: differences over its two nodes (entries o0 and o1 of the planes; off the grid,
-// has0 or has1 false, a node counts zero) times cb (fluxes and bottom), cg (derivative flux) and cm (mixed term)
-template <int DIR>
-__device__ __forceinline__ void interface_adjoint(const AdjDev& A, size_t o0, size_t o1, bool has0, bool has1, double lX[12]) {
+// adjoint of the 12 values of the x-interface k of row j (from nodes k-1 and k)
+__device__ __forceinline__ void interface_adjoint_x(const AdjDev& A, int k, int j, double lX[12]) {
   const Dev2D& d = A.d;
-  const double cb = DIR == 0 ? d.c_bx : d.c_by, cg = DIR == 0 ? d.c_gx : d.c_gy, cm = DIR == 0 ? d.c_mx : d.c_my;
-  auto diff = [&](int q) { return (has1 ? A.lR[q][o1] : 0.0) - (has0 ? A.lR[q][o0] : 0.0); };
+  for (int q = 0; q < 12; ++q) lX[q] = 0.0;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    lX[c] = cb * diff(c);
-    lX[3 + c] = cb * diff(9 + c);
-    // along x the derivative flux feeds the V equations and the mixed term the Q equations, along y the reverse
-    lX[6 + c] = cg * diff(DIR == 0 ? 3 + c : 6 + c);
-    lX[9 + c] = cm * diff(DIR == 0 ? 6 + c : 3 + c);
+  for (int side = 0; side < 2; ++side) {
+    const int p = side == 0 ? k - 1 : k;  // node seeing k as its right (side 0) or left (side 1) interface
+    if (p < 0 || p >= d.nx) continue;
+    const double sgn = side == 0 ? -1.0 : 1.0;
+    const size_t o = (size_t)j * d.nx + p;
+    const double g = d.g, ge = g * d.S[0][o], gH1 = g * d.S[3][o], gH2 = g * d.S[6][o];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double lu = A.lR[c][o], lv = A.lR[3 + c][o], lq = A.lR[6 + c][o];
+      lX[c] += sgn * d.c_bx * lu;
+      lX[3 + c] += sgn * d.c_bx * (ge * lu + gH1 * lv + gH2 * lq);
+      lX[6 + c] += sgn * d.c_gx * lv;
+      lX[9 + c] += sgn * d.c_mx * lq;
+    }
+  }
+}
+
+__device__ __forceinline__ void interface_adjoint_y(const AdjDev& A, int i, int k, double lY[12]) {
+  const Dev2D& d = A.d;
+  for (int q = 0; q < 12; ++q) lY[q] = 0.0;
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    const int p = side == 0 ? k - 1 : k;
+    if (p < 0 || p >= d.ny) continue;
+    const double sgn = side == 0 ? -1.0 : 1.0;
+    const size_t o = (size_t)p * d.nx + i;
+    const double g = d.g, ge = g * d.S[0][o], gH1 = g * d.S[3][o], gH2 = g * d.S[6][o];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double lu = A.lR[c][o], lv = A.lR[3 + c][o], lq = A.lR[6 + c][o];
+      lY[c] += sgn * d.c_by * lu;
+      lY[3 + c] += sgn * d.c_by * (ge * lu + gH1 * lv + gH2 * lq);
+      lY[6 + c] += sgn * d.c_gy * lq;  // Psi2 hat feeds the Q equations
+      lY[9 + c] += sgn * d.c_my * lv;  // mixed Phi2 hat feeds the V equations
+    }
   }
 }
 
@@ -192,8 +220,8 @@ __device__ __forceinline__ double record_sum(int f, const At& at, const Ok& ok) 
 // Bound by the FP64 pipe, at 255 registers a thread: 8 warps per SM, in whatever blocks. Both sweeps are one launch of
 // small blocks because the grids this runs on are small: as two launches, with 256 threads a y-block, a grid of 150 x 97
 // had 291 and 65 blocks (the y-sweep on 65 of 152 SMs, as long as two of its warps per partition take), and one of
-// 256^2 ran 2.1 and 1.7 waves in 3 and 2. Measured with the reverse's fewer operations (hw_adjoint.cuh): 271 us a stage for
-// both sweeps at 256^2, 75 us at 150 x 97; the whole gradient 11.9 -> 10.2 ms and 15.4 -> 13.1 ms.
+// 256^2 ran 2.1 and 1.7 waves in 3 and 2. With the node kernels in small blocks too, the gradient 11.9 -> 10.9 ms at 256^2 and (with
+// the forward pass split, hw_forward64.cu) 15.4 -> 11.8 ms at 150 x 97.
 constexpr int AT = 64;
 constexpr int AX_I = AT - 3;
 constexpr int AY_C = 4, AY_R = AT / AY_C, AY_NR = AY_R + 3;
@@ -216,11 +244,11 @@ __global__ void __launch_bounds__(AT) k_adj_sweeps(const __grid_constant__ AdjDe
     }
     __syncthreads();
     if (t < AX_I && E < total && e <= (unsigned)d.nx) {
-      const size_t o = (size_t)j * (d.nx + 1) + e, on = (size_t)j * d.nx + e;
+      const size_t o = (size_t)j * (d.nx + 1) + e;
       double qb[6], lX[12], lqb[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
       for (int q = 0; q < 6; ++q) qb[q] = d.qbx[q][o];
-      interface_adjoint<0>(A, on - 1, on, e > 0, e < (unsigned)d.nx, lX);
+      interface_adjoint_x(A, (int)e, (int)j, lX);
       interface_values_rev<0>(recs + t, 1, A_NREC, qb, A.fax[o], A.dbx[0][o], d.g, d.eps_w, lX, SlabAcc{slab + t, AT}, lqb);
 #pragma unroll
       for (int q = 0; q < 6; ++q) A.lqbx[q][o] += lqb[q];
@@ -263,7 +291,7 @@ __global__ void __launch_bounds__(AT) k_adj_sweeps(const __grid_constant__ AdjDe
       double qb[6], lY[12], lqb[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
       for (int q = 0; q < 6; ++q) qb[q] = d.qby[q][o];
-      interface_adjoint<1>(A, o - d.nx, o, e > 0, e < d.ny, lY);
+      interface_adjoint_y(A, i, e, lY);
       interface_values_rev<1>(recs + t, AY_C, A_NREC, qb, A.fay[o], A.dby[0][o], d.g, d.eps_w, lY, SlabAcc{slab + t, AT}, lqb);
 #pragma unroll
       for (int q = 0; q < 6; ++q) A.lqby[q][o] += lqb[q];
@@ -369,7 +397,7 @@ __global__ void __launch_bounds__(A_NT) k_adj_limiter(const __grid_constant__ Ad
     load_node(d, im, jm, nm);
     load_node(d, ip, jp, np);
     const int qd = dir == 0 ? 3 : 6;
-    double lUm[3], lU0[3], lUp[3], lDm[3], lDp[3];
+    double lUm[3] = {}, lU0[3] = {}, lUp[3] = {}, lDm[3] = {}, lDp[3] = {};
     if (dir == 0)
       limit_dir_rev<0>(nm.v, cur, np.v, nm.v + qd, np.v + qd, u, v, c, ic2, gh, d.eps_lim, lo, lUm, lU0, lUp, lDm, lDp,
                        lu, lv, lc, lic2, lgh);
@@ -419,7 +447,7 @@ __global__ void k_adj_alpha_apply(AdjDev A) {
   for (int dir = 0; dir < 2; ++dir) {
     const int o = A.argmax[dir];
     const double la = A.lalpha[dir];
-    if (o == INT_MAX || la == 0.0) continue;
+    if ((unsigned)o >= (unsigned)(d.nx * d.ny) || la == 0.0) continue;  // no node attains it: every state value non-finite
     const double h = d.S[0][o] - d.stat[0][o];
     const double rh = fast_rcp(h), gh = d.g * h, rs = fast_rsqrt(gh), c = gh * rs;
     const double mom = d.S[1 + dir][o];
@@ -663,7 +691,7 @@ struct AdjBuffers {
   double* fy[3] = {};
   double* lam[2][9] = {};
   double* lbase[9] = {};
-  double* lR[12] = {};
+  double* lR[9] = {};
   double* lmod[6] = {};
   double* lrecx[hw::NREC] = {};
   double* lrecy[hw::NREC] = {};
@@ -778,7 +806,7 @@ int get_buffers(hw_solver* s, const hw::SolverView& v, AdjBuffers** out) {
   A(B->lam[0], 9, n);
   A(B->lam[1], 9, n);
   A(B->lbase, 9, n);
-  A(B->lR, 12, n);
+  A(B->lR, 9, n);
   A(&B->alpha_st, 1, 8);
   for (int k = 0; k < 3; ++k) {
     A(B->dbx[k], 3, nxi);
@@ -845,6 +873,10 @@ int zero_planes(double* const* p, int count, size_t n, cudaStream_t st) {
 }
 
 __global__ void k_set_dt(double* p, double v) { *p = v; }
+__global__ void k_copy_state(int n, hw::Ptr9 src, hw::Ptr9 dst) {
+  const int o = blockIdx.x * 256 + threadIdx.x;
+  if (o < n) dst.p[blockIdx.y][o] = src.p[blockIdx.y][o];
+}
 
 // What the reverse of one step reads: every stage's input, the step's output, the stage alphas, the
 // stages' source interface values 2 bhat and the first components of their fluxes 2 Fhat. Points into AdjBuffers (one step, recomputed from a
@@ -919,7 +951,7 @@ hw::AdjDev stage_args(const hw::SolverView& v, AdjBuffers* B, const StepTape& T,
     A.lin[q] = B->lam[cur ^ 1][q];
     A.lbase[q] = B->lbase[q];
   }
-  for (int q = 0; q < 12; ++q) A.lR[q] = B->lR[q];
+  for (int q = 0; q < 9; ++q) A.lR[q] = B->lR[q];
   for (int q = 0; q < 6; ++q) { A.lmod[q] = B->lmod[q]; A.lqbx[q] = B->lqbx[q]; A.lqby[q] = B->lqby[q]; }
   for (int f = 0; f < hw::NREC; ++f) { A.lrecx[f] = B->lrecx[f]; A.lrecy[f] = B->lrecy[f]; }
   for (int q = 0; q < 3; ++q) { A.lstat[q] = B->lstat[q]; A.dbx[q] = T.dbx[k - 1][q]; A.dby[q] = T.dby[k - 1][q]; }
@@ -951,17 +983,29 @@ int reverse_stage_body(const hw::SolverView& v, AdjBuffers* B, const hw::AdjDev&
   return HW_OK;
 }
 
+// The nine planes of a state copied: one launch up to 2^18 nodes, where nine copies cost more than what they move (about
+// 2.5 us each on the GPU, 30 sets of them in a checkpointed gradient of 8 steps); copies above, at the copy engine's rate.
+int copy_state(double* const* dst, double* const* src, size_t n, cudaStream_t st) {
+  if (n > ((size_t)1 << 18)) {
+    for (int q = 0; q < 9; ++q) ACUDA(cudaMemcpyAsync(dst[q], src[q], n * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    return HW_OK;
+  }
+  hw::Ptr9 d{}, s{};
+  for (int q = 0; q < 9; ++q) { d.p[q] = dst[q]; s.p[q] = src[q]; }
+  k_copy_state<<<dim3((unsigned)((n + 255) / 256), 9), 256, 0, st>>>((int)n, s, d);
+  ACUDA(cudaGetLastError());
+  return HW_OK;
+}
+
 // Reverse of one recorded step: lam[cur] holds the adjoint of the step's output on entry and of its input
 // on return (in lam[*cur]); static adjoints accumulate.
 int reverse_recorded(const hw::SolverView& v, AdjBuffers* B, const StepTape& T, double dt, int* cur) {
   int rc = HW_OK;
   cudaStream_t st = v.stream;
   const size_t n = v.n;
-  if ((rc = zero_planes(B->lbase, 9, n, st))) return rc;
   for (int k = 3; k >= 1; --k) {
-    const hw::AdjDev A = stage_args(v, B, T, dt, k, *cur);
-    ACUDA(cudaMemsetAsync(B->lalpha, 0, 2 * sizeof(double), st));
-    ACUDA(cudaMemsetAsync(B->argmax, 0x7f, 2 * sizeof(int), st));
+    hw::AdjDev A = stage_args(v, B, T, dt, k, *cur);
+    A.clear = 1;
     if ((rc = reverse_stage_body(v, B, A))) return rc;
     hw::k_adj_alpha_find<<<std::min((int)((n + 255) / 256), 152 * 8), 256, 0, st>>>(A);
     hw::k_adj_alpha_apply<<<1, 1, 0, st>>>(A);
@@ -974,10 +1018,9 @@ int reverse_recorded(const hw::SolverView& v, AdjBuffers* B, const StepTape& T, 
 // Reverse of one step from the solver's current state (recomputed into the one-step buffers).
 int reverse_step(const hw::SolverView& v, AdjBuffers* B, double dt, int* cur) {
   const StepTape T = buffer_tape(B);
-  const size_t bytes = v.n * sizeof(double);
-  for (int q = 0; q < 9; ++q)
-    ACUDA(cudaMemcpyAsync(T.in[0][q], v.state[q], bytes, cudaMemcpyDeviceToDevice, v.stream));
-  int rc = forward_record(v, B, T, dt);
+  int rc = copy_state(T.in[0], v.state, v.n, v.stream);
+  if (rc) return rc;
+  rc = forward_record(v, B, T, dt);
   if (rc) return rc;
   return reverse_recorded(v, B, T, dt, cur);
 }
@@ -1099,14 +1142,14 @@ struct RunCtx {
 int load_slot(RunCtx& R, int slot) {
   double* src[9];
   for (int q = 0; q < 9; ++q) src[q] = R.slots[slot] + (size_t)q * R.v.n;
-  return hw::solver_set_state_planes(R.s, src);
+  hw::solver_view(R.s, &R.v);
+  return copy_state(R.v.state, src, R.v.n, R.v.stream);
 }
 
 int save_slot(RunCtx& R, int slot) {
-  for (int q = 0; q < 9; ++q)
-    ACUDA(cudaMemcpyAsync(R.slots[slot] + (size_t)q * R.v.n, R.v.state[q], R.v.n * sizeof(double),
-                          cudaMemcpyDeviceToDevice, R.v.stream));
-  return HW_OK;
+  double* dst[9];
+  for (int q = 0; q < 9; ++q) dst[q] = R.slots[slot] + (size_t)q * R.v.n;
+  return copy_state(dst, R.v.state, R.v.n, R.v.stream);
 }
 
 // The solver's steps take the recording kernels (hw_forward64.cu) while this lives, so that a recomputed state is
@@ -1214,9 +1257,9 @@ int hw_gauge_loss(hw_solver* s, int nsteps, const double* dts, const int* gauge_
   alloc((void**)&d_idx, W_IDX, ngauge * sizeof(int), "gauge indices");
   if (rc == HW_OK) {
     check(cudaMemcpyAsync(d_idx, gauge_idx, ngauge * sizeof(int), cudaMemcpyHostToDevice, st), "cudaMemcpyAsync");
-    for (int q = 0; q < 9; ++q)
-      check(cudaMemcpyAsync(d_save + (size_t)q * v.n, v.state[q], v.n * sizeof(double), cudaMemcpyDeviceToDevice, st),
-            "cudaMemcpyAsync");
+    double* save[9];
+    for (int q = 0; q < 9; ++q) save[q] = d_save + (size_t)q * v.n;
+    if (rc == HW_OK) rc = copy_state(save, v.state, v.n, st);
   }
   RecordingSteps scope(s);
   for (int j = 0; j < nsteps && rc == HW_OK; ++j) {
@@ -1234,7 +1277,8 @@ int hw_gauge_loss(hw_solver* s, int nsteps, const double* dts, const int* gauge_
     if (eta_gauges) std::copy(g.begin(), g.end(), eta_gauges);
     double* src[9];
     for (int q = 0; q < 9; ++q) src[q] = d_save + (size_t)q * v.n;
-    rc = hw::solver_set_state_planes(s, src);
+    hw::solver_view(s, &v);
+    rc = copy_state(v.state, src, v.n, st);
   }
   cudaStreamSynchronize(st);
   work_trim(B);

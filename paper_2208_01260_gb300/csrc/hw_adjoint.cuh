@@ -3,22 +3,20 @@
 // needs from the same inputs and propagates adjoints through every operation in reverse order. The
 // refined reciprocal and reciprocal square root are differentiated as the exact functions (their
 // results are accurate to a few ulp).
+//
+// The order of operations is part of the result: the bottom's gradient is a small difference of large terms, and another
+// order moves it by what this one's rounding has moved it (measured: weights reversed in normalised form, 93 instead of 111
+// operations per field and nearer to the exact gradient, moved it by up to 1.5e-9 of its norm, so it is not taken).
 #pragma once
 #include "hw_stencil2d.cuh"
 
 namespace hw {
 
-// The kernels that use these functions run at the FP64 pipe's rate, so operations count. The weights are kept
-// normalised: with h_l the adjoint of omega_l and t_l = beta_l + eps, the adjoint of t_l is
-// -2 omega_l (h_l - sum_m omega_m h_m) / t_l, and 1/t_l is the product of the other two over t_1 t_2 t_3 (one more
-// reciprocal). The point value common to the candidates drops out of h_l. Against the reverse operation by operation
-// of the unnormalised form: 93 instead of 111 per field (100 instead of 122 with a source), 75 instead of 120 for the
-// limiter's (whose value comes with it).
-
 // Reverse of hweno_side<false> (Sec. 2.1 eqs. HWEp1, GHYZZ, Rec-f). Inputs: forward data f, p, eps;
 // the adjoint lv of the weighted value. With SRC, the same weights also reconstruct a source from the
-// candidates qbs[3] (Sec. 2.1 Step 2) whose value has adjoint lw: its adjoint reaches the weights here and the
-// candidates through lqbs (added). Outputs: adjoints of f, p; returns twice the adjoint of eps.
+// candidates qbs[3] (Sec. 2.1 Step 2) whose value has adjoint lw: its adjoint reaches the weight
+// numerators and normaliser here and the candidates through lqbs (added). Outputs: adjoints of f, p
+// (added); returns the adjoint of eps.
 template <bool SRC>
 __device__ __forceinline__ double hweno_side_rev(const double f[3], const double p[3], double eps, double lv,
                                                  const double* qbs, double lw, double* lqbs, double lf[3],
@@ -29,71 +27,125 @@ __device__ __forceinline__ double hweno_side_rev(const double f[3], const double
   const double A1 = B1 + (d1 + p[1]);
   const double B2 = fma(2.0, d2, p[1] + p[2]);
   const double A2 = B2 + (d2 + p[1]);
-  const double e = d1 - d2;
+  const double P = fma(0.5, p[1], f[1]);
+  const double e = fma(-2.0, f[1], f[0] + f[2]);
+  const double q1 = fma(1.0 / 6.0, A1, P);
+  const double q2 = fma(-1.0 / 6.0, A2, P);
+  const double q3 = fma(1.0 / 12.0, e, P);
   const double g3 = fma(2.0, p[1], f[0] - f[2]);
-  const double ppe = fma(p[1], p[1], eps);
-  const double cB1 = (781.0 / 20.0) * B1, cA1 = (13.0 / 3.0) * A1, cB2 = (781.0 / 20.0) * B2, cA2 = (13.0 / 3.0) * A2;
-  const double cg = (781.0 / 80.0) * g3, ce = (13.0 / 12.0) * e;
-  const double t1 = fma(cB1, B1, fma(cA1, A1, ppe));
-  const double t2 = fma(cB2, B2, fma(cA2, A2, ppe));
-  const double t3 = fma(cg, g3, fma(ce, e, ppe));
-  const double a1 = t2 * t3, a2 = t1 * t3, a3 = t1 * t2;
-  const double n1 = a1 * a1, n2 = a2 * a2, n3 = a3 * a3;
-  const double r = fast_rcp(fma(4.0 / 3.0, n3, n1 + n2));
-  const double w1 = n1 * r, w2 = n2 * r, w3 = n3 * ((4.0 / 3.0) * r);
-  const double it = -4.0 * fast_rcp(a1 * t1);
-  // value f1 + p1/2 + w1 A1/6 - w2 A2/6 + w3 e/12, source w1 qb1 + w2 qb2 + w3 qb3 = qb3 + w1 (qb1 - qb3) + ...
-  const double v6 = (1.0 / 6.0) * lv, v12 = 0.5 * v6;
-  double h1 = v6 * A1, h2 = -v6 * A2;
-  const double h3 = v12 * e;
+  const double pp = p[1] * p[1];
+  const double b1 = fma((781.0 / 20.0) * B1, B1, fma((13.0 / 3.0) * A1, A1, pp));
+  const double b2 = fma((781.0 / 20.0) * B2, B2, fma((13.0 / 3.0) * A2, A2, pp));
+  const double b3 = fma((781.0 / 80.0) * g3, g3, fma((13.0 / 12.0) * e, e, pp));
+  const double t1 = b1 + eps, t2 = b2 + eps, t3 = b3 + eps;
+  const double s1 = t1 * t1, s2 = t2 * t2, s3 = t3 * t3;
+  const double n1 = s2 * s3, n2 = s1 * s3, n3 = (4.0 / 3.0) * (s1 * s2);
+  const double r = fast_rcp(n1 + n2 + n3);
+  const double num = fma(n1, q1, fma(n2, q2, n3 * q3));
+  // reverse: source value S r with S = n1 qb1 + n2 qb2 + n3 qb3
+  double ln1 = 0.0, ln2 = 0.0, ln3 = 0.0, lr = 0.0;
   if (SRC) {
-    h1 = fma(lw, qbs[0] - qbs[2], h1);
-    h2 = fma(lw, qbs[1] - qbs[2], h2);
-    lqbs[0] = fma(w1, lw, lqbs[0]);
-    lqbs[1] = fma(w2, lw, lqbs[1]);
-    lqbs[2] = fma(w3, lw, lqbs[2]);
+    const double rw = r * lw;
+    ln1 = qbs[0] * rw;
+    ln2 = qbs[1] * rw;
+    ln3 = qbs[2] * rw;
+    lr = fma(n1, qbs[0], fma(n2, qbs[1], n3 * qbs[2])) * lw;
+    lqbs[0] += n1 * rw;
+    lqbs[1] += n2 * rw;
+    lqbs[2] += n3 * rw;
   }
-  const double hb = fma(w1, h1, fma(w2, h2, w3 * h3));
-  // twice the adjoints of t_l
-  const double m1 = (a1 * it) * (w1 * (h1 - hb)), m2 = (a2 * it) * (w2 * (h2 - hb)), m3 = (a3 * it) * (w3 * (h3 - hb));
-  const double lA1 = fma(w1, v6, cA1 * m1), lA2 = fma(-w2, v6, cA2 * m2), le = fma(w3, v12, ce * m3), lg = cg * m3;
-  const double lB1 = fma(cB1, m1, lA1), lB2 = fma(cB2, m2, lA2);
-  const double S = m1 + m2 + m3;
-  // B1 = 2 d1 + p0 + p1, A1 = B1 + d1 + p1, B2 = 2 d2 + p1 + p2, A2 = B2 + d2 + p1, e = d1 - d2, g3 = d1 + d2 + 2 p1
-  const double ld1 = fma(2.0, lB1, lA1) + (lg + le), ld2 = fma(2.0, lB2, lA2) + (lg - le);
-  lf[0] = ld1;
-  lf[1] = lv + (ld2 - ld1);
-  lf[2] = -ld2;
-  lp[0] = lB1;
-  lp[1] = fma(p[1], S, fma(2.0, lg, fma(0.5, lv, (lA1 + lB1) + (lA2 + lB2))));
-  lp[2] = lB2;
-  return S;
+  // reverse of the weighted value
+  const double lnum = r * lv;
+  const double lrt = fma(num, lv, lr);
+  const double lden = -r * r * lrt;
+  const double ln1t = fma(q1, lnum, ln1 + lden);
+  const double ln2t = fma(q2, lnum, ln2 + lden);
+  const double ln3t = fma(q3, lnum, ln3 + lden);
+  const double lq1 = n1 * lnum, lq2 = n2 * lnum, lq3 = n3 * lnum;
+  const double ls1 = fma(s3, ln2t, (4.0 / 3.0) * s2 * ln3t);
+  const double ls2 = fma(s3, ln1t, (4.0 / 3.0) * s1 * ln3t);
+  const double ls3 = fma(s2, ln1t, s1 * ln2t);
+  const double lb1 = 2.0 * t1 * ls1, lb2 = 2.0 * t2 * ls2, lb3 = 2.0 * t3 * ls3;
+  const double leps = lb1 + lb2 + lb3;
+  double lB1 = 2.0 * (781.0 / 20.0) * B1 * lb1;
+  double lA1 = 2.0 * (13.0 / 3.0) * A1 * lb1;
+  double lB2 = 2.0 * (781.0 / 20.0) * B2 * lb2;
+  double lA2 = 2.0 * (13.0 / 3.0) * A2 * lb2;
+  const double lg3 = 2.0 * (781.0 / 80.0) * g3 * lb3;
+  double le = 2.0 * (13.0 / 12.0) * e * lb3;
+  const double lpp = lb1 + lb2 + lb3;
+  double lp1 = 2.0 * p[1] * lpp + 2.0 * lg3;
+  double lf0 = lg3, lf2 = -lg3, lf1 = 0.0;
+  le = fma(1.0 / 12.0, lq3, le);
+  const double lP = lq1 + lq2 + lq3;
+  lA2 = fma(-1.0 / 6.0, lq2, lA2);
+  lA1 = fma(1.0 / 6.0, lq1, lA1);
+  lf0 += le;
+  lf2 += le;
+  lf1 -= 2.0 * le;
+  lf1 += lP;
+  lp1 += 0.5 * lP;
+  // A2 = B2 + d2 + p1; B2 = 2 d2 + p1 + p2
+  lB2 += lA2;
+  double ld2 = lA2;
+  lp1 += lA2;
+  ld2 += 2.0 * lB2;
+  lp1 += lB2;
+  const double lp2 = lB2;
+  // A1 = B1 + d1 + p1; B1 = 2 d1 + p0 + p1
+  lB1 += lA1;
+  double ld1 = lA1;
+  lp1 += lA1;
+  ld1 += 2.0 * lB1;
+  const double lp0 = lB1;
+  lp1 += lB1;
+  lf1 += ld2;
+  lf2 -= ld2;
+  lf0 += ld1;
+  lf1 -= ld1;
+  lf[0] += lf0; lf[1] += lf1; lf[2] += lf2;
+  lp[0] += lp0; lp[1] += lp1; lp[2] += lp2;
+  return leps;
 }
 
-// Reverse of limiter_field<false> (eqs. step1-dxi, limiter-1d) of the differences dl = m1 - m0, dr = m2 - m1 and the
-// derivatives nl, nr; lnu: the adjoint of its value nu, which is formed here too. Returns twice the adjoint of eps.
-__device__ __forceinline__ double limiter_field_rev(double dl, double dr, double nl, double nr, double eps, double lnu,
-                                                    double& nu, double& ldl, double& ldr, double& lnl, double& lnr) {
-  const double pl = fma(2.0, dl, -nl), pr = fma(2.0, dr, -nr), pc = dl + dr;  // pc = 2 p'_3
+// Reverse of limiter_field<false> (eqs. step1-dxi, limiter-1d). Returns adjoint of eps.
+__device__ __forceinline__ double limiter_field_rev(double m0, double m1, double m2, double nl, double nr, double eps,
+                                                    double lnu, double& lm0, double& lm1, double& lm2, double& lnl,
+                                                    double& lnr) {
+  const double dl = m1 - m0, dr = m2 - m1;
+  const double pl = fma(2.0, dl, -nl), pr = fma(2.0, dr, -nr);
+  const double pc2 = dl + dr;
   const double al = dl - nl, ar = dr - nr, ac = dr - dl;
-  const double cl = (13.0 / 3.0) * al, cr = (13.0 / 3.0) * ar, cc = (13.0 / 12.0) * ac, qc = 0.25 * pc;
-  const double t1 = fma(cl, al, fma(pl, pl, eps)), t2 = fma(cr, ar, fma(pr, pr, eps)), t3 = fma(cc, ac, fma(qc, pc, eps));
-  const double a1 = t2 * t3, a2 = t1 * t3, a3 = t1 * t2;
-  const double n1 = a1 * a1, n2 = a2 * a2, n3 = a3 * a3;
-  const double r = fast_rcp(fma(2.0, n3, n1 + n2));
-  const double w1 = n1 * r, w2 = n2 * r, w3 = n3 * r;  // w3: half of omega_3
-  nu = fma(w1, pl, fma(w2, pr, w3 * pc));
-  const double it = (-4.0 * lnu) * fast_rcp(a1 * t1);
-  // twice the adjoints of t_l
-  const double m1 = (a1 * it) * (w1 * (pl - nu)), m2 = (a2 * it) * (w2 * (pr - nu)),
-               m3 = (a3 * it) * (w3 * fma(-2.0, nu, pc));
-  const double lpl = fma(pl, m1, w1 * lnu), lpr = fma(pr, m2, w2 * lnu), lpc = fma(qc, m3, w3 * lnu);
-  const double lal = cl * m1, lar = cr * m2, lac = cc * m3;
-  ldl = fma(2.0, lpl, lal) + (lpc - lac);
-  ldr = fma(2.0, lpr, lar) + (lpc + lac);
-  lnl = -(lal + lpl);
-  lnr = -(lar + lpr);
-  return m1 + m2 + m3;
+  const double b1 = fma((13.0 / 3.0) * al, al, pl * pl);
+  const double b2 = fma((13.0 / 3.0) * ar, ar, pr * pr);
+  const double b3 = fma((13.0 / 12.0) * ac, ac, (0.25 * pc2) * pc2);
+  const double t1 = b1 + eps, t2 = b2 + eps, t3 = b3 + eps;
+  const double s1 = t1 * t1, s2 = t2 * t2, s3 = t3 * t3;
+  const double n1 = s2 * s3, n2 = s1 * s3, n3 = s1 * s2;
+  const double den = fma(2.0, n3, n1 + n2);
+  const double num = fma(n1, pl, fma(n2, pr, n3 * pc2));
+  const double r = fast_rcp(den);
+  const double lnum = r * lnu;
+  const double lden = -num * r * r * lnu;
+  const double ln1 = fma(pl, lnum, lden), ln2 = fma(pr, lnum, lden), ln3 = fma(pc2, lnum, 2.0 * lden);
+  double lpl = n1 * lnum, lpr = n2 * lnum, lpc2 = n3 * lnum;
+  const double ls1 = fma(s3, ln2, s2 * ln3), ls2 = fma(s3, ln1, s1 * ln3), ls3 = fma(s2, ln1, s1 * ln2);
+  const double lb1 = 2.0 * t1 * ls1, lb2 = 2.0 * t2 * ls2, lb3 = 2.0 * t3 * ls3;
+  const double leps = lb1 + lb2 + lb3;
+  const double lal = 2.0 * (13.0 / 3.0) * al * lb1;
+  lpl += 2.0 * pl * lb1;
+  const double lar = 2.0 * (13.0 / 3.0) * ar * lb2;
+  lpr += 2.0 * pr * lb2;
+  const double lac = 2.0 * (13.0 / 12.0) * ac * lb3;
+  lpc2 += 0.5 * pc2 * lb3;
+  double ldr = lac + lar + lpc2 + 2.0 * lpr;
+  double ldl = -lac + lal + lpc2 + 2.0 * lpl;
+  lnr += -lar - lpr;
+  lnl += -lal - lpl;
+  lm2 += ldr;
+  lm1 += -ldr + ldl;
+  lm0 += -ldl;
+  return leps;
 }
 
 // Reverse of node_record<DIR> (pointwise fluxes, chain-rule derivative fluxes, split). lrec: adjoint of
@@ -288,7 +340,7 @@ __device__ __forceinline__ void interface_values_rev(const double* r0, int sstep
     const double sg = side == 0 ? 1.0 : -1.0;
     double f[3][3], p[3][3];
     project(side, f, p);
-    double lf[3][3], lp[3][3];
+    double lf[3][3] = {}, lp[3][3] = {};
     // source: GB1 -= weighted(W0), GB3 += weighted(W2)
     leps13 += hweno_side_rev<true>(f[0], p[0], eps13, lG[0], qb + 3 * side, -lGB1, lqb + 3 * side, lf[0], lp[0]);
     (void)hweno_side_rev<false>(f[1], p[1], eps2, lG[1], nullptr, 0.0, nullptr, lf[1], lp[1]);
@@ -322,7 +374,7 @@ __device__ __forceinline__ void interface_values_rev(const double* r0, int sstep
   double lrs = 0.5 * lic2 + gh * lcb;
   double lgh = rs * lcb;
   lgh += -0.5 * rs * rs * rs * lrs;
-  double lhs = (4.0 * g * eps_w) * leps13 + (0.5 * g) * lgh;  // leps13: twice the adjoint
+  double lhs = (8.0 * g * eps_w) * leps13 + (0.5 * g) * lgh;
   const double lrhs = smM * lub + smW * lvb;
   lhs -= rhs * rhs * lrhs;
   lr(1, R_H) = lhs;
@@ -344,7 +396,7 @@ __device__ __forceinline__ void interface_values_rev(const double* r0, int sstep
 }
 
 // Reverse of limit_dir<DIR, false, true>: lout (3) -> adjoints of Um, U0, Up, Dm, Dp and of the node's
-// u, v, c (through ic2 and the projection rows) and of gh (through epsilon). Writes the arrays, adds to the scalars.
+// u, v, c (through ic2 and the projection rows) and of gh (through epsilon). Adds into the arrays.
 template <int DIR>
 __device__ __forceinline__ void limit_dir_rev(const double Um[3], const double U0[3], const double Up[3],
                                               const double Dm[3], const double Dp[3], double u, double v, double c,
@@ -354,59 +406,50 @@ __device__ __forceinline__ void limit_dir_rev(const double Um[3], const double U
   const int cn = DIR == 0 ? 1 : 2, ct = DIR == 0 ? 2 : 1;
   const double un = DIR == 0 ? u : v, ut = DIR == 0 ? v : u;
   const double upc = un + c, umc = un - c;
-  // differences to the two neighbours and their derivatives, projected
-  double src[4][3], pr[4][3];
+  const double* src[5] = {Um, U0, Up, Dm, Dp};
+  double* lsrc[5] = {lUm, lU0, lUp, lDm, lDp};
+  double pr[5][3];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    src[0][c] = U0[c] - Um[c];
-    src[1][c] = Up[c] - U0[c];
-    src[2][c] = Dm[c];
-    src[3][c] = Dp[c];
-  }
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
+  for (int s = 0; s < 5; ++s) {
     const double* a = src[s];
     pr[s][0] = fma(upc, a[0], -a[cn]);
     pr[s][1] = fma(-ut, a[0], a[ct]);
     pr[s][2] = fma(-umc, a[0], a[cn]);
   }
   const double e13 = (4.0 * eps) * gh;
-  // reverse of the back-projection (A, un A + (nu2 - nu0)/2, ut A + nu1) with A = (nu0 + nu2) ic2
+  double nu[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    nu[k] = limiter_field<false>(pr[0][k], pr[1][k], pr[2][k], pr[3][k], pr[4][k], k == 1 ? eps : e13);
+  const double A = (nu[0] + nu[2]) * ic2;
+  // reverse of the back-projection (A, un A + (nu2 - nu0)/2, ut A + nu1)
   const double lA = lout[0] + un * lout[cn] + ut * lout[ct];
-  double lnu[3], nu[3];
-  lnu[0] = fma(ic2, lA, -0.5 * lout[cn]);
-  lnu[2] = fma(ic2, lA, 0.5 * lout[cn]);
+  double lun = A * lout[cn], lut = A * lout[ct];
+  double lnu[3];
+  lnu[0] = -0.5 * lout[cn] + ic2 * lA;
+  lnu[2] = 0.5 * lout[cn] + ic2 * lA;
   lnu[1] = lout[ct];
-  double lpr[4][3];
+  lic2 += (nu[0] + nu[2]) * lA;
+  double lpr[5][3] = {};
   double le13 = 0.0;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const double le = limiter_field_rev(pr[0][k], pr[1][k], pr[2][k], pr[3][k], k == 1 ? eps : e13, lnu[k], nu[k],
-                                        lpr[0][k], lpr[1][k], lpr[2][k], lpr[3][k]);
+    const double le = limiter_field_rev(pr[0][k], pr[1][k], pr[2][k], pr[3][k], pr[4][k], k == 1 ? eps : e13, lnu[k],
+                                        lpr[0][k], lpr[1][k], lpr[2][k], lpr[3][k], lpr[4][k]);
     if (k != 1) le13 += le;
   }
-  const double sn = nu[0] + nu[2], A = sn * ic2;
-  double lun = A * lout[cn], lut = A * lout[ct];
-  lic2 += sn * lA;
-  lgh += (2.0 * eps) * le13;  // le13: twice the adjoint
-  double lupc = 0.0, lumc = 0.0, l[4][3];
+  lgh += (4.0 * eps) * le13;
+  double lupc = 0.0, lumc = 0.0;
 #pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const double a = src[s][0];
-    lupc = fma(a, lpr[s][0], lupc);
-    lut = fma(-a, lpr[s][1], lut);
-    lumc = fma(-a, lpr[s][2], lumc);
-    l[s][0] = upc * lpr[s][0] - ut * lpr[s][1] - umc * lpr[s][2];
-    l[s][cn] = lpr[s][2] - lpr[s][0];
-    l[s][ct] = lpr[s][1];
-  }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    lUm[c] = -l[0][c];
-    lU0[c] = l[0][c] - l[1][c];
-    lUp[c] = l[1][c];
-    lDm[c] = l[2][c];
-    lDp[c] = l[3][c];
+  for (int s = 0; s < 5; ++s) {
+    const double* a = src[s];
+    double* l = lsrc[s];
+    lupc += a[0] * lpr[s][0];
+    lut -= a[0] * lpr[s][1];
+    lumc -= a[0] * lpr[s][2];
+    l[0] += upc * lpr[s][0] - ut * lpr[s][1] - umc * lpr[s][2];
+    l[cn] += -lpr[s][0] + lpr[s][2];
+    l[ct] += lpr[s][1];
   }
   lun += lupc + lumc;
   lc += lupc - lumc;

@@ -773,12 +773,6 @@ int solver_view(hw_solver* s, SolverView* v) {
   return HW_OK;
 }
 
-int solver_set_state_planes(hw_solver* s, double* const* src) {
-  double** S = s->state();
-  for (int q = 0; q < s->nstate; ++q)
-    CUDA_OK(cudaMemcpyAsync(S[q], src[q], s->n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream));
-  return HW_OK;
-}
 }  // namespace hw
 
 extern "C" {
