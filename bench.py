@@ -64,21 +64,21 @@ PEAK_FP64_OPS = SMS * DFMA_PER_SM_CLK * SM_GHZ * 1e9
 # The whole-step HBM fraction is taken against it.
 ALGO_BYTES_PER_NODE_STAGE = 216.0
 # DRAM bytes per unit from ncu captures (dram__bytes_read.sum + dram__bytes_write.sum of one launch of this
-# benchmark at 2048^2, a one-pass capture; the node kernel at RK stage 3), valid only for the kernel sources
-# they were taken on (sources_sha); times the units of a launch.
+# workload at 2048x1024; the node kernel at RK stage 3), valid only for the kernel sources they were taken on
+# (sources_sha); times the units of a launch.
 TRAFFIC = {
-    "sweep_x": {"bytes_per_unit": 231.5, "sha": "e0ac982961c54e0f"},
-    "sweep_y": {"bytes_per_unit": 235.4, "sha": "e0ac982961c54e0f"},
-    "node": {"bytes_per_unit": 533.9, "sha": "e0ac982961c54e0f"},
+    "sweep_x": {"bytes_per_unit": 235.9, "sha": "e17dae5e7f0f81be"},
+    "sweep_y": {"bytes_per_unit": 229.0, "sha": "e17dae5e7f0f81be"},
+    "node": {"bytes_per_unit": 505.7, "sha": "e17dae5e7f0f81be"},
 }
-# FP64-pipe instructions per unit (ncu --set full at 2048x1024: DFMA + DADD + DMUL thread instructions of
-# one launch over its units; the count per unit does not depend on the grid size). Part of the products
-# run on the integer pipes (each bit-identical to DMUL), so these are below the algorithmic "ops" above;
-# valid only for the kernel sources they were taken on (sources_sha).
+# FP64-pipe instructions per unit (ncu at 2048x1024: sm__inst_executed_pipe_fp64 of one launch times 32 over its
+# units, the node kernel's mean over the three stages; the count per unit does not depend on the grid size). The
+# reconstruction and the limiter run in fixed point on the integer pipes, so these are below the algorithmic "ops"
+# above; valid only for the kernel sources they were taken on (sources_sha).
 FP64_PIPE_OPS = {
-    "sweep_x": {"ops_per_unit": 341.9, "sha": "e0ac982961c54e0f"},
-    "sweep_y": {"ops_per_unit": 342.8, "sha": "e0ac982961c54e0f"},
-    "node": {"ops_per_unit": 243.0, "sha": "e0ac982961c54e0f"},
+    "sweep_x": {"ops_per_unit": 68.7, "sha": "e17dae5e7f0f81be"},
+    "sweep_y": {"ops_per_unit": 70.5, "sha": "e17dae5e7f0f81be"},
+    "node": {"ops_per_unit": 100.0, "sha": "e17dae5e7f0f81be"},
 }
 STATE_BYTES = 9 * NX * NY * 8
 
@@ -90,7 +90,7 @@ def hbm_peak():
         return 6800.0, "fallback"
 
 
-FORWARD_SOURCES = ("hw_device.cuh", "hw_fp64_int.h", "hw_stencil2d.cuh", "hw_kernels2d.cu", "hw_internal.h")
+FORWARD_SOURCES = ("hw_device.cuh", "hw_fp64_int.h", "hw_fixed.h", "hw_stencil2d.cuh", "hw_kernels2d.cu", "hw_internal.h")
 
 
 def sources_sha():
@@ -695,8 +695,8 @@ def main():
                 "peak_how": "FP64 fma throughput measured live on this GPU before the timed region "
                             "(hw_measure_fp64_peak, median of 20 launches; fma = 2 flops); see fp64_peak",
                 "algo_ops_frac": kd["algo_ops_frac"], "fp64_pipe_frac": kd["fp64_pipe_frac"],
-                "int_pipe_note": "part of the products run on the integer pipes (bit-identical binary64), so the "
-                                 "algorithmic rate can exceed the FP64 pipe's share; fp64_pipe_frac is the pipe's own use",
+                "int_pipe_note": "the reconstruction and the limiter run in fixed point on the integer pipes, so the "
+                                 "algorithmic rate exceeds the FP64 pipe's; fp64_pipe_frac is the pipe's own use",
                 "hbm_peak_gbs": hbm, "hbm_peak_src": hbm_src,
                 "sources_sha": sha}
     step_ops = sum(ALGO[k]["ops"] * UNITS_PER_LAUNCH[k] for k in ALGO) * STAGES

@@ -1,5 +1,6 @@
 // 2D kernels of the well-balanced fifth-order FD HWENO scheme (Zhao & Zhang, arXiv:2208.01260,
-// Sec. 3) for sm_103a. One RK stage is four launches on the solver's stream:
+// Sec. 3) for sm_103a. One RK stage is four launches on the solver's stream (three on grids whose sweeps share one, two
+// in single precision, hw_stage32.cu; the adjoint's forward pass has its own, hw_forward64.cu):
 //   k_alpha2d_* global Lax-Friedrichs constants alpha_x = max(|u|+c), alpha_y = max(|v|+c)
 //   k_sweep_x   x-interfaces: Sec. 2.1 Steps 1-2 along x for (F1, Phi1, tilde-b, tilde-B1) and the
 //               mixed term Psi1 of eq. (mixed)
@@ -21,9 +22,9 @@ constexpr int YS_C = 2;  // columns per y-tile group of the double y-sweep (meas
 
 // The double kernels run the nonlinear reconstruction and the limiter in fixed point (hw_fixed.h): on the FP64
 // pipe alone these kernels took 2.80 (x), 2.85 (y) and 2.03 ms (node) per stage at 2048^2, its operations at the
-// pipe's rate; now 0.78, 0.84 and 0.87 ms. What bounds the sweeps is the sum of what is left on the FP64 pipe (69
+// pipe's rate; now 0.80, 0.85 and 0.91 ms. What bounds the sweeps is the sum of what is left on the FP64 pipe (69
 // operations per x-interface, 58% busy) and integer work (4110 instructions per warp, 54% of the issue slots, the integer
-// pipe 60% busy); the node kernel the FP64 pipe (99 operations, 70% busy) with the latency of its loads.
+// pipe 60% busy); the node kernel the FP64 pipe (100 operations, 73-79% busy) with the latency of its loads.
 template <class R>
 constexpr bool kFixed = std::is_same<R, double>::value;
 template <class R>
