@@ -217,7 +217,7 @@ __device__ __forceinline__ double record_sum(int f, const At& at, const Ok& ok) 
 // has finished, each record sums its contributions, so only the three records (rows of records) a block shares with
 // each neighbour are added atomically.
 //
-// Bound by the FP64 pipe, at 255 registers a thread: 8 warps per SM, in whatever blocks. Both sweeps are one launch of
+// Bound by the FP64 pipe, at 198 registers a thread and 48 KB a block: 8 warps per SM. Both sweeps are one launch of
 // small blocks because the grids this runs on are small: as two launches, with 256 threads a y-block, a grid of 150 x 97
 // had 291 and 65 blocks (the y-sweep on 65 of 152 SMs, as long as two of its warps per partition take), and one of
 // 256^2 ran 2.1 and 1.7 waves in 3 and 2. With the node kernels in small blocks too, the gradient 11.9 -> 10.9 ms at 256^2 and (with
