@@ -348,7 +348,7 @@ __device__ __forceinline__ void alpha_block_done(unsigned long long* slots, cons
 }
 
 // The nodes alpha_exact_range would evaluate, in the tiles whose coarse maxima reach the thresholds. keys: the
-// maxima; FINISH: keys are the slots of alpha_block_done.
+// maxima; FINISH: keys are the slots of alpha_block_done, and m32 one of them.
 template <bool FINISH>
 __global__ void __launch_bounds__(256) k_alpha2d_exact(Dev2D d, const unsigned int* m32, const uint2* tiles,
                                                        unsigned long long* keys, int* status, AlphaOut f) {
@@ -383,9 +383,11 @@ __global__ void __launch_bounds__(256) k_alpha2d_exact(Dev2D d, const unsigned i
       if (FINISH) __threadfence();
     }
     if (bad) atomicOr(status, bad);
-    if (FINISH) __syncthreads();
   }
-  if (FINISH && threadIdx.x == 0) alpha_block_done(keys, f);
+  if (!FINISH) return;
+  // also in a skipped tile: the last block to arrive clears m32, which every warp of every block must have read by then
+  __syncthreads();
+  if (threadIdx.x == 0) alpha_block_done(keys, f);
 }
 
 // The whole reduction in one launch, for small grids (kAlphaOneMax): each block takes 256 U nodes.
