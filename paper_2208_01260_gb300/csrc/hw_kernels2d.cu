@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(192, 3) k_node2d_split(const __grid_constant__
       if (sa.base) sa.base[3 * role + q][o] = cq;
       *out = fma(dt, R, cq);
     } else if (sa.k == 2) {
-      *out = fx_quarter(fma(dt, R, fma(3.0, __ldg(sa.base[3 * role + q] + o), cq)));
+      *out = fma(0.75, __ldg(sa.base[3 * role + q] + o), fx_quarter(fma(dt, R, cq)));
     } else {
       *out = fma(1.0 / 3.0, __ldg(sa.base[3 * role + q] + o), (2.0 / 3.0) * fma(dt, R, cq));
     }

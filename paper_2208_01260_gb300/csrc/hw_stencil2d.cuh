@@ -1050,11 +1050,14 @@ __device__ __forceinline__ void node_update_faces(const Dev2DT<R>& d, const S sr
     return;
   }
   if constexpr (std::is_same<R, double>::value) {
-    if (sa.k == 2) {  // (3 base + cq + dt R) / 4: two operations on the FP64 pipe
+    // 3/4 base + (cq + dt R)/4, the quarter without the FP64 pipe. As (3 base + cq + dt R)/4, also two operations, the sum
+    // 3 base + cq is rounded at the result's own last place where here only a quarter of a rounding comes in: errors of runs
+    // against 64 bits were 5 to 8% larger with it.
+    if (sa.k == 2) {
 #pragma unroll
       for (int q = 0; q < 9; ++q) {
         const R cq = q < 3 ? cur[q] : mod[q - 3];
-        sa.out[q][o] = fx_quarter(fma(dt, Rv[q], fma(3.0, ldp<COH>(sa.base[q] + o), cq)));
+        sa.out[q][o] = fma(0.75, ldp<COH>(sa.base[q] + o), fx_quarter(fma(dt, Rv[q], cq)));
       }
       return;
     }
