@@ -234,8 +234,8 @@ int hw_batch_get_phase_times(hw_batch* b, double* ms);
  * characteristic projection, gauge index outside the grid, grid above about 2^30 nodes), HW_ERR_STATE
  * (before hw_init), HW_ERR_NOMEM (working buffers, snapshots or tape), HW_ERR_CUDA.
  * Working buffers (about 180 planes of nx*ny doubles) are allocated at the first call and freed by
- * hw_destroy; so is a call's own memory (tape, snapshots, gauge values), of which up to 2 GiB are kept for the
- * solver's next call.
+ * hw_destroy; so is a call's own memory (tape, snapshots, gauge values), of which up to 2 GiB in all are kept for
+ * the solvers' next calls. While device memory is short, calls of this library that allocate give back what is kept.
  * ------------------------------------------------------------------------------------------- */
 /* Reverse of one hw_rk3_step(dt) taken from the solver's current state: lam_state (9 device planes,
  * equilibrium layout) holds the adjoint of the step's output on entry and of its input on return;

@@ -25,6 +25,7 @@
 #include "hw_adjoint.cuh"
 #include "hw_halo.h"
 #include "hw_internal.h"
+#include "hw_workpool.h"
 
 namespace hw {
 
@@ -677,6 +678,16 @@ int afail(int code, const std::string& m) { return hw::set_last_error(code, m.c_
     if (e_ != cudaSuccess) return afail(HW_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
+struct DeviceMem {
+  static void* get(size_t bytes) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
+  }
+  static void put(void* p) { cudaFree(p); }
+};
+
 struct AdjBuffers {
   hw_solver* owner = nullptr;
   size_t n = 0;
@@ -704,15 +715,12 @@ struct AdjBuffers {
   int* argmax = nullptr;
   double* lstatic_phys[3] = {};
   unsigned long long* amax = nullptr;  // the forward alpha reduction's keys and scratch (kAlpha2dScratch)
-  // memory of one call (hw_gauge_loss, hw_adjoint_run), kept for the solver's next one up to kKeep bytes each
-  // and freed with the buffers above: allocating and freeing it cost as much as a small run's kernels
-  struct Work {
-    void* p = nullptr;
-    size_t bytes = 0;
-  };
-  std::vector<Work> work;
+  // memory of one call (hw_gauge_loss, hw_adjoint_run), kept for the solver's next one (WorkScope) and freed with the
+  // buffers above at the latest
+  hw::WorkPool<DeviceMem> work;
+  bool busy = false;  // a call uses the pool (under g_adj_mu)
 };
-constexpr size_t kKeep = (size_t)1 << 31;
+constexpr size_t kKeep = (size_t)1 << 31;  // bytes kept in all, over every solver
 enum { W_SAVE = 0, W_GVALS, W_OBS, W_IDX, W_TAPE, W_SLOT };  // W_SLOT + k: snapshot k
 
 std::mutex g_adj_mu;
@@ -723,7 +731,7 @@ std::vector<AdjBuffers*> g_adj;  // one per live solver that used the adjoint (r
 // is done), so they must start at zero, not at whatever the memory held.
 int adj_alloc(AdjBuffers* B, double** p, int count, size_t cnt, cudaStream_t st) {
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, count * cnt * sizeof(double));
+  cudaError_t e = hw::device_alloc(&q, count * cnt * sizeof(double));
   if (e != cudaSuccess) return afail(HW_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   B->allocs.push_back(q);
   for (int k = 0; k < count; ++k) p[k] = (double*)q + (size_t)k * cnt;
@@ -746,51 +754,34 @@ AdjBuffers* find_entry(hw_solver* s, const hw::SolverView& v) {
   return B;
 }
 
-// At least `bytes` of the entry's memory number k, reused between calls (its contents are not). A call asks in
-// rising order of k; when memory is short, what an earlier call left above k is given back first.
-void* work_get(AdjBuffers* B, int k, size_t bytes) {
-  if (B->work.size() <= (size_t)k) B->work.resize(k + 1);
-  AdjBuffers::Work& w = B->work[k];
-  if (w.bytes >= bytes) return w.p;
-  cudaFree(w.p);
-  w = {};
-  cudaError_t e = cudaMalloc(&w.p, bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    for (size_t l = k + 1; l < B->work.size(); ++l) {
-      cudaFree(B->work[l].p);
-      B->work[l] = {};
-    }
-    e = cudaMalloc(&w.p, bytes);
-  }
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    w.p = nullptr;
-    return nullptr;
-  }
-  w.bytes = bytes;
-  return w.p;
+// The pools of solvers that are in no call, freed; whether they held anything.
+bool release_idle_pools() {
+  bool any = false;
+  for (AdjBuffers* B : g_adj)
+    if (!B->busy) any |= B->work.release_unclaimed();
+  return any;
 }
 
-// Gives back what a call needed beyond kKeep (its stream has drained).
-void work_trim(AdjBuffers* B) {
-  size_t held = 0;
-  for (AdjBuffers::Work& w : B->work) {
-    held += w.bytes;
-    if (w.p && held > kKeep) {
-      cudaFree(w.p);
-      held -= w.bytes;
-      w = {};
-    }
+// A call's use of its solver's pool. At its end up to kKeep bytes stay; if all solvers together keep more, those of the
+// others that are in no call are freed.
+struct WorkScope {
+  AdjBuffers* const B;
+  explicit WorkScope(AdjBuffers* B_) : B(B_) {
+    std::lock_guard<std::mutex> lk(g_adj_mu);
+    B->busy = true;
+    B->work.begin();
   }
-}
-
-// Bytes held by the memories from number k on.
-size_t work_bytes(const AdjBuffers* B, size_t k) {
-  size_t held = 0;
-  for (; k < B->work.size(); ++k) held += B->work[k].bytes;
-  return held;
-}
+  void* get(int k, size_t bytes) { return B->work.get(k, bytes, hw::release_idle_memory); }
+  ~WorkScope() {
+    std::lock_guard<std::mutex> lk(g_adj_mu);
+    B->work.end(kKeep);
+    size_t held = 0;
+    for (const AdjBuffers* X : g_adj)
+      if (!X->busy || X == B) held += X->work.held();
+    if (held > kKeep) release_idle_pools();
+    B->busy = false;
+  }
+};
 
 int get_buffers(hw_solver* s, const hw::SolverView& v, AdjBuffers** out) {
   AdjBuffers* B = find_entry(s, v);
@@ -838,12 +829,26 @@ int get_buffers(hw_solver* s, const hw::SolverView& v, AdjBuffers** out) {
 
 }  // namespace
 
+bool hw::release_idle_memory() {
+  std::lock_guard<std::mutex> lk(g_adj_mu);
+  return release_idle_pools();
+}
+
+cudaError_t hw::device_alloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && release_idle_memory()) {
+    cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
 void hw::adjoint_release(hw_solver* s) {
   std::lock_guard<std::mutex> lk(g_adj_mu);
   for (size_t k = 0; k < g_adj.size(); ++k)
     if (g_adj[k]->owner == s) {
       for (void* p : g_adj[k]->allocs) cudaFree(p);
-      for (AdjBuffers::Work& w : g_adj[k]->work) cudaFree(w.p);
+      g_adj[k]->work.end(0);
       delete g_adj[k];
       g_adj.erase(g_adj.begin() + k);
       return;
@@ -1243,13 +1248,13 @@ int hw_gauge_loss(hw_solver* s, int nsteps, const double* dts, const int* gauge_
   cudaStream_t st = v.stream;
   double *d_save = nullptr, *d_g = nullptr;
   int* d_idx = nullptr;
-  AdjBuffers* B = find_entry(s, v);
+  WorkScope work(find_entry(s, v));
   auto check = [&](cudaError_t e, const char* what) {
     if (rc == HW_OK && e != cudaSuccess) rc = afail(HW_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
   };
   auto alloc = [&](void** p, int k, size_t bytes, const char* what) {
     if (rc != HW_OK) return;
-    *p = work_get(B, k, bytes);
+    *p = work.get(k, bytes);
     if (!*p) rc = afail(HW_ERR_NOMEM, std::string("hw_gauge_loss: allocation failed: ") + what);
   };
   alloc((void**)&d_save, W_SAVE, 9 * v.n * sizeof(double), "saved state");
@@ -1280,8 +1285,7 @@ int hw_gauge_loss(hw_solver* s, int nsteps, const double* dts, const int* gauge_
     hw::solver_view(s, &v);
     rc = copy_state(v.state, src, v.n, st);
   }
-  cudaStreamSynchronize(st);
-  work_trim(B);
+  cudaStreamSynchronize(st);  // before the end of work
   return rc;
 }
 
@@ -1311,7 +1315,9 @@ int hw_adjoint_run(hw_solver* s, int nsteps, const double* dts, const int* gauge
   if (snapshots == HW_ADJ_TAPE || snapshots == HW_ADJ_AUTO) {
     size_t free_b = 0, total_b = 0;
     ACUDA(cudaMemGetInfo(&free_b, &total_b));
-    const double budget = 0.9 * ((double)free_b + (double)work_bytes(B, W_TAPE));  // what is kept is reused or given back
+    if ((double)layout.bytes() > 0.9 * (double)free_b && hw::release_idle_memory())
+      ACUDA(cudaMemGetInfo(&free_b, &total_b));
+    const double budget = 0.9 * (double)free_b;
     if ((double)layout.bytes() <= budget) {
       use_tape = true;
     } else if (snapshots == HW_ADJ_TAPE) {
@@ -1330,14 +1336,14 @@ int hw_adjoint_run(hw_solver* s, int nsteps, const double* dts, const int* gauge
   double* d_obs = nullptr;
   int* d_idx = nullptr;
   double* tape = nullptr;
+  WorkScope work(B);
   auto cleanup = [&]() {
-    cudaStreamSynchronize(st);
-    work_trim(B);
+    cudaStreamSynchronize(st);  // before the end of work
     if (forward_steps_out) *forward_steps_out = R.fwd_steps;
   };
   auto alloc = [&](void** p, int k, size_t bytes, const char* what) {
     if (rc != HW_OK) return;
-    *p = work_get(B, k, bytes);
+    *p = work.get(k, bytes);
     if (!*p) rc = afail(HW_ERR_NOMEM, std::string("hw_adjoint_run: allocation failed: ") + what);
   };
   alloc((void**)&R.d_gvals, W_GVALS, (size_t)nsteps * ngauge * sizeof(double), "gauge values");
@@ -1492,7 +1498,7 @@ int dd_adjoint_impl(hw_dd* dd, int nsteps, const double* dts, const int* gauge_i
   };
   auto alloc = [&](void** q, size_t bytes, const char* what) {
     if (rc != HW_OK) return;
-    if (cudaMalloc(q, bytes) != cudaSuccess) {
+    if (hw::device_alloc(q, bytes) != cudaSuccess) {
       cudaGetLastError();
       rc = afail(HW_ERR_NOMEM, std::string("hw_dd_adjoint_run: allocation failed: ") + what);
     }
@@ -1778,7 +1784,7 @@ int hw_part_adj_create(hw_solver* s, int nsteps, int ngauge, int nloc, const int
   a->layout = new RunTape(a->v, nsteps);
   auto alloc = [&](void** q, size_t bytes) {
     if (rc != HW_OK) return;
-    if (cudaMalloc(q, bytes) != cudaSuccess) {
+    if (hw::device_alloc(q, bytes) != cudaSuccess) {
       cudaGetLastError();
       rc = afail(HW_ERR_NOMEM, "hw_part_adj_create: allocation failed");
     }

@@ -134,7 +134,7 @@ static void timed(hw_solver* s, int cls, Fn&& fn, int kernels = 1) {
 
 static int dalloc(hw_solver* s, double** p, size_t count) {
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, count * sizeof(double));
+  cudaError_t e = hw::device_alloc(&q, count * sizeof(double));
   if (e != cudaSuccess) return fail(HW_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   s->allocs.push_back(q);
   *p = (double*)q;
@@ -143,7 +143,7 @@ static int dalloc(hw_solver* s, double** p, size_t count) {
 
 static int falloc(hw_solver* s, float** p, size_t count) {
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, count * sizeof(float));
+  cudaError_t e = hw::device_alloc(&q, count * sizeof(float));
   if (e != cudaSuccess) return fail(HW_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   s->allocs.push_back(q);
   *p = (float*)q;

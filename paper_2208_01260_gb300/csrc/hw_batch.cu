@@ -159,7 +159,7 @@ struct hw_batch {
 
 namespace {
 int balloc(hw_batch* b, void** p, size_t bytes) {
-  cudaError_t e = cudaMalloc(p, bytes);
+  cudaError_t e = hw::device_alloc(p, bytes);
   if (e != cudaSuccess) return bfail(HW_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   b->allocs.push_back(*p);
   return HW_OK;
@@ -207,7 +207,7 @@ int upload_items(hw_batch* b, std::vector<int4> lists[5], int4** dst, int* count
     if (dst[p]) { cudaFree(dst[p]); dst[p] = nullptr; }
     counts[p] = (int)lists[p].size();
     if (counts[p] == 0) continue;
-    BCUDA(cudaMalloc(&dst[p], lists[p].size() * sizeof(int4)));
+    BCUDA(hw::device_alloc((void**)&dst[p], lists[p].size() * sizeof(int4)));
     BCUDA(cudaMemcpyAsync(dst[p], lists[p].data(), lists[p].size() * sizeof(int4), cudaMemcpyHostToDevice, b->stream));
   }
   BCUDA(cudaStreamSynchronize(b->stream));

@@ -298,7 +298,7 @@ int dd_fail(int code, const std::string& msg) { return hw::set_last_error(code, 
   } while (0)
 
 int dd_alloc(hw_dd* d, void** p, size_t bytes) {
-  cudaError_t e = cudaMalloc(p, bytes);
+  cudaError_t e = hw::device_alloc(p, bytes);
   if (e != cudaSuccess) return dd_fail(HW_ERR_NOMEM, std::string("hw_dd: cudaMalloc: ") + cudaGetErrorString(e));
   d->allocs.push_back(*p);
   return HW_OK;

@@ -250,5 +250,9 @@ int dd_exchange_adjoint(hw_dd* d, double* const* const* planes, int nplanes, uns
 int dd_fork_blocks(hw_dd* d, cudaStream_t st);
 int dd_join_blocks(hw_dd* d, cudaStream_t st);
 void adjoint_release(hw_solver* s);  // frees a solver's adjoint working buffers; hw_destroy calls it
+// Frees what solvers that are in no call keep for their next adjoint call; whether there was any.
+bool release_idle_memory();
+// cudaMalloc, once more after release_idle_memory while memory is short.
+cudaError_t device_alloc(void** p, size_t bytes);
 
 }  // namespace hw
