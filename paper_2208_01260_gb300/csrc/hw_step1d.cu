@@ -562,8 +562,9 @@ __global__ void __launch_bounds__(kThreads<N>) k_run1d(Dev1D d, Run1D r) {
   double alpha = r.tm.alpha[0];
   if (t < 3) sm.dt[t] = r.tm.dt[t];
   unsigned long long steps = 0;
-  int p = 0, pending = 0, used = 0;
-  cluster_barrier();  // every block runs; shared memory loaded
+  // flags of the state that the next stage reads, from the launch before (slot[2], as k_stage1d's) and to the next one
+  int p = 0, pending = (int)r.tm.slot[2], used = 0;
+  cluster_barrier();  // every block runs; shared memory and slot[2] read
   for (int step = 0; step < r.nsteps; ++step) {
     if (r.t_end > 0.0 && sm.dt[2] >= r.t_end) break;  // the same in every block
     for (int k = 1; k <= 3; ++k) {
@@ -621,6 +622,7 @@ __global__ void __launch_bounds__(kThreads<N>) k_run1d(Dev1D d, Run1D r) {
     if (t < 3) r.tm.dt[t] = sm.dt[t];
     if (t == 0) {
       r.tm.alpha[0] = alpha;
+      r.tm.slot[2] = (unsigned long long)pending;
       if (used) atomicOr(r.tm.status, used);
     }
     if (t == 32) *r.tm.nsteps += steps;
