@@ -67,18 +67,18 @@ ALGO_BYTES_PER_NODE_STAGE = 216.0
 # workload at 2048x1024; the node kernel at RK stage 3), valid only for the kernel sources they were taken on
 # (sources_sha); times the units of a launch.
 TRAFFIC = {
-    "sweep_x": {"bytes_per_unit": 235.9, "sha": "e17dae5e7f0f81be"},
-    "sweep_y": {"bytes_per_unit": 229.0, "sha": "e17dae5e7f0f81be"},
-    "node": {"bytes_per_unit": 505.7, "sha": "e17dae5e7f0f81be"},
+    "sweep_x": {"bytes_per_unit": 235.3, "sha": "fc316f2231bbc83e"},
+    "sweep_y": {"bytes_per_unit": 227.5, "sha": "fc316f2231bbc83e"},
+    "node": {"bytes_per_unit": 503.4, "sha": "fc316f2231bbc83e"},
 }
 # FP64-pipe instructions per unit (ncu at 2048x1024: sm__inst_executed_pipe_fp64 of one launch times 32 over its
 # units, the node kernel's mean over the three stages; the count per unit does not depend on the grid size). The
 # reconstruction and the limiter run in fixed point on the integer pipes, so these are below the algorithmic "ops"
 # above; valid only for the kernel sources they were taken on (sources_sha).
 FP64_PIPE_OPS = {
-    "sweep_x": {"ops_per_unit": 68.7, "sha": "e17dae5e7f0f81be"},
-    "sweep_y": {"ops_per_unit": 70.5, "sha": "e17dae5e7f0f81be"},
-    "node": {"ops_per_unit": 100.0, "sha": "e17dae5e7f0f81be"},
+    "sweep_x": {"ops_per_unit": 68.7, "sha": "fc316f2231bbc83e"},
+    "sweep_y": {"ops_per_unit": 70.5, "sha": "fc316f2231bbc83e"},
+    "node": {"ops_per_unit": 100.0, "sha": "fc316f2231bbc83e"},
 }
 STATE_BYTES = 9 * NX * NY * 8
 

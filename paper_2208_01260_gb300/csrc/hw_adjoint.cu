@@ -990,6 +990,8 @@ int reverse_stage_body(const hw::SolverView& v, AdjBuffers* B, const hw::AdjDev&
 
 // The nine planes of a state copied: one launch up to 2^18 nodes, where nine copies cost more than what they move (about
 // 2.5 us each on the GPU, 30 sets of them in a checkpointed gradient of 8 steps); copies above, at the copy engine's rate.
+// A gradient of 6 steps with 2 snapshots, one launch / nine copies: 4.58 / 5.21 ms at 4096 nodes, 18.0 / 18.4 at 65,536,
+// 36.8 / 37.6 at 160,000, 55.8 / 55.6 at 2^18, 75.5 / 75.6 at 360,000.
 int copy_state(double* const* dst, double* const* src, size_t n, cudaStream_t st) {
   if (n > ((size_t)1 << 18)) {
     for (int q = 0; q < 9; ++q) ACUDA(cudaMemcpyAsync(dst[q], src[q], n * sizeof(double), cudaMemcpyDeviceToDevice, st));

@@ -132,7 +132,10 @@ struct AlphaOut {
   double t_end;
   float* fsc;
 };
-constexpr size_t kAlphaOneMax = (size_t)1 << 18;  // nodes up to which the double reduction is one launch
+// Nodes up to which the double reduction is one launch. The two forms are within 0.5% of a step of each other from 131,072
+// nodes on (10 steps, one launch / two: 3.41 / 3.43 ms at 131,044 nodes, 5.84 / 5.84 at 2^18, 6.08 / 6.06 at 266,240, 20.13 /
+// 20.10 at 2^20); two keep the FP64 pipe out of the tiles that cannot hold the maximum.
+constexpr size_t kAlphaOneMax = (size_t)1 << 18;
 void launch_alpha_finish2d(const Dev2D& d, unsigned long long* amax, int* status, const AlphaOut& out, cudaStream_t st);
 void launch_alpha_finish2d(const Dev2DT<float>& d, unsigned long long* amax, int* status, const AlphaOut& out,
                            cudaStream_t st);

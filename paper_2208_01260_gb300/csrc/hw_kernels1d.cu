@@ -38,9 +38,10 @@ __global__ void __launch_bounds__(X1_T) k_sweep1d(Dev1D d, const double* __restr
   for (int q = 0; q < 6; ++q) d.X[q][k] = out[q];
 }
 
-// The same interface with its four independent reconstructions (field k on side s, Sec. 2.1 Step 1) on four lanes of a warp: lanes 4j .. 4j + 3 compute interface j, lane r taking field r >> 1 on
-// side r & 1, and exchange their values by shuffles in the order interface_values1d adds them, so the
-// outputs are the same values. Lane r returns output components {0, 1}, {2, 3}, {4} or {5} for
+// The same interface with its four independent reconstructions (field k on side s, Sec. 2.1 Step 1) on four
+// lanes of a warp: lanes 4j .. 4j + 3 compute interface j, lane r taking field r >> 1 on side r & 1, and
+// exchange their values by shuffles in the order interface_values1d adds them, so the outputs are the same
+// values. Lane r returns output components {0, 1}, {2, 3}, {4} or {5} for
 // r = 0, 1, 2, 3 in o[0..1]. Every lane of the warp must call (the shuffles take the full warp).
 // For grids whose sweep has too few interfaces to occupy the GPU: one warp's chain of FP64 instructions,
 // not the GPU's FP64 throughput, then sets the kernel's duration, and this chain is about a third as long.
@@ -130,7 +131,7 @@ __device__ __forceinline__ void interface_values1d_lanes(const double* r0, const
 // The four-lane sweep: XL_I interfaces per block of 4 XL_I threads, used while the grid has at most
 // kLaneSweepMax interfaces (up to one such warp per SM partition: 152 SMs x 4 partitions x 8 interfaces). 20 steps at
 // N = 200 0.90 ms against 1.13 with a thread per interface, at 4863 0.98 against 1.19; without the projection 0.72 against
-// 0.94 and 0.80 against 1.01. At 20,000 a thread per interface, which fills the SMs with a quarter of the warps.
+// 0.94 and 0.80 against 1.01.
 constexpr int XL_I = 32;
 constexpr int XL_T = 4 * XL_I;
 constexpr int XL_N = XL_I + 3;

@@ -782,6 +782,8 @@ void launch_alpha2d(const Dev2D& d, unsigned long long* amax, int* status, cudaS
 void launch_alpha_finish2d(const Dev2D& d, unsigned long long* amax, int* status, const AlphaOut& out, cudaStream_t st) {
   unsigned long long* slots = amax + kAlpha2dSlots;
   const size_t n = (size_t)d.nx * d.ny;
+  // one node a thread while one block an SM takes the grid; beyond, four a thread, which is the slower form up to 2^18 nodes (10
+  // steps at 65,536 nodes 1.90 ms with one, 2.00 with four; at 131,044 3.35 and 3.39; at 2^18 5.74 and 5.80)
   if (n <= (size_t)152 * 256) {
     k_alpha2d_one<1><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(d, slots, status, out);
   } else if (n <= kAlphaOneMax) {
@@ -846,7 +848,9 @@ void launch_sweep_x2d(const Dev2D& d, const double* alpha, bool linear, bool chr
 void launch_sweep_y2d(const Dev2D& d, const double* alpha, bool linear, bool chr, cudaStream_t st) {
   sweep_y_impl(d, alpha, linear, chr, st);
 }
-// Tiles of both sweeps up to which they share a launch.
+// Tiles of both sweeps up to which they share a launch: one launch has one partly empty last wave instead of two. Four steps
+// in one / two launches: 1.39 / 1.49 ms at 131,044 nodes, 2.61 / 2.67 at 291,600, 2.81 / 2.87 at 313,600 (this line lies
+// between), 8.05 / 8.08 at 2^20, 30.7 / 30.6 at 2^22.
 constexpr unsigned long long kSweepsOneMax = 152 * 4 * 8;
 
 void launch_sweeps2d(const Dev2D& d, const double* alpha, bool linear, bool chr, cudaStream_t st) {

@@ -5,7 +5,7 @@
 // node, and each kernel lay between the memory and the issue limit. A tile of 16 x 16 nodes forms (16 + 4) x 16 records
 // along each direction (1.25 per node) and 17 x 16 interfaces (1.06 per node). What bounds it is instruction issue (59% of
 // the slots, 2290 instructions per node) with the latency of its loads, at 30 warps per SM. Measured at 2048^2: 0.411 ms a stage,
-// a job of four steps 6.14 -> 5.84 ms; with 4 blocks per SM (48 registers) 6.01 ms, with the tile's nodes held in shared
+// a job of four steps 6.14 -> 5.78 ms; with 4 blocks per SM (48 registers) 6.01 ms, with the tile's nodes held in shared
 // memory (68 KB a block) 6.13 ms.
 #include "hw_stencil2d.cuh"
 

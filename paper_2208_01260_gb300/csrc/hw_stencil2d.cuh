@@ -997,8 +997,9 @@ __device__ __forceinline__ void right_hand_side(const Dev2DT<R>& d, size_t o, co
   }
 }
 
-// RHS assembly, limiter and RK combination (or the bare RHS) at node (i, j) of one grid, read through faces. FIXED: the limiter in fixed point where the node's data fits it. on: offset of the grid in pooled
-// node planes (0 for one grid). COH: loads of the state and base planes as in ldp.
+// RHS assembly, limiter and RK combination (or the bare RHS) at node (i, j) of one grid, read through faces. FIXED: the
+// limiter in fixed point where the node's data fits it. on: offset of the grid in pooled node planes (0 for one grid). COH:
+// loads of the state and base planes as in ldp.
 template <int MODE, bool LINEAR, bool CHAR, bool FIXED, bool COH, class S, class R, class Faces>
 __device__ __forceinline__ void node_update_faces(const Dev2DT<R>& d, const S src, const StageArgsT<R>& sa, int i, int j, size_t on,
                                                   const Faces& faces) {

@@ -13,7 +13,7 @@
 //     one launch instead of three.
 // Blocks own N = 31 or 63 nodes and compute the two interfaces on their ends themselves. Grids of at most 504 nodes
 // run whole steps in one launch of one thread-block cluster (k_run1d), larger ones a launch per stage (k_stage1d).
-// Measured (a job of 20 steps at N = 200, of 10 at N = 12801): 1.09 -> 0.40 ms and 0.87 -> 0.50 ms against three
+// Measured (a job of 20 steps at N = 200, of 10 at N = 12801): 1.14 -> 0.41 ms and 0.90 -> 0.51 ms against three
 // launches per stage on the FP64 pipe; one launch per stage takes 0.66 ms at N = 200. k_stage1d at N = 12801 holds
 // three blocks per SM (96 registers), all 413 at once: 17 us per stage against 21 with two.
 #include "hw_fixed.h"
@@ -123,7 +123,8 @@ __device__ __noinline__ void interface_fp64(const Dev1D& d, double alpha, const 
 
 // Interface k by four lanes of a warp: lane r takes field r >> 1 (without projection: component r >> 1) on side
 // r & 1; the sides and fields meet by shuffles. r0: the first of its four records in shared memory; S: the first
-// of its four nodes (T: static planes); ist: its state; qb: its source candidates. Lane r writes X components {0, 1}, {2, 3}, {4}, {5} for r = 0 .. 3 unless live is false.
+// of its four nodes (T: static planes); ist: its state; qb: its source candidates. Lane r writes X components {0, 1},
+// {2, 3}, {4}, {5} for r = 0 .. 3 unless live is false.
 template <bool CHAR>
 __device__ __forceinline__ void interface_lanes(const Dev1D& d, double alpha, const double* r0, const double* S, const double* T,
                                                 int stride, const double* ist, const double* qb, int r, bool live,
